@@ -20,14 +20,15 @@
 // one level L = s + t stays an exact integer over a chunk of 256 K values
 // (at most (L-1) 2^22 <= 2^24 for L <= 5), so after every chunk the epilogue
 // warps move levels 2-5 into exact int64 accumulators (shifted into one common
-// scale, at most 2^54 in total) and levels 6-7, whose weights are at most
+// scale, at most 2^54 in total; levels 2 and 3, which have one and two pairs,
+// every fourth and second chunk) and levels 6-7, whose weights are at most
 // 2^-32 of the leading level, into an FP32 accumulator (its rounding is then
 // below 2^-56 of the leading level).
 // The result is W = 2^(e_i + f_j) (acc 2^-40 + acc67 2^-48), accurate to a few
 // units of 2^-48 relative to |A_i.| |Y_.j| per term: FP64-class.
-// Extended variant (LMAX = 8): the five pairs of level 8 are kept too (26 MMAs
-// per K step instead of 21, level 8 drained into the FP32 accumulator at weight
-// 2^-64). The dropped pairs then weigh at most 2^-58 instead of 2^-50 of
+// Extended variant (LMAX = 8): the five pairs of level 8 are kept too (26 pairs
+// per K step instead of 21, levels 6-8 drained into a second int64 accumulator
+// at weight 2^-64). The dropped pairs then weigh at most 2^-58 instead of 2^-50 of
 // 2^(e_i + f_j) per term, so a product over K terms whose result cancels
 // almost completely (a Gram of nearly orthonormal columns with entries near 1,
 // the residual X - T U of a triangular solve) keeps an error near the digit
@@ -36,10 +37,11 @@
 // Kernel structure (128 x 64 real output tile = 32 complex columns, 10 warps):
 //   warp 0    TMA producer: 6 A digit tiles (128 x 32) and 6 B digit tiles
 //             (64 x 32) per K block into a 3-stage ring (64B swizzle)
-//   warp 1    TMEM allocator and MMA issuer: 21 (26) tcgen05.mma (M=128,
-//             N=64, K=16) per 16-wide K step, one accumulator per level (6 (7)
-//             x 64 TMEM columns); after each 256-wide chunk it hands the
-//             accumulators to the epilogue and waits until they are drained
+//   warp 1    TMEM allocator and MMA issuer: the 21 (26) digit pairs of a
+//             16-wide K step as 13 (21) tcgen05.mma (M=128, N=64 or 128, K=16)
+//             on 8 accumulators of 64 TMEM columns; after each 256-wide chunk it
+//             hands the accumulators to the epilogue and waits until they are
+//             drained
 //   warps 2-9 epilogue: warp w owns TMEM lane quarter w % 4 and half of the
 //             complex columns; int64/FP32 accumulators in registers; at the
 //             end forms the FP64 result and applies the fused update.
@@ -61,6 +63,9 @@ constexpr int OS = 6;                    // digits per operand
 static_assert(OS == 6, "the epilogue keeps levels 2-5 exact and levels 6-7 in FP32");
 constexpr int TM = 128, TN = 64, TK = 32, STAGES = 3;
 constexpr int CHUNK_KB = 8;              // K blocks per exact chunk (256 values)
+// a chunk's sum of level L is an integer of at most (L - 1) 2^22, so level 2 may
+// run over four chunks and level 3 over two before it leaves 2^24
+constexpr int kDrain2 = 4, kDrain3 = 2;
 constexpr int A_TILE = TM * TK * 2;      // 8 KB per digit
 constexpr int B_TILE = TN * TK * 2;      // 4 KB per digit
 constexpr int STAGE_BYTES = OS * (A_TILE + B_TILE);  // 72 KB
@@ -132,15 +137,72 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
   d |= (uint64_t)4 << 61;
   return d;
 }
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                            ((uint32_t)(TM >> 4) << 24);
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
+// FP32 accumulate, BF16 A and B, both K-major, M = TM, N = n columns.
+constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) |
+         ((uint32_t)(TM >> 4) << 24);
+}
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
+                                          uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
+      "l"(a), "l"(b), "r"(id), "r"(acc)
       : "memory");
+}
+// TMEM accumulators (TN columns each). Levels that get a neighbour's product
+// in the same MMA lie side by side; a primed slot takes the one pair of its
+// level that has no neighbour (added in the epilogue). An accumulator is only
+// ever written by MMAs of one shape and one destination, which execute in issue
+// order.
+template <int LMAX> struct Slots;
+template <> struct Slots<7> {
+  static constexpr int L2 = 0, L3 = 1, L4 = 2, L5 = 3, L6 = 4, L7 = 5, L5b = 6, L7b = 7;
+};
+template <> struct Slots<8> {
+  static constexpr int L2 = 0, L3 = 1, L4 = 2, L5 = 3, L6 = 4, L7 = 5, L8 = 6, L7b = 7;
+};
+// The digit pairs of one 16-wide K step. An MMA of N = 64 moves 6 KB of
+// operands through shared memory in the 32 cycles its products take, more than
+// the 128 bytes a cycle it has; one of N = 128 moves 8 KB in 64. So A digit s
+// meets B digits t and t + 1 in one MMA wherever the two results are neighbours
+// (the B digit tiles lie one after the other, their 64 rows are whole swizzle
+// atoms). 36 filter steps with N = 9273 and up to 316 columns: 132 ms with 21
+// MMAs of N = 64 and every level drained per chunk, 99 ms so.
+// r2, r3, r: this step restarts levels 2, 3 and the others.
+template <int LMAX>
+__device__ __forceinline__ void digit_pairs(uint32_t tmem, uint32_t sa, uint32_t sb, bool r2,
+                                            bool r3, bool r) {
+  using S = Slots<LMAX>;
+  auto one = [&](int slot, int s, int t, bool restart) {
+    umma_bf16(tmem + (uint32_t)(slot * TN), sdesc_sw64(sa + (s - 1) * A_TILE),
+              sdesc_sw64(sb + (t - 1) * B_TILE), idesc(TN), restart ? 0u : 1u);
+  };
+  auto two = [&](int slot, int s, int t, bool restart) {  // digits t, t + 1
+    umma_bf16(tmem + (uint32_t)(slot * TN), sdesc_sw64(sa + (s - 1) * A_TILE),
+              sdesc_sw64(sb + (t - 1) * B_TILE), idesc(2 * TN), restart ? 0u : 1u);
+  };
+  one(S::L2, 1, 1, r2);
+  one(S::L3, 1, 2, r3);
+  one(S::L3, 2, 1, false);
+  if constexpr (LMAX == 7) {
+#pragma unroll
+    for (int s = 1; s <= 3; ++s) two(S::L4, s, 4 - s, r && s == 1);
+    one(S::L5b, 4, 1, r);
+  } else {
+#pragma unroll
+    for (int s = 1; s <= 3; ++s) one(S::L4, s, 4 - s, r && s == 1);
+#pragma unroll
+    for (int s = 1; s <= 4; ++s) one(S::L5, s, 5 - s, r && s == 1);
+  }
+#pragma unroll
+  for (int s = 1; s <= 5; ++s) two(S::L6, s, 6 - s, r && s == 1);
+  one(S::L7b, 6, 1, r);
+  if constexpr (LMAX == 8) {
+#pragma unroll
+    for (int s = 2; s <= 6; ++s) one(S::L8, s, 8 - s, r && s == 2);
+  }
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile(
@@ -159,6 +221,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
       : "r"(taddr));
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+// acc += v 2^SH for an integer-valued v of at most 2^24
+template <int SH>
+__device__ __forceinline__ void add_level(long long& acc, float v) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(__float2int_rn(v)), "r"(1 << SH));
 }
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -289,20 +356,10 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
 #pragma unroll
           for (int kk = 0; kk < TK / 16; ++kk) {
             const uint32_t off = kk * 32;
-#pragma unroll
-            for (int L = 2; L <= LMAX; ++L) {
-              const int sa0 = L - OS > 1 ? L - OS : 1;  // first pair of level L
-#pragma unroll
-              for (int sa = sa0; sa < L && sa <= OS; ++sa) {
-                const int tb = L - sa;
-                // every level restarts each 256-long chunk (levels 2-5 then stay
-                // exact integers below 2^24)
-                const uint32_t acc = (kc == 0 && kk == 0 && sa == sa0) ? 0u : 1u;
-                umma_bf16(tmem + (uint32_t)((L - 2) * TN),
-                          sdesc_sw64(st + (sa - 1) * A_TILE + off),
-                          sdesc_sw64(st + OS * A_TILE + (tb - 1) * B_TILE + off), acc);
-              }
-            }
+            // levels restart often enough to stay exact integers: see kDrain2, kDrain3
+            const bool r = kc == 0 && kk == 0;
+            digit_pairs<LMAX>(tmem, st + off, st + OS * A_TILE + off, r && c % kDrain2 == 0,
+                              r && c % kDrain3 == 0, r);
           }
           umma_commit(smem_u32(&bars[STAGES + s]));
         }
@@ -320,12 +377,13 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
     const int64_t row = m0 + q * 32 + lane;
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
     long long acc[2 * HC];                    // re[0..16), im[16..32): levels 2-5, weight 2^-40
-    // levels 6-LMAX, weight 2^-48. In the extended variant they are summed over
-    // the chunks in FP64: its products are Grams whose diagonal adds squared
-    // digits coherently (sum_k d_3(x_k)^2 grows like K), where FP32 sums over
+    // levels 6-LMAX. In FP32 at weight 2^-48; in the extended variant in int64 at
+    // weight 2^-64: its products are Grams whose diagonal adds squared digits
+    // coherently (sum_k d_3(x_k)^2 grows like K), where FP32 sums over
     // K = 80000 lost about 2^-44 of the scale (orthogonality 2e-11 at
     // N = 40000 after CholeskyQR2); per chunk the values stay below 2^25.
-    using Acc67 = typename std::conditional<LMAX == 8, double, float>::type;
+    using Acc67 = typename std::conditional<LMAX == 8, long long, float>::type;
+    constexpr double kW67 = LMAX == 8 ? 0x1p-64 : 0x1p-48;
     Acc67 acc67[2 * HC];
 #pragma unroll
     for (int j = 0; j < 2 * HC; ++j) {
@@ -338,38 +396,64 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
       go = __all_sync(0xffffffffu, ok && !*(volatile int*)&s_abort);
       if (!go) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // levels 2..5 are exact integers below 2^24 per chunk: int64 at weight
-      // 2^-40 (level L shifted by 8 (5 - L) bits). Levels 6 and 7 (weights
-      // 2^-48, 2^-56, at most 2^-24 of the leading level) go to FP32 registers
-      // per chunk. (Accumulating them in TMEM over the whole K range instead
-      // lost accuracy at K = 80000: a Ritz-value floor near 1e-10 ||A||.)
-      // loads issued two levels at a time, one wait per pair (the TMEM load
-      // latency is paid 6 times per chunk instead of 12)
+      // levels 2..5 are exact integers of at most 2^24: int64 at weight 2^-40
+      // (level L times 2^(8 (5 - L)), one wide multiply-add per value). Levels 6
+      // and 7 (weights 2^-48, 2^-56, at most 2^-24 of the leading level) go to
+      // FP32 registers per chunk. (Accumulating them in TMEM over the whole K
+      // range instead lost accuracy at K = 80000: a Ritz-value floor near 1e-10
+      // ||A||.) Loads are issued three slots at a time, one wait each.
+      using S = Slots<LMAX>;
+      const bool last = c == nchunks - 1;
+      const bool d2 = last || c % kDrain2 == kDrain2 - 1, d3 = last || c % kDrain3 == kDrain3 - 1;
 #pragma unroll
       for (int part = 0; part < 2; ++part) {  // real columns, then imaginary
+        const uint32_t tp = tl + (uint32_t)(part * CT + h * HC);
+        long long* ac = acc + part * HC;
+        Acc67* af = acc67 + part * HC;
+        float v[3][HC];
+        tmem_ld16(tp + S::L4 * TN, v[0]);
+        tmem_ld16(tp + S::L5 * TN, v[1]);
+        if constexpr (LMAX == 7) tmem_ld16(tp + Slots<7>::L5b * TN, v[2]);
+        tmem_wait_ld();
 #pragma unroll
-        for (int g = 0; g < LMAX / 2; ++g) {  // levels 2-3, 4-5, 6-7 (, 8)
-          float v[2][HC];
-#pragma unroll
-          for (int l = 0; l < 2; ++l)
-            if (2 + 2 * g + l <= LMAX)
-              tmem_ld16(tl + (uint32_t)((2 * g + l) * TN + part * CT + h * HC), v[l]);
+        for (int j = 0; j < HC; ++j) {
+          add_level<8>(ac[j], v[0][j]);
+          add_level<0>(ac[j], LMAX == 7 ? v[1][j] + v[2][j] : v[1][j]);
+        }
+        if constexpr (LMAX == 7) {
+          tmem_ld16(tp + S::L6 * TN, v[0]);
+          tmem_ld16(tp + S::L7 * TN, v[1]);
+          tmem_ld16(tp + S::L7b * TN, v[2]);
           tmem_wait_ld();
 #pragma unroll
-          for (int l = 0; l < 2; ++l) {
-            const int L = 2 + 2 * g + l;
-            if (L > LMAX) continue;
-            if (L <= 5) {
-              const int sh = 8 * (5 - L);
+          for (int j = 0; j < HC; ++j) {
+            af[j] += v[0][j];
+            af[j] = fmaf(0x1p-8f, v[1][j] + v[2][j], af[j]);
+          }
+        } else {
+          tmem_ld16(tp + S::L7 * TN, v[0]);
+          tmem_ld16(tp + S::L7b * TN, v[1]);
+          tmem_wait_ld();
 #pragma unroll
-              for (int j = 0; j < HC; ++j)
-                acc[part * HC + j] += (long long)__float2int_rn(v[l][j]) << sh;
-            } else {
-              const Acc67 w = L == 6 ? Acc67(1) : (L == 7 ? Acc67(0x1p-8) : Acc67(0x1p-16));
+          for (int j = 0; j < HC; ++j) add_level<8>(af[j], v[0][j] + v[1][j]);
+          tmem_ld16(tp + S::L6 * TN, v[0]);
+          tmem_ld16(tp + Slots<8>::L8 * TN, v[1]);
+          tmem_wait_ld();
 #pragma unroll
-              for (int j = 0; j < HC; ++j)
-                acc67[part * HC + j] = fma(w, (Acc67)v[l][j], acc67[part * HC + j]);
-            }
+          for (int j = 0; j < HC; ++j) {
+            add_level<16>(af[j], v[0][j]);
+            add_level<0>(af[j], v[1][j]);
+          }
+        }
+        if (d3) {
+          tmem_ld16(tp + S::L3 * TN, v[0]);
+          if (d2) tmem_ld16(tp + S::L2 * TN, v[1]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < HC; ++j) add_level<16>(ac[j], v[0][j]);
+          if (d2) {
+#pragma unroll
+            for (int j = 0; j < HC; ++j) add_level<24>(ac[j], v[1][j]);
           }
         }
       }
@@ -389,8 +473,8 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
         if (col < P.j0 || col >= P.ncols) continue;
         const double sc = sa * ldexp(1.0, P.escale_b[col]);
         const double2 b = P.diag ? P.Bsrc[row + col * P.ldbs] : make_double2(0.0, 0.0);
-        const double lr = fma((double)acc[jj], 0x1p-40, (double)acc67[jj] * 0x1p-48);
-        const double li = fma((double)acc[HC + jj], 0x1p-40, (double)acc67[HC + jj] * 0x1p-48);
+        const double lr = fma((double)acc[jj], 0x1p-40, (double)acc67[jj] * kW67);
+        const double li = fma((double)acc[HC + jj], 0x1p-40, (double)acc67[HC + jj] * kW67);
         const double wr = fma(dg.x, b.x, fma(-dg.y, b.y, sc * lr));
         const double wi = fma(dg.x, b.y, fma(dg.y, b.x, sc * li));
         if (P.mode == EPI_STORE) {
