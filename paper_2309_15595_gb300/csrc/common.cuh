@@ -78,9 +78,12 @@ struct Epilogue {
   double* partial;            // resid: [row_tile + col * n_row_tiles] sums of |.|^2
 };
 
-// P = A (M x K) * B (K x n); A column-major (lda), B column-major (ldb).
+// P = A (M x K) * B (K x n); A column-major (lda), B column-major (ldb). tri: an
+// operand that is square and upper triangular (its zeros are not multiplied).
+enum Triangular { TRI_NONE = 0, TRI_A = 1, TRI_B = 2 };
 cudaError_t zgemm_nn(cudaStream_t s, int64_t M, int64_t n, int64_t K, const double2* A,
-                     int64_t lda, const double2* B, int64_t ldb, const Epilogue& ep);
+                     int64_t lda, const double2* B, int64_t ldb, const Epilogue& ep,
+                     int tri = TRI_NONE);
 // Number of 64-row tiles the residual epilogue writes partials for.
 int64_t zgemm_row_tiles(int64_t M);
 // Fixed-order reduction of the residual partials: out[j] = sqrt(sum_t partial).

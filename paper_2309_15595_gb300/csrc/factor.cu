@@ -359,7 +359,7 @@ cudaError_t trinv_rec(cudaStream_t s, int64_t n, const double2* U, int64_t ldu,
   ep.mode = EPI_STORE;  // T = U12 Y22 (n1 x n2, ld n1)
   ep.Y = T;
   ep.ldy = n1;
-  e = zgemm_nn(s, n1, n2, n2, U + n1 * ldu, ldu, Y + n1 + n1 * ldy, ldy, ep);
+  e = zgemm_nn(s, n1, n2, n2, U + n1 * ldu, ldu, Y + n1 + n1 * ldy, ldy, ep, TRI_B);
   if (e != cudaSuccess) return e;
   Epilogue e2{};
   e2.mode = EPI_FILTER;  // Y12 = -(Y11 T) (beta = 0: the old Y12 is not read)
@@ -370,7 +370,7 @@ cudaError_t trinv_rec(cudaStream_t s, int64_t n, const double2* U, int64_t ldu,
   e2.ldx = ldy;
   e2.Y = Y + n1 * ldy;
   e2.ldy = ldy;
-  return zgemm_nn(s, n1, n2, n1, Y, ldy, T, n1, e2);
+  return zgemm_nn(s, n1, n2, n1, Y, ldy, T, n1, e2, TRI_A);
 }
 
 std::once_flag g_attr_once[kMaxDevices];

@@ -1,11 +1,16 @@
 // Complex FP64 GEMM kernels on the DFMA pipe.
 //
 // On sm_103 the FP64 rate is two DFMA per clock per SM (about 1.2 TFLOP/s for
-// the GPU), so every product here is bound by the FP64 pipe as soon as a tile
-// reuses each loaded element a few times. The kernels use 64 x 64 output tiles,
-// 256 threads with 4 x 4 complex accumulators each, and double-buffered shared
-// memory; the epilogues fuse the Chebyshev three-term update (Eq. 1), plain
-// stores, and the per-column residual sums of squares (Alg. 2 residual lines).
+// the GPU), so every product here is bound by the FP64 pipe: a warp's DFMA
+// holds the pipe for 64 clocks, and a complex multiply-add per element loaded
+// from L2 would still be enough. What decides the time is how evenly the tiles
+// fall on the 152 SMs. The tiles are therefore small, 16 x 16 with two warps of
+// 2 x 2 accumulators, up to a dozen CTAs on an SM: a 2600 x 195 x 2600 product
+// is 2119 tiles, 13.9 per SM, where 64 x 64 tiles were 164 CTAs, two on some SMs
+// and one on the others, with a quarter of the columns padding.
+// Double-buffered shared memory; the epilogues fuse the Chebyshev three-term
+// update (Eq. 1), plain stores, and the per-column residual sums of squares
+// (Alg. 2 residual lines).
 #include <algorithm>
 
 #include "common.cuh"
@@ -13,90 +18,98 @@
 namespace chase {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 8, NT = 256;
+constexpr int BN = 16, BK = 8;
+constexpr int MT = 2;        // accumulators per thread and direction
+constexpr int BM = 16;       // rows of a tile
+constexpr int RESID_BM = 64;  // rows of a tile of the residual epilogue: one partial each
+constexpr int threads_of(int bm) { return bm / MT * (BN / MT); }
 constexpr int kMaxSplits = 8;
+constexpr size_t kMinGramWs = (size_t)1 << 19;  // room for many splits of a small product
 
 // A operand: normal (M x K column-major) or conjugate-transpose of a K x M
 // column-major X (Gram products X^H Y).
-template <bool ACONJT>
+// Every thread moves two elements of the TM x BK slab.
+template <bool ACONJT, int TM>
 __device__ __forceinline__ void load_a(const double2* __restrict__ A, int64_t lda, int64_t M,
                                        int64_t m0, int64_t k0, int64_t kend, int t,
                                        double2 (&ra)[2]) {
-  if (!ACONJT) {
-    const int r = t & 63, kk = t >> 6;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int64_t row = m0 + r, k = k0 + kk + 4 * h;
+  for (int h = 0; h < 2; ++h) {
+    const int e = t + h * threads_of(TM);
+    if (!ACONJT) {
+      const int64_t row = m0 + e % TM, k = k0 + e / TM;
       ra[h] = (row < M && k < kend) ? A[row + k * lda] : make_double2(0.0, 0.0);
-    }
-  } else {
-    const int kk = t & 7, r = t >> 3;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int64_t row = m0 + r + 32 * h, k = k0 + kk;
+    } else {
+      const int64_t row = m0 + e / BK, k = k0 + e % BK;
       ra[h] = (row < M && k < kend) ? conjz(A[k + row * lda]) : make_double2(0.0, 0.0);
     }
   }
 }
 
-template <bool ACONJT>
-__device__ __forceinline__ void store_a(double2 (*As)[BM], int t, const double2 (&ra)[2]) {
-  if (!ACONJT) {
-    const int r = t & 63, kk = t >> 6;
-    As[kk][r] = ra[0];
-    As[kk + 4][r] = ra[1];
-  } else {
-    const int kk = t & 7, r = t >> 3;
-    As[kk][r] = ra[0];
-    As[kk][r + 32] = ra[1];
+template <bool ACONJT, int TM>
+__device__ __forceinline__ void store_a(double2 (*As)[TM], int t, const double2 (&ra)[2]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int e = t + h * threads_of(TM);
+    if (!ACONJT) As[e / TM][e % TM] = ra[h];
+    else As[e % BK][e / BK] = ra[h];
   }
 }
 
+constexpr int kBElems = BN * BK;
+template <int TM>
 __device__ __forceinline__ void load_b(const double2* __restrict__ B, int64_t ldb, int64_t n,
                                        int64_t n0, int64_t k0, int64_t kend, int t,
                                        double2 (&rb)[2]) {
-  const int kk = t & 7, c = t >> 3;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int64_t col = n0 + c + 32 * h, k = k0 + kk;
+    const int e = t + h * threads_of(TM);
+    if (e >= kBElems) continue;
+    const int64_t col = n0 + e / BK, k = k0 + e % BK;
     rb[h] = (col < n && k < kend) ? B[k + col * ldb] : make_double2(0.0, 0.0);
   }
 }
 
+template <int TM>
 __device__ __forceinline__ void store_b(double2 (*Bs)[BN], int t, const double2 (&rb)[2]) {
-  const int kk = t & 7, c = t >> 3;
-  Bs[kk][c] = rb[0];
-  Bs[kk][c + 32] = rb[1];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int e = t + h * threads_of(TM);
+    if (e < kBElems) Bs[e % BK][e / BK] = rb[h];
+  }
 }
 
-// One 64 x 64 tile of P = op(A) * B over k in [kbeg, kend).
-template <bool ACONJT, int EPI>
-__global__ void __launch_bounds__(NT)
+// One TM x BN tile of P = op(A) * B over k in [kbeg, kend). tri: B (TRI_B) or A
+// (TRI_A) is upper triangular, so the tile's k range ends at its last column or
+// starts at its first row.
+template <bool ACONJT, int EPI, int TM = BM>
+__global__ void __launch_bounds__(threads_of(TM))
     zgemm_kernel(int64_t M, int64_t n, int64_t K, const double2* __restrict__ A, int64_t lda,
                  const double2* __restrict__ B, int64_t ldb, Epilogue ep, int64_t kchunk,
-                 int64_t split_stride, bool upper_only) {
+                 int64_t split_stride, bool upper_only, int tri) {
   if (upper_only && blockIdx.x > blockIdx.y) return;
-  __shared__ double2 As[2][BK][BM];
+  __shared__ double2 As[2][BK][TM];
   __shared__ double2 Bs[2][BK][BN];
   const int t = threadIdx.x;
-  const int tx = t & 15, ty = t >> 4;
-  const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
-  const int64_t kbeg = (int64_t)blockIdx.z * kchunk;
-  const int64_t kend = min(K, kbeg + kchunk);
+  constexpr int TX = TM / MT, TY = BN / MT;  // threads across rows and columns
+  const int tx = t % TX, ty = t / TX;
+  const int64_t m0 = (int64_t)blockIdx.x * TM, n0 = (int64_t)blockIdx.y * BN;
+  const int64_t kbeg = tri == TRI_A ? m0 : (int64_t)blockIdx.z * kchunk;
+  const int64_t kend = min(K, tri == TRI_B ? n0 + BN : kbeg + kchunk);
 
-  double2 acc[4][4];
+  double2 acc[MT][MT];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
+    for (int j = 0; j < MT; ++j) acc[i][j] = make_double2(0.0, 0.0);
 
   const int64_t nkt = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
   double2 ra[2], rb[2];
   if (nkt > 0) {
-    load_a<ACONJT>(A, lda, M, m0, kbeg, kend, t, ra);
-    load_b(B, ldb, n, n0, kbeg, kend, t, rb);
-    store_a<ACONJT>(As[0], t, ra);
-    store_b(Bs[0], t, rb);
+    load_a<ACONJT, TM>(A, lda, M, m0, kbeg, kend, t, ra);
+    load_b<TM>(B, ldb, n, n0, kbeg, kend, t, rb);
+    store_a<ACONJT, TM>(As[0], t, ra);
+    store_b<TM>(Bs[0], t, rb);
   }
   __syncthreads();
   for (int64_t kt = 0; kt < nkt; ++kt) {
@@ -104,24 +117,24 @@ __global__ void __launch_bounds__(NT)
     const bool more = kt + 1 < nkt;
     if (more) {
       const int64_t k0 = kbeg + (kt + 1) * BK;
-      load_a<ACONJT>(A, lda, M, m0, k0, kend, t, ra);
-      load_b(B, ldb, n, n0, k0, kend, t, rb);
+      load_a<ACONJT, TM>(A, lda, M, m0, k0, kend, t, ra);
+      load_b<TM>(B, ldb, n, n0, k0, kend, t, rb);
     }
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      double2 a[4], b[4];
+      double2 a[MT], b[MT];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[cur][kk][tx + 16 * i];
+      for (int i = 0; i < MT; ++i) a[i] = As[cur][kk][tx + TX * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[cur][kk][ty + 16 * j];
+      for (int j = 0; j < MT; ++j) b[j] = Bs[cur][kk][ty + TY * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < MT; ++j) cfma(acc[i][j], a[i], b[j]);
     }
     if (more) {
-      store_a<ACONJT>(As[cur ^ 1], t, ra);
-      store_b(Bs[cur ^ 1], t, rb);
+      store_a<ACONJT, TM>(As[cur ^ 1], t, ra);
+      store_b<TM>(Bs[cur ^ 1], t, rb);
     }
     __syncthreads();
   }
@@ -130,24 +143,24 @@ __global__ void __launch_bounds__(NT)
   if (EPI == EPI_STORE) {
     double2* Y = ep.Y + (int64_t)blockIdx.z * split_stride;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t col = n0 + ty + 16 * j;
+    for (int j = 0; j < MT; ++j) {
+      const int64_t col = n0 + ty + TY * j;
       if (col >= n) continue;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int64_t row = m0 + tx + 16 * i;
+      for (int i = 0; i < MT; ++i) {
+        const int64_t row = m0 + tx + TX * i;
         if (row < M) Y[row + col * ep.ldy] = acc[i][j];
       }
     }
   } else if (EPI == EPI_FILTER) {
     // Eq. 1: Y_new = alpha (A Y_cur - gamma Y_cur) + beta Y_prev, in place over Y_prev.
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t col = n0 + ty + 16 * j;
+    for (int j = 0; j < MT; ++j) {
+      const int64_t col = n0 + ty + TY * j;
       if (col >= n) continue;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int64_t row = m0 + tx + 16 * i;
+      for (int i = 0; i < MT; ++i) {
+        const int64_t row = m0 + tx + TX * i;
         if (row >= M) continue;
         const double2 x = ep.X[row + col * ep.ldx];
         double2 v = make_double2(ep.alpha * fma(-ep.gamma, x.x, acc[i][j].x),
@@ -163,14 +176,14 @@ __global__ void __launch_bounds__(NT)
     }
   } else {  // EPI_RESID: sum_rows |P - theta_col X|^2 for this row tile
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t col = n0 + ty + 16 * j;
+    for (int j = 0; j < MT; ++j) {
+      const int64_t col = n0 + ty + TY * j;
       double s = 0.0;
       if (col < n) {
         const double th = ep.theta[col];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int64_t row = m0 + tx + 16 * i;
+        for (int i = 0; i < MT; ++i) {
+          const int64_t row = m0 + tx + TX * i;
           if (row < M) {
             const double2 x = ep.X[row + col * ep.ldx];
             const double dx = fma(-th, x.x, acc[i][j].x), dy = fma(-th, x.y, acc[i][j].y);
@@ -179,7 +192,7 @@ __global__ void __launch_bounds__(NT)
         }
       }
 #pragma unroll
-      for (int off = 8; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      for (int off = TX / 2; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
       if (tx == 0 && col < n) ep.partial[blockIdx.x + col * gridDim.x] = s;
     }
   }
@@ -295,21 +308,23 @@ int num_sms() {
   return g_num_sms[dev];
 }
 
-int64_t zgemm_row_tiles(int64_t M) { return cdiv(M, BM); }
+int64_t zgemm_row_tiles(int64_t M) { return cdiv(M, RESID_BM); }
 
 cudaError_t zgemm_nn(cudaStream_t s, int64_t M, int64_t n, int64_t K, const double2* A,
-                     int64_t lda, const double2* B, int64_t ldb, const Epilogue& ep) {
+                     int64_t lda, const double2* B, int64_t ldb, const Epilogue& ep, int tri) {
   if (M <= 0 || n <= 0) return cudaSuccess;
-  dim3 grid((unsigned)cdiv(M, BM), (unsigned)cdiv(n, BN), 1);
+  const int bm = ep.mode == EPI_RESID ? RESID_BM : BM;
+  const dim3 grid((unsigned)cdiv(M, bm), (unsigned)cdiv(n, BN), 1);
+  const int NT = threads_of(bm);
   switch (ep.mode) {
     case EPI_STORE:
-      zgemm_kernel<false, EPI_STORE><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false); count_launch();
+      zgemm_kernel<false, EPI_STORE><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false, tri); count_launch();
       break;
     case EPI_FILTER:
-      zgemm_kernel<false, EPI_FILTER><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false); count_launch();
+      zgemm_kernel<false, EPI_FILTER><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false, tri); count_launch();
       break;
     default:
-      zgemm_kernel<false, EPI_RESID><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false); count_launch();
+      zgemm_kernel<false, EPI_RESID, RESID_BM><<<grid, NT, 0, s>>>(M, n, K, A, lda, B, ldb, ep, K, 0, false, tri); count_launch();
       break;
   }
   return cudaGetLastError();
@@ -322,7 +337,9 @@ cudaError_t resid_reduce(cudaStream_t s, const double* partial, int64_t ntiles, 
   return cudaGetLastError();
 }
 
-size_t gram_workspace_elems(int64_t m, int64_t n) { return (size_t)kMaxSplits * m * n; }
+size_t gram_workspace_elems(int64_t m, int64_t n) {
+  return std::max((size_t)kMaxSplits * m * n, kMinGramWs);
+}
 
 cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2* X, int64_t ldx,
                   const double2* Y, int64_t ldy, double2* G, int64_t ldg, bool hermitian,
@@ -331,19 +348,19 @@ cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2
   if (ws_elems < (size_t)m * n) return cudaErrorInvalidValue;  // no room for one partial
   const int64_t tm = cdiv(m, BM), tn = cdiv(n, BN);
   const int64_t tiles = hermitian ? tm * (tm + 1) / 2 : tm * tn;
-  // split-K factor: the one (up to the workspace, 8, and K / 512) whose CTA
-  // count fills the last wave best (3 resident CTAs per SM); ties to fewer splits
-  const int64_t slots = 3 * (int64_t)num_sms();
+  // split-K factor: the one (up to the workspace and K / 64) for which the most
+  // loaded SM has the fewest k steps, a tile counting 16 more for its start and
+  // its partial (a 96 x 64 Gram over 2048 rows is 24 tiles: split 25 ways it
+  // takes 0.1 ms, in 4 pieces 0.9 ms); ties to fewer splits
+  const int64_t sms = num_sms();
   const int64_t smax = std::max<int64_t>(
-      1, std::min<int64_t>({(int64_t)kMaxSplits, std::max<int64_t>(1, K / 512),
-                            (int64_t)(ws_elems / ((size_t)m * n))}));
+      1, std::min<int64_t>(K / 64, (int64_t)(ws_elems / ((size_t)m * n))));
   int64_t splits = 1;
-  double best = -1.0;
-  for (int64_t sp = 1; sp <= smax; ++sp) {
-    const int64_t ctas = tiles * sp;
-    const double eff = (double)ctas / (double)(cdiv(ctas, slots) * slots);
-    if (eff > best + 1e-9) {
-      best = eff;
+  int64_t best = -1;
+  for (int64_t sp = 1; sp <= smax && tiles * (sp - 1) < 8 * sms; ++sp) {
+    const int64_t load = cdiv(tiles * sp, sms) * (cdiv(K, sp) + 16);
+    if (best < 0 || load < best) {
+      best = load;
       splits = sp;
     }
   }
@@ -353,8 +370,8 @@ cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2
   ep.Y = ws;
   ep.ldy = m;
   dim3 grid((unsigned)tm, (unsigned)tn, (unsigned)splits);
-  zgemm_kernel<true, EPI_STORE><<<grid, NT, 0, s>>>(m, n, K, X, ldx, Y, ldy, ep, kchunk,
-                                                    m * n, hermitian); count_launch();
+  zgemm_kernel<true, EPI_STORE><<<grid, threads_of(BM), 0, s>>>(m, n, K, X, ldx, Y, ldy, ep, kchunk,
+                                                    m * n, hermitian, TRI_NONE); count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   dim3 g2((unsigned)cdiv(m, 128), (unsigned)n, 1);
