@@ -13,135 +13,167 @@ namespace {
 constexpr int NB = kNB;  // 64
 constexpr int FT = 256;  // threads
 
-// Unblocked Cholesky of the kb x kb diagonal block at (k0, k0), in shared
-// memory, plus the inverse of the resulting upper-triangular block.
-__global__ void __launch_bounds__(FT)
-    potf2_kernel(double2* G, int64_t ldg, int64_t k0, int kb, double2* dinv_blk, int* info) {
-  extern __shared__ double2 sm[];
-  double2* S = sm;             // kb x kb, column-major, ld NB
-  double2* W = sm + NB * NB;   // inverse
-  __shared__ int failed;
-  const int t = threadIdx.x;
-  if (*info != 0) return;
-  if (t == 0) failed = 0;
-  for (int e = t; e < NB * NB; e += FT) {
-    const int r = e % NB, c = e / NB;
-    S[e] = (r < kb && c < kb && r <= c) ? G[(k0 + r) + (k0 + c) * ldg] : make_double2(0.0, 0.0);
-    W[e] = make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (t == 0) {
-      const double p = S[j + j * NB].x;
-      if (!(p > 0.0)) {  // also catches NaN
-        failed = 1;
-        *info = (int)(k0 + j + 1);
-      } else {
-        S[j + j * NB] = make_double2(sqrt(p), 0.0);
-      }
-    }
-    __syncthreads();
-    if (failed) return;
-    const double rd = 1.0 / S[j + j * NB].x;
-    for (int c = j + 1 + t; c < kb; c += FT) S[j + c * NB] = cscale(rd, S[j + c * NB]);
-    __syncthreads();
-    // G(r, c) -= conj(U(j, r)) U(j, c) for j < r <= c
-    const int rem = kb - j - 1;
-    for (int e = t; e < rem * rem; e += FT) {
-      const int r = j + 1 + e % rem, c = j + 1 + e / rem;
-      if (r <= c) S[r + c * NB] = csub(S[r + c * NB], cmulc(S[j + r * NB], S[j + c * NB]));
-    }
-    __syncthreads();
-  }
-  // inverse of the upper-triangular block, one column per thread
-  if (t < kb) {
-    const int c = t;
-    W[c + c * NB] = make_double2(1.0 / S[c + c * NB].x, 0.0);
-    for (int r = c - 1; r >= 0; --r) {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int l = r + 1; l <= c; ++l) acc = cadd(acc, cmul(S[r + l * NB], W[l + c * NB]));
-      W[r + c * NB] = cscale(-1.0 / S[r + r * NB].x, acc);
-    }
-  }
-  __syncthreads();
-  for (int e = t; e < NB * NB; e += FT) {
-    const int r = e % NB, c = e / NB;
-    if (r < kb && c < kb) G[(k0 + r) + (k0 + c) * ldg] = (r <= c) ? S[e] : make_double2(0.0, 0.0);
-    dinv_blk[e] = W[e];
-  }
+// Unblocked Cholesky of the kb x kb diagonal block at (k0, k0) and the inverse
+// of the resulting upper-triangular block, in registers.
+//
+// The elimination that turns G into U turns an identity beside it into
+// V = U^-H, and the two fit one 64 x 64 array: U on and above the diagonal, V
+// below it. Step j subtracts conj(M(j, r)) M(j, c) / p_j from M(r, c) for all
+// r > j and c >= r (U) or c <= j (V); rows are divided by their sqrt(p) at the
+// end. Each of the 256 threads owns 16 entries, a warp an 8 x 4 patch of every
+// 16 x 16 block, so patches that a step does not touch cost nothing on the
+// FP64 pipe (2 DFMA a clock on this one SM: 85 us for the 87 thousand complex
+// multiply-adds, which is what bounds the kernel). The owner of the next pivot
+// takes its reciprocal square root while the others still update, and the row
+// buffer alternates, so a step has one barrier.
+__device__ __forceinline__ bool pivot_rsqrt(double p, double* rd) {
+  const bool ok = p > 0.0;  // false for NaN too
+  *rd = ok ? rsqrt(p) : 0.0;
+  return ok;
 }
 
-// Panel: U(k-block, j) = W^H G(k-block, j) for one 64-column block j.
+__global__ void __launch_bounds__(FT)
+    potf2_kernel(double2* G, int64_t ldg, int64_t k0, int kb, double2* dinv_blk, int* info) {
+  __shared__ double2 row_s[2][NB];  // raw row j of M, 1 at column j
+  __shared__ double rd_s[NB];       // 1 / sqrt(p_j)
+  __shared__ int ok_s[NB];
+  if (*info != 0) return;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int rl = (warp & 1) * 8 + (lane & 7), cl = (warp >> 1) * 4 + (lane >> 3);
+  double2 m[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = 16 * a + rl, c = 16 * b + cl;
+      m[a][b] = (r <= c && c < kb) ? G[(k0 + r) + (k0 + c) * ldg] : make_double2(0.0, 0.0);
+    }
+  // raw row j from its owners; the pivot's owner also takes its root
+  auto publish = [&](int j) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      if (16 * a + rl != j) continue;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int c = 16 * b + cl;
+        row_s[j & 1][c] = c == j ? make_double2(1.0, 0.0) : m[a][b];
+        if (c == j) ok_s[j] = pivot_rsqrt(m[a][b].x, &rd_s[j]);
+      }
+    }
+  };
+  publish(0);
+  __syncthreads();
+  for (int j = 0; j < kb; ++j) {
+    if (!ok_s[j]) {
+      if (t == 0) *info = (int)(k0 + j + 1);
+      return;
+    }
+    const double ip = rd_s[j] * rd_s[j];
+    const double2* w = row_s[j & 1];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int r = 16 * a + rl;
+      if (r <= j) continue;
+      const double2 f = cscale(-ip, conjz(w[r]));
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int c = 16 * b + cl;
+        if (c >= r || c <= j) cfma(m[a][b], f, w[c]);
+      }
+    }
+    if (j + 1 < kb) publish(j + 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = 16 * a + rl, c = 16 * b + cl;
+      const bool in = r < kb && c < kb;
+      const double rd = r < kb ? rd_s[r] : 0.0;
+      double2 u = make_double2(0.0, 0.0);  // U(r, c)
+      double2 v = make_double2(0.0, 0.0);  // V(r, c) = conj(U^-1(c, r))
+      if (in && r == c) {
+        u.x = sqrt(m[a][b].x);
+        v.x = rd;
+      } else if (in && r < c) {
+        u = cscale(rd, m[a][b]);
+      } else if (in) {
+        v = cscale(rd, m[a][b]);
+      }
+      if (in) G[(k0 + r) + (k0 + c) * ldg] = u;
+      dinv_blk[c + r * NB] = conjz(v);
+    }
+}
+
+// Panel: U(k-block, j) = W^H G(k-block, j), PC columns per CTA (a 64 x 64 block
+// per CTA kept at most n / 64 SMs busy), one row and column per thread.
+constexpr int PC = FT / NB;  // 4
+constexpr int PANEL_SMEM = (NB * (NB + 1) + PC * NB) * (int)sizeof(double2);
 __global__ void __launch_bounds__(FT)
     panel_kernel(int64_t n, double2* G, int64_t ldg, int64_t k0, int kb, const double2* dinv_blk,
                  const int* info) {
   extern __shared__ double2 sm[];
-  double2* Wt = sm;            // W, ld NB
-  double2* P = sm + NB * NB;   // G block, ld NB
+  double2* Wt = sm;                    // W(l, r) at l (NB + 1) + r
+  double2* P = sm + NB * (NB + 1);     // G block, ld NB
   if (*info != 0) return;
-  const int t = threadIdx.x;
-  const int64_t c0 = k0 + kb + (int64_t)blockIdx.x * NB;
-  const int cb = (int)min((int64_t)NB, n - c0);
-  for (int e = t; e < NB * NB; e += FT) {
-    const int r = e % NB, c = e / NB;
-    Wt[e] = dinv_blk[e];
-    P[e] = (r < kb && c < cb) ? G[(k0 + r) + (c0 + c) * ldg] : make_double2(0.0, 0.0);
-  }
+  const int t = threadIdx.x, r = t % NB;
+  const int64_t c = k0 + kb + (int64_t)blockIdx.x * PC + t / NB;
+  const bool in = r < kb && c < n;
+  for (int e = t; e < NB * NB; e += FT) Wt[(e % NB) * (NB + 1) + e / NB] = dinv_blk[e];
+  P[t] = in ? G[(k0 + r) + c * ldg] : make_double2(0.0, 0.0);
   __syncthreads();
-  for (int e = t; e < kb * cb; e += FT) {
-    const int r = e % kb, c = e / kb;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l <= r; ++l) acc = cadd(acc, cmulc(Wt[l + r * NB], P[l + c * NB]));
-    G[(k0 + r) + (c0 + c) * ldg] = acc;
-  }
+  if (!in) return;
+  double2 acc = make_double2(0.0, 0.0);
+  const double2* p = P + (t / NB) * NB;
+  for (int l = 0; l <= r; ++l) cfma(acc, conjz(Wt[l * (NB + 1) + r]), p[l]);
+  G[(k0 + r) + c * ldg] = acc;
 }
 
 // Trailing update of upper tiles: G(i, j) -= sum_l conj(U(l, i)) U(l, j),
-// l over the k-block rows, k0 + kb <= i <= j (tile-wise upper).
-__global__ void __launch_bounds__(FT)
+// l over the k-block rows, k0 + kb <= i <= j (tile-wise upper). 16 x 16 tiles of
+// two warps: FP64-bound like the GEMM, and even at n = 128 on many SMs.
+constexpr int TB = 16, TT = 64;
+__global__ void __launch_bounds__(TT)
     trailing_kernel(int64_t n, double2* G, int64_t ldg, int64_t k0, int kb, const int* info) {
   if (*info != 0) return;
   if (blockIdx.x > blockIdx.y) return;
-  __shared__ double2 Ui[NB][NB / 4 + 1];  // staged in 4 chunks of 16 rows
-  __shared__ double2 Uj[NB][NB / 4 + 1];
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  __shared__ double2 Ui[TB][NB + 1];
+  __shared__ double2 Uj[TB][NB + 1];
+  const int t = threadIdx.x, tx = t & 7, ty = t >> 3;
   const int64_t s0 = k0 + kb;
-  const int64_t i0 = s0 + (int64_t)blockIdx.x * NB, j0 = s0 + (int64_t)blockIdx.y * NB;
-  double2 acc[4][4];
+  const int64_t i0 = s0 + (int64_t)blockIdx.x * TB, j0 = s0 + (int64_t)blockIdx.y * TB;
+  for (int c = 0; c < TB; ++c) {  // thread t: row t of the k-block
+    const bool okl = t < kb;
+    Ui[c][t] = (okl && i0 + c < n) ? G[(k0 + t) + (i0 + c) * ldg] : make_double2(0.0, 0.0);
+    Uj[c][t] = (okl && j0 + c < n) ? G[(k0 + t) + (j0 + c) * ldg] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  double2 acc[2][2];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = make_double2(0.0, 0.0);
-  for (int l0 = 0; l0 < kb; l0 += NB / 4) {
-    for (int e = t; e < NB * (NB / 4); e += FT) {
-      const int ll = e % (NB / 4), c = e / (NB / 4);
-      const int64_t l = k0 + l0 + ll;
-      const bool okl = (l0 + ll) < kb;
-      Ui[c][ll] = (okl && i0 + c < n) ? G[l + (i0 + c) * ldg] : make_double2(0.0, 0.0);
-      Uj[c][ll] = (okl && j0 + c < n) ? G[l + (j0 + c) * ldg] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
+    for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
 #pragma unroll 4
-    for (int ll = 0; ll < NB / 4; ++ll) {
-      double2 a[4], b[4];
+  for (int l = 0; l < kb; ++l) {
+    double2 a[2], b[2];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a[q] = conjz(Ui[tx + 16 * q][ll]);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) b[q] = Uj[ty + 16 * q][ll];
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) cfma(acc[p][q], a[p], b[q]);
+    for (int q = 0; q < 2; ++q) {
+      a[q] = conjz(Ui[tx + 8 * q][l]);
+      b[q] = Uj[ty + 8 * q][l];
     }
-    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) cfma(acc[p][q], a[p], b[q]);
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int64_t j = j0 + ty + 16 * q;
+  for (int q = 0; q < 2; ++q) {
+    const int64_t j = j0 + ty + 8 * q;
     if (j >= n) continue;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int64_t i = i0 + tx + 16 * p;
+    for (int p = 0; p < 2; ++p) {
+      const int64_t i = i0 + tx + 8 * p;
       if (i < n && i <= j) G[i + j * ldg] = csub(G[i + j * ldg], acc[p][q]);
     }
   }
@@ -376,10 +408,7 @@ cudaError_t trinv_rec(cudaStream_t s, int64_t n, const double2* U, int64_t ldu,
 std::once_flag g_attr_once[kMaxDevices];
 void set_attrs() {
   once_per_device(g_attr_once, []() {
-    cudaFuncSetAttribute(potf2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         2 * NB * NB * (int)sizeof(double2));
-    cudaFuncSetAttribute(panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         2 * NB * NB * (int)sizeof(double2));
+    cudaFuncSetAttribute(panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PANEL_SMEM);
     cudaFuncSetAttribute(trsm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (NB * RP + NB * NB + TK * RP + TK * NB) * (int)sizeof(double2));
   });
@@ -392,16 +421,16 @@ cudaError_t potrf_upper(cudaStream_t s, int64_t n, double2* G, int64_t ldg, doub
   set_attrs();
   cudaError_t e = cudaMemsetAsync(info, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  const size_t sm2 = 2 * NB * NB * sizeof(double2);
   for (int64_t k0 = 0, b = 0; k0 < n; k0 += NB, ++b) {
     const int kb = (int)std::min<int64_t>(NB, n - k0);
-    potf2_kernel<<<1, FT, sm2, s>>>(G, ldg, k0, kb, dinv + b * NB * NB, info); count_launch();
+    potf2_kernel<<<1, FT, 0, s>>>(G, ldg, k0, kb, dinv + b * NB * NB, info); count_launch();
     const int64_t rest = n - k0 - kb;
     if (rest > 0) {
-      panel_kernel<<<(unsigned)cdiv(rest, NB), FT, sm2, s>>>(n, G, ldg, k0, kb, dinv + b * NB * NB,
-                                                             info); count_launch();
-      const unsigned tt = (unsigned)cdiv(rest, NB);
-      trailing_kernel<<<dim3(tt, tt, 1), FT, 0, s>>>(n, G, ldg, k0, kb, info); count_launch();
+      panel_kernel<<<(unsigned)cdiv(rest, PC), FT, PANEL_SMEM, s>>>(n, G, ldg, k0, kb,
+                                                                    dinv + b * NB * NB, info);
+      count_launch();
+      const unsigned tt = (unsigned)cdiv(rest, TB);
+      trailing_kernel<<<dim3(tt, tt, 1), TT, 0, s>>>(n, G, ldg, k0, kb, info); count_launch();
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
