@@ -645,92 +645,129 @@ __device__ __forceinline__ int64_t bj_gidx(int a, int64_t i0, int ni, int64_t j0
   return a < ni ? i0 + a : j0 + (a - ni);
 }
 
-constexpr int BJ_INNER_SMEM = 2 * BJ_M * (BJ_M + 1) * (int)sizeof(float2);
+constexpr int BJ_IT = 512;           // threads of the inner kernel
+constexpr int BJ_P = BJ_M / 2;       // rotations of a round
+constexpr int BJ_LD = BJ_M + 1;
+constexpr int BJ_INNER_SMEM = 2 * BJ_M * BJ_LD * (int)sizeof(float2);
 
-__global__ void __launch_bounds__(BJ_T)
+// J = [[c, u], [-conj(u), c]] with u = s phi
+struct Jrot {
+  float c, ux, uy;
+  int on;
+};
+
+// One cyclic sweep on S (64 x 64, Hermitian, ld BJ_LD in shared memory; a
+// smaller matrix is padded with zeros, which no rotation touches), its rotations
+// accumulated into R, by BJ_IT threads. It is a chain of 63 rounds, so what
+// counts is a round's latency and its instructions: the 2 x 2 block of S where
+// pairs k < l meet is rotated from both sides at once (one barrier instead of
+// two), its mirror image is written and not computed, the pairs' own blocks are
+// set exactly by the threads that compute the rotations. Warp w takes the blocks
+// of pair w and of pair 31 - w, together one per lane, and rows w, w + 16, .. of
+// R, a lane per pair.
+__device__ __forceinline__ void bj_sweep(float2* S, float2* R, Jrot* rots, int2* pq) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  static_assert(BJ_P == 32 && BJ_IT / 32 == BJ_P / 2, "one pair per lane, two per warp");
+  // the off-diagonal block of this lane: pairs k < l
+  const bool lower = lane < warp;
+  const int k = lower ? BJ_P - 1 - warp : warp, l = lower ? BJ_P - 1 - lane : lane;
+  for (int rd = 0; rd < BJ_M - 1; ++rd) {
+    __syncthreads();
+    if (t < BJ_P) {
+      int p, q;
+      rr_pair(BJ_M, rd, t, p, q);
+      const RotT<float> r =
+          make_rot_t<float>(S[p * BJ_LD + p].x, S[q * BJ_LD + q].x, S[p * BJ_LD + q]);
+      Jrot j;
+      j.c = r.c;
+      j.ux = r.s * r.px;
+      j.uy = r.s * r.py;
+      j.on = r.s != 0.f;
+      rots[t] = j;
+      pq[t] = make_int2(p, q);
+      if (j.on) {  // the rotated 2 x 2 block exactly (no other thread reads it)
+        S[p * BJ_LD + p] = make_float2(r.app, 0.f);
+        S[q * BJ_LD + q] = make_float2(r.aqq, 0.f);
+        S[p * BJ_LD + q] = make_float2(0.f, 0.f);
+        S[q * BJ_LD + p] = make_float2(0.f, 0.f);
+      }
+    }
+    __syncthreads();
+    const Jrot jm = rots[lane];
+    const int2 pm = pq[lane];
+    if (k != l) {  // B <- J_k^H B J_l
+      const Jrot jk = rots[k], jl = rots[l];
+      if (jk.on | jl.on) {
+        const int2 pk = pq[k], pl = pq[l];
+        float2 b00 = S[pk.x * BJ_LD + pl.x], b01 = S[pk.x * BJ_LD + pl.y];
+        float2 b10 = S[pk.y * BJ_LD + pl.x], b11 = S[pk.y * BJ_LD + pl.y];
+        auto cols = [](float2& x, float2& y, const Jrot& j) {
+          const float2 nx = make_float2(j.c * x.x - (j.ux * y.x + j.uy * y.y),
+                                        j.c * x.y - (j.ux * y.y - j.uy * y.x));
+          y = make_float2(j.ux * x.x - j.uy * x.y + j.c * y.x,
+                          j.ux * x.y + j.uy * x.x + j.c * y.y);
+          x = nx;
+        };
+        auto rows = [](float2& x, float2& y, const Jrot& j) {
+          const float2 nx = make_float2(j.c * x.x - (j.ux * y.x - j.uy * y.y),
+                                        j.c * x.y - (j.ux * y.y + j.uy * y.x));
+          y = make_float2(j.ux * x.x + j.uy * x.y + j.c * y.x,
+                          j.ux * x.y - j.uy * x.x + j.c * y.y);
+          x = nx;
+        };
+        cols(b00, b01, jl);
+        cols(b10, b11, jl);
+        rows(b00, b10, jk);
+        rows(b01, b11, jk);
+        S[pk.x * BJ_LD + pl.x] = b00;
+        S[pk.x * BJ_LD + pl.y] = b01;
+        S[pk.y * BJ_LD + pl.x] = b10;
+        S[pk.y * BJ_LD + pl.y] = b11;
+        S[pl.x * BJ_LD + pk.x] = make_float2(b00.x, -b00.y);
+        S[pl.y * BJ_LD + pk.x] = make_float2(b01.x, -b01.y);
+        S[pl.x * BJ_LD + pk.y] = make_float2(b10.x, -b10.y);
+        S[pl.y * BJ_LD + pk.y] = make_float2(b11.x, -b11.y);
+      }
+    }
+    if (jm.on) {
+#pragma unroll
+      for (int h = 0; h < BJ_M / (BJ_IT / 32); ++h) {
+        float2* row = R + (warp + h * (BJ_IT / 32)) * BJ_LD;
+        const float2 x = row[pm.x], y = row[pm.y];
+        row[pm.x] = make_float2(jm.c * x.x - (jm.ux * y.x + jm.uy * y.y),
+                                jm.c * x.y - (jm.ux * y.y - jm.uy * y.x));
+        row[pm.y] = make_float2(jm.ux * x.x - jm.uy * x.y + jm.c * y.x,
+                                jm.ux * x.y + jm.uy * x.x + jm.c * y.y);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(BJ_IT)
     bj_inner_kernel(int64_t n, int nb, int nbp, int round, const float2* __restrict__ G,
                     float2* __restrict__ Rbuf) {
   extern __shared__ float2 bj_smem[];
-  float2 (*S)[BJ_M + 1] = reinterpret_cast<float2 (*)[BJ_M + 1]>(bj_smem);
-  float2 (*R)[BJ_M + 1] = reinterpret_cast<float2 (*)[BJ_M + 1]>(bj_smem + BJ_M * (BJ_M + 1));
-  __shared__ RotT<float> rots[BJ_M / 2];
-  __shared__ int pq[BJ_M / 2][2];  // this round's index pairs
-  const int k = blockIdx.x, t = threadIdx.x;
+  float2* S = bj_smem;
+  float2* R = bj_smem + BJ_M * BJ_LD;
+  __shared__ Jrot rots[BJ_P];
+  __shared__ int2 pq[BJ_P];  // a round's index pairs
+  const int t = threadIdx.x;
   int64_t i0, j0;
   int ni, nj;
-  bj_pair(n, nb, nbp, round, k, i0, ni, j0, nj);
+  bj_pair(n, nb, nbp, round, blockIdx.x, i0, ni, j0, nj);
   const int m = ni + nj;
-  // a full pair (m = 64, the common case): thread t always takes row/column
-  // t % 64 of the pairs t / 64, t / 64 + 4, ... (no index arithmetic per element)
-  static_assert(BJ_T % BJ_M == 0, "fixed element mapping");
-  const bool full = m == BJ_M;
-  for (int e = t; e < m * m; e += BJ_T) {
-    const int a = e % m, c = e / m;
-    S[a][c] = G[bj_gidx(a, i0, ni, j0) + bj_gidx(c, i0, ni, j0) * n];
-    R[a][c] = make_float2(a == c ? 1.f : 0.f, 0.f);
+  for (int e = t; e < BJ_M * BJ_M; e += BJ_IT) {
+    const int a = e % BJ_M, c = e / BJ_M;
+    S[a * BJ_LD + c] = (a < m && c < m)
+                           ? G[bj_gidx(a, i0, ni, j0) + bj_gidx(c, i0, ni, j0) * n]
+                           : make_float2(0.f, 0.f);
+    R[a * BJ_LD + c] = make_float2(a == c ? 1.f : 0.f, 0.f);
   }
-  __syncthreads();
-  const int mp = m + (m & 1);
-  for (int rd = 0; rd < mp - 1; ++rd) {
-    if (t < mp / 2) {
-      int p, q;
-      rr_pair(mp, rd, t, p, q);
-      pq[t][0] = p;
-      pq[t][1] = q;
-      rots[t] = q < m ? make_rot_t<float>(S[p][p].x, S[q][q].x, S[p][q])
-                      : make_rot_t<float>(0.f, 0.f, make_float2(0.f, 0.f));
-    }
-    __syncthreads();
-    if (full) {  // column rotations of S and R
-      const int i = t % BJ_M;
-#pragma unroll 4
-      for (int kk = t / BJ_M; kk < BJ_M / 2; kk += BJ_T / BJ_M) {
-        const RotT<float> r = rots[kk];
-        if (r.s == 0.f) continue;
-        const int p = pq[kk][0], q = pq[kk][1];
-        rot_cols_t(S[i][p], S[i][q], r);
-        rot_cols_t(R[i][p], R[i][q], r);
-      }
-    } else {
-      for (int e = t; e < (mp / 2) * m; e += BJ_T) {
-        const int kk = e / m, i = e % m;
-        const int p = pq[kk][0], q = pq[kk][1];
-        if (q >= m || rots[kk].s == 0.f) continue;
-        rot_cols_t(S[i][p], S[i][q], rots[kk]);
-        rot_cols_t(R[i][p], R[i][q], rots[kk]);
-      }
-    }
-    __syncthreads();
-    if (full) {  // row rotations of S
-      const int j = t % BJ_M;
-#pragma unroll 4
-      for (int kk = t / BJ_M; kk < BJ_M / 2; kk += BJ_T / BJ_M) {
-        const RotT<float> r = rots[kk];
-        if (r.s == 0.f) continue;
-        rot_rows_t(S[pq[kk][0]][j], S[pq[kk][1]][j], r);
-      }
-    } else {
-      for (int e = t; e < (mp / 2) * m; e += BJ_T) {
-        const int kk = e / m, j = e % m;
-        const int p = pq[kk][0], q = pq[kk][1];
-        if (q >= m || rots[kk].s == 0.f) continue;
-        rot_rows_t(S[p][j], S[q][j], rots[kk]);
-      }
-    }
-    __syncthreads();
-    if (t < mp / 2) {  // the rotated 2 x 2 block exactly
-      const int p = pq[t][0], q = pq[t][1];
-      if (q < m && rots[t].s != 0.f) {
-        S[p][p] = make_float2(rots[t].app, 0.f);
-        S[q][q] = make_float2(rots[t].aqq, 0.f);
-        S[p][q] = make_float2(0.f, 0.f);
-        S[q][p] = make_float2(0.f, 0.f);
-      }
-    }
-    __syncthreads();
-  }
-  float2* Rk = Rbuf + (int64_t)k * BJ_M * BJ_M;
-  for (int e = t; e < m * m; e += BJ_T) Rk[(e % m) + (e / m) * BJ_M] = R[e % m][e / m];
+  bj_sweep(S, R, rots, pq);
+  float2* Rk = Rbuf + (int64_t)blockIdx.x * BJ_M * BJ_M;
+  for (int e = t; e < m * m; e += BJ_IT)
+    Rk[(e % m) + (e / m) * BJ_M] = R[(e % m) * BJ_LD + e / m];
 }
 
 // Columns of the pair: M(r0:r0+64, idx) <- M(r0:r0+64, idx) R for M = G and Z.
@@ -921,7 +958,7 @@ int run_block_jacobi32(cudaStream_t s, int64_t n, float2* G, float2* Z, float2* 
     off_prev = off;
     if (sw == max_sweeps) break;
     for (int rd = 0; rd < nbp - 1; ++rd) {
-      bj_inner_kernel<<<npair, BJ_T, BJ_INNER_SMEM, s>>>(n, nb, nbp, rd, G, Rbuf);
+      bj_inner_kernel<<<npair, BJ_IT, BJ_INNER_SMEM, s>>>(n, nb, nbp, rd, G, Rbuf);
       bj_cols_kernel<<<dim3(gt, (unsigned)npair, 1), BJ_T, BJ_UPD_SMEM, s>>>(n, nb, nbp, rd, G, Z,
                                                                           Rbuf);
       bj_rows_kernel<<<dim3(gt, (unsigned)npair, 1), BJ_T, BJ_UPD_SMEM, s>>>(n, nb, nbp, rd, G,
