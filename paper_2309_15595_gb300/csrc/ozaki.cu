@@ -565,19 +565,56 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // |x| < 1/2: x = sum_s d_s 2^-8s + r with |r| <= 2^-49 and integer digits
 // |d_s| <= 128 (exact in BF16). X = rint(x 2^48) (|X| <= 2^47) is written in
 // balanced base 256, the low digits in [-128, 127] and the leading one in
-// [-128, 128]; so sum_s d_s 2^-8s = X 2^-48 exactly. Integer arithmetic: the
-// FP64 pipe (1/64 of the FP32 rate on this part) does one multiply and one
-// conversion per value instead of a multiply, a rounding and a subtraction
-// per digit.
-__device__ __forceinline__ void digits_of(double x, __nv_bfloat16* d) {
-  long long X = __double2ll_rn(x * 0x1p48);
+// [-128, 128]; so sum_s d_s 2^-8s = X 2^-48 exactly.
+//
+// The FP64 pipe runs at 1/64 of the FP32 rate on this part and conversions at a
+// half to a quarter of it, so everything below is integer work and FP32 adds:
+// X is the significand shifted and rounded to even, all low digits come from
+// the bytes of X + 0x8080808080 (the additions of 128 that balance each digit,
+// with their carries, done at once), and a byte b becomes the float b - 128
+// through the bit pattern of 2^23 + b. A BF16 digit is the upper half of that
+// float. (With FP64 scaling and one conversion per digit and format, slicing a
+// 20000-row matrix took 8.8 ms, 2.9 of the copy bandwidth's 6.8 TB/s.)
+__device__ __forceinline__ long long fixed48(double x, int e) {  // rint(x 2^(48 - e))
+  const long long b = __double_as_longlong(x);
+  const int E = (int)(b >> 52) & 0x7ff;
+  const long long m = (b & 0xfffffffffffffll) | (E ? 1ll << 52 : 0);
+  const int sh = 1027 - (E ? E : 1) + e;
+  if (E == 0x7ff || sh < 1) return __double2ll_rn(x * ldexp(1.0, -e) * 0x1p48);
+  if (sh > 53) return 0;
+  const long long X = (m + (1ll << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh;
+  return b < 0 ? -X : X;
+}
+struct Digits {
+  float d[OS];  // leading digit first
+};
+__device__ __forceinline__ Digits digits_of(double x, int e) {
+  const unsigned long long X = (unsigned long long)fixed48(x, e) + 0x8080808080ull;
+  const unsigned lo = (unsigned)X, hi = (unsigned)(X >> 32);
+  Digits r;
 #pragma unroll
-  for (int s = OS - 1; s > 0; --s) {
-    const int low = (int)(((unsigned)X + 128u) & 255u) - 128;  // X mod 256, balanced
-    d[s] = __float2bfloat16_rn((float)low);
-    X = (X - low) >> 8;  // exact: X - low is a multiple of 256
+  for (int s = 0; s < OS - 1; ++s) {  // byte s of X: digit OS - 1 - s
+    const unsigned f = __byte_perm(s < 4 ? lo : hi, 0x4b000000u, 0x7440u | (unsigned)(s & 3));
+    r.d[OS - 1 - s] = __uint_as_float(f) - 8388736.0f;  // 2^23 + 128
   }
-  d[0] = __float2bfloat16_rn((float)X);
+  r.d[0] = (float)((int)hi >> 8);
+  return r;
+}
+// BF16 of two digits, the first one in the lower half. Digits of finite values
+// have at most eight significant bits, so their lower halves are zero.
+__device__ __forceinline__ unsigned pack_digits(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+// max(|a.x|, |a.y|) and running maxima as bit patterns of non-negative doubles
+// (monotone in unsigned order); NaN counts as 0, as in fmax
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & ~(1ull << 63);
+  return b > 0x7ff0000000000000ull ? 0ull : b;
+}
+__device__ __forceinline__ unsigned long long max_bits(unsigned long long m, double2 a) {
+  const unsigned long long x = abs_bits(a.x), y = abs_bits(a.y);
+  m = x > m ? x : m;
+  return y > m ? y : m;
 }
 
 __device__ __forceinline__ int scale_exp(double mx) {
@@ -594,13 +631,13 @@ __global__ void rowmax_kernel(int64_t M, int64_t K, bool skip_diag, const double
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M) return;
   const int64_t k0 = (int64_t)blockIdx.y * 256, k1 = min(K, k0 + 256);
-  double m = 0.0;
+  unsigned long long m = 0;
+#pragma unroll 8
   for (int64_t k = k0; k < k1; ++k) {
     if (skip_diag && k == i) continue;  // the diagonal is applied separately, exactly
-    const double2 a = A[i + k * lda];
-    m = fmax(m, fmax(fabs(a.x), fabs(a.y)));
+    m = max_bits(m, A[i + k * lda]);
   }
-  atomicMax(&amax[i], (unsigned long long)__double_as_longlong(m));
+  atomicMax(&amax[i], m);
 }
 
 __global__ void diag_kernel(int64_t N, const double2* __restrict__ A, int64_t lda,
@@ -615,33 +652,39 @@ __global__ void exps_kernel(int64_t n, const unsigned long long* __restrict__ mx
 }
 
 // A (M x K, column-major) -> OS digit planes, each M rows x 2 Np (row-major
-// [Ar | Ai]), stacked; skip_diag leaves the diagonal out (square A).
-__global__ void slice_a_kernel(int64_t M, int64_t K, int64_t Np, bool skip_diag,
-                               const double2* __restrict__ A, int64_t lda,
-                               const int* __restrict__ ea, __nv_bfloat16* __restrict__ out) {
-  __shared__ double2 tile[32][33];
-  const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
+// [Ar | Ai]), stacked; skip_diag leaves the diagonal out (square A). A warp
+// writes a row of 64 entries, two per lane: 128 bytes of each of its 12 rows.
+constexpr int SA_K = 64;
+__global__ void __launch_bounds__(256)
+    slice_a_kernel(int64_t M, int64_t K, int64_t Np, bool skip_diag,
+                   const double2* __restrict__ A, int64_t lda, const int* __restrict__ ea,
+                   __nv_bfloat16* __restrict__ out) {
+  __shared__ double2 tile[SA_K][33];
+  const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * SA_K;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int r = ty; r < 32; r += 8) {
+#pragma unroll
+  for (int r = ty; r < SA_K; r += 8) {
     const int64_t i = i0 + tx, k = k0 + r;
-    tile[r][tx] = (i < M && k < K) ? A[i + k * lda] : make_double2(0.0, 0.0);
+    tile[r][tx] = (i < M && k < K && !(skip_diag && i == k)) ? A[i + k * lda]
+                                                             : make_double2(0.0, 0.0);
   }
   __syncthreads();
   const int64_t ld = 2 * Np;
   const size_t plane = (size_t)M * ld;
+  const int64_t k = k0 + 2 * tx;  // k + 1 may be K: the padding's digits are zero
+  if (k >= K) return;
   for (int r = ty; r < 32; r += 8) {
-    const int64_t i = i0 + r, k = k0 + tx;
-    if (i < M && k < K) {
-      const double2 a = (skip_diag && i == k) ? make_double2(0.0, 0.0) : tile[tx][r];
-      const double s = ldexp(1.0, -ea[i]);
-      __nv_bfloat16 dr[OS], di[OS];
-      digits_of(a.x * s, dr);
-      digits_of(a.y * s, di);
+    const int64_t i = i0 + r;
+    if (i >= M) continue;
+    const double2 a0 = tile[2 * tx][r], a1 = tile[2 * tx + 1][r];
+    const int e = ea[i];
+    const Digits r0 = digits_of(a0.x, e), r1 = digits_of(a1.x, e);
+    const Digits c0 = digits_of(a0.y, e), c1 = digits_of(a1.y, e);
+    __nv_bfloat16* o = out + i * ld + k;
 #pragma unroll
-      for (int d = 0; d < OS; ++d) {
-        out[d * plane + i * ld + k] = dr[d];
-        out[d * plane + i * ld + Np + k] = di[d];
-      }
+    for (int d = 0; d < OS; ++d) {
+      *reinterpret_cast<unsigned*>(o + d * plane) = pack_digits(r0.d[d], r1.d[d]);
+      *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
     }
   }
 }
@@ -654,85 +697,97 @@ __global__ void round_left_kernel(int64_t M, int64_t K, double2* __restrict__ X,
   const int64_t k = blockIdx.y;
   if (i >= M || k >= K) return;
   const double2 x = X[i + k * ldx];
-  const double s = ldexp(1.0, -ea[i]);
-  __nv_bfloat16 dr[OS], di[OS];
-  digits_of(x.x * s, dr);
-  digits_of(x.y * s, di);
-  double vr = 0.0, vi = 0.0;
-#pragma unroll
-  for (int d = OS - 1; d >= 0; --d) {  // exact: 48 bits below the scale
-    vr = (vr + __bfloat162float(dr[d])) * (1.0 / 256.0);
-    vi = (vi + __bfloat162float(di[d])) * (1.0 / 256.0);
-  }
-  X[i + k * ldx] = make_double2(ldexp(vr, ea[i]), ldexp(vi, ea[i]));
+  const int e = ea[i];
+  // exact: 48 bits below the scale
+  X[i + k * ldx] = make_double2(ldexp((double)fixed48(x.x, e), e - 48),
+                                ldexp((double)fixed48(x.y, e), e - 48));
 }
 
 // Left operand X^H for X (K x M, column-major): row i of X^H is conj(X[:, i]),
 // contiguous, so no transpose is needed. Exponents per row come from colexp.
+// Two entries per thread.
 __global__ void slice_ct_kernel(int64_t M, int64_t K, int64_t Np, const double2* __restrict__ X,
                                 int64_t ldx, const int* __restrict__ ea,
                                 __nv_bfloat16* __restrict__ out) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t i = blockIdx.y;
   if (k >= K) return;
-  const double2 x = X[k + i * ldx];
-  const double s = ldexp(1.0, -ea[i]);
-  __nv_bfloat16 dr[OS], di[OS];
-  digits_of(x.x * s, dr);
-  digits_of(-x.y * s, di);
+  const double2 x0 = X[k + i * ldx];
+  const double2 x1 = k + 1 < K ? X[k + 1 + i * ldx] : make_double2(0.0, 0.0);
+  const int e = ea[i];
+  const Digits r0 = digits_of(x0.x, e), r1 = digits_of(x1.x, e);
+  const Digits c0 = digits_of(-x0.y, e), c1 = digits_of(-x1.y, e);
   const int64_t ld = 2 * Np;
   const size_t plane = (size_t)M * ld;
+  __nv_bfloat16* o = out + i * ld + k;
 #pragma unroll
   for (int d = 0; d < OS; ++d) {
-    out[d * plane + i * ld + k] = dr[d];
-    out[d * plane + i * ld + Np + k] = di[d];
+    *reinterpret_cast<unsigned*>(o + d * plane) = pack_digits(r0.d[d], r1.d[d]);
+    *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
   }
 }
 
 // Column maxima of Y (complex columns j0 .. j0 + gridDim.x): one CTA per column.
-__global__ void colexp_kernel(int64_t N, int64_t j0, const double2* __restrict__ Y, int64_t ldy,
-                              int* __restrict__ eb) {
-  __shared__ double red[256];
-  const int64_t j = j0 + blockIdx.x;
-  double m = 0.0;
-  for (int64_t k = threadIdx.x; k < N; k += 256) {
-    const double2 y = Y[k + j * ldy];
-    m = fmax(m, fmax(fabs(y.x), fabs(y.y)));
+__device__ __forceinline__ unsigned long long block_max_bits(unsigned long long m,
+                                                             unsigned long long* red) {
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
+    m = o > m ? o : m;
   }
-  red[threadIdx.x] = m;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
-  for (int s = 128; s >= 1; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = red[w] > m ? red[w] : m;
+  return m;
+}
+__device__ __forceinline__ unsigned long long column_max(int64_t N, const double2* __restrict__ Y,
+                                                         unsigned long long* red) {
+  unsigned long long m = 0;
+#pragma unroll 4
+  for (int64_t k = threadIdx.x; k < N; k += 256) m = max_bits(m, Y[k]);
+  return block_max_bits(m, red);
+}
+__global__ void __launch_bounds__(256)
+    colexp_kernel(int64_t N, int64_t j0, const double2* __restrict__ Y, int64_t ldy,
+                  int* __restrict__ eb) {
+  __shared__ unsigned long long red[8];
+  const int64_t j = j0 + blockIdx.x;
+  const unsigned long long m = column_max(N, Y + j * ldy, red);
+  if (threadIdx.x == 0) eb[j] = scale_exp(__longlong_as_double((long long)m));
+}
+
+// Digits of entries k, k + 1 (zero past N) of one column of the right operand
+// into its rows of B^T. Real row: [Yr | -Yi]; imaginary row: [Yi | Yr].
+__device__ __forceinline__ void slice_b_pair(int64_t N, int64_t Np, size_t plane, int64_t k,
+                                             const double2* __restrict__ Y, int e,
+                                             __nv_bfloat16* __restrict__ re,
+                                             __nv_bfloat16* __restrict__ im) {
+  const double2 y0 = Y[k];
+  const double2 y1 = k + 1 < N ? Y[k + 1] : make_double2(0.0, 0.0);
+  const Digits r0 = digits_of(y0.x, e), r1 = digits_of(y1.x, e);
+  const Digits c0 = digits_of(y0.y, e), c1 = digits_of(y1.y, e);
+#pragma unroll
+  for (int d = 0; d < OS; ++d) {
+    const unsigned r = pack_digits(r0.d[d], r1.d[d]), c = pack_digits(c0.d[d], c1.d[d]);
+    *reinterpret_cast<unsigned*>(re + d * plane + k) = r;
+    *reinterpret_cast<unsigned*>(re + d * plane + Np + k) = c ^ 0x80008000u;
+    *reinterpret_cast<unsigned*>(im + d * plane + k) = c;
+    *reinterpret_cast<unsigned*>(im + d * plane + Np + k) = r;
   }
-  if (threadIdx.x == 0) eb[j] = scale_exp(red[0]);
 }
 
 // Y columns -> OS digit planes of B^T (rows: 32-column tiles of 64 rows), stacked
-// with `brows` rows per plane. Real row: [Yr | -Yi]; imaginary row: [Yi | Yr].
+// with `brows` rows per plane; two entries per thread.
 __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
                                const double2* __restrict__ Y, int64_t ldy, const int* __restrict__ eb,
                                __nv_bfloat16* __restrict__ out) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t j = j0 + blockIdx.y;
   if (k >= N) return;
-  const double2 y = Y[k + j * ldy];
-  const double s = ldexp(1.0, -eb[j]);
-  __nv_bfloat16 dr[OS], di[OS];
-  digits_of(y.x * s, dr);
-  digits_of(y.y * s, di);
-  const int64_t ld = 2 * Np;
-  const size_t plane = (size_t)brows * ld;
-  const int64_t br = brow_re(j), bi = br + CT;
-#pragma unroll
-  for (int d = 0; d < OS; ++d) {
-    __nv_bfloat16* o = out + d * plane;
-    const __nv_bfloat16 ndi = __hneg(di[d]);
-    o[br * ld + k] = dr[d];
-    o[br * ld + Np + k] = ndi;
-    o[bi * ld + k] = di[d];
-    o[bi * ld + Np + k] = dr[d];
-  }
+  const int64_t ld = 2 * Np, br = brow_re(j);
+  slice_b_pair(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], out + br * ld,
+               out + (br + CT) * ld);
 }
 
 // The right-operand digits of many problems' filter steps in one launch: one
@@ -749,8 +804,7 @@ struct OzSliceEntry {
 
 __global__ void __launch_bounds__(256)
     slice_b_grouped_kernel(const OzSliceEntry* __restrict__ tab, int count) {
-  __shared__ double red[256];
-  __shared__ int s_e;
+  __shared__ unsigned long long red[8];
   const int id = (int)blockIdx.x;
   int lo = 0, hi = count - 1;
   while (lo < hi) {  // last entry with first <= id
@@ -761,41 +815,11 @@ __global__ void __launch_bounds__(256)
   const OzSliceEntry& e = tab[lo];
   const int64_t N = e.N, j = e.j0 + (id - e.first);
   const double2* __restrict__ Y = e.B + j * e.ldb;
-  double m = 0.0;
-  for (int64_t k = threadIdx.x; k < N; k += 256) {
-    const double2 y = Y[k];
-    m = fmax(m, fmax(fabs(y.x), fabs(y.y)));
-  }
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = 128; w >= 1; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    s_e = scale_exp(red[0]);
-    e.eb[j] = s_e;
-  }
-  __syncthreads();
-  const double sc = ldexp(1.0, -s_e);
-  const int64_t ld = 2 * e.Np;
-  const size_t plane = (size_t)e.brows * ld;
-  const int64_t br = brow_re(j), bi = br + CT;
-  for (int64_t k = threadIdx.x; k < N; k += 256) {
-    const double2 y = Y[k];
-    __nv_bfloat16 dr[OS], di[OS];
-    digits_of(y.x * sc, dr);
-    digits_of(y.y * sc, di);
-#pragma unroll
-    for (int d = 0; d < OS; ++d) {
-      __nv_bfloat16* o = e.out + d * plane;
-      const __nv_bfloat16 ndi = __hneg(di[d]);
-      o[br * ld + k] = dr[d];
-      o[br * ld + e.Np + k] = ndi;
-      o[bi * ld + k] = di[d];
-      o[bi * ld + e.Np + k] = dr[d];
-    }
-  }
+  const int ex = scale_exp(__longlong_as_double((long long)column_max(N, Y, red)));
+  if (threadIdx.x == 0) e.eb[j] = ex;
+  const int64_t ld = 2 * e.Np, br = brow_re(j);
+  for (int64_t k = 2 * threadIdx.x; k < N; k += 512)
+    slice_b_pair(N, e.Np, (size_t)e.brows * ld, k, Y, ex, e.out + br * ld, e.out + (br + CT) * ld);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 lookup_encoder() {
@@ -920,7 +944,7 @@ cudaError_t ozaki_prepare_a(cudaStream_t s, const double2* A, int64_t lda, Ozaki
   count_launch();
   diag_kernel<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(N, A, lda, w.diag);
   count_launch();
-  slice_a_kernel<<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, 32), 1), dim3(32, 8, 1), 0, s>>>(
+  slice_a_kernel<<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
       N, N, w.Np, true, A, lda, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
   count_launch();
   w.A_ready = A;
@@ -935,7 +959,7 @@ cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const doub
   // digits of the active columns of B
   colexp_kernel<<<(unsigned)n, 256, 0, s>>>(N, j0, B, ldb, w.eb);
   count_launch();
-  slice_b_kernel<<<dim3((unsigned)cdiv(N, 256), (unsigned)n, 1), 256, 0, s>>>(
+  slice_b_kernel<<<dim3((unsigned)cdiv(N, 512), (unsigned)n, 1), 256, 0, s>>>(
       N, w.Np, w.brows, j0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
   count_launch();
   const Maps* maps = static_cast<const Maps*>(w.maps);
@@ -966,7 +990,7 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
   if (conj_trans) {  // left = X^H, X is K x M
     colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
     count_launch();
-    slice_ct_kernel<<<dim3((unsigned)cdiv(K, 256), (unsigned)M, 1), 256, 0, s>>>(M, K, Kp, X, ldx,
+    slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(M, K, Kp, X, ldx,
                                                                                  w.el, L);
     count_launch();
   } else {           // left = X, M x K
@@ -976,14 +1000,14 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
     count_launch();
     exps_kernel<<<(unsigned)cdiv(M, 256), 256, 0, s>>>(M, w.amax, w.el);
     count_launch();
-    slice_a_kernel<<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, 32), 1), dim3(32, 8, 1), 0, s>>>(
+    slice_a_kernel<<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
         M, K, Kp, false, X, ldx, w.el, L);
     count_launch();
   }
   // right operand digits, K rows
   colexp_kernel<<<(unsigned)ncols, 256, 0, s>>>(K, 0, B, ldb, w.eb);
   count_launch();
-  slice_b_kernel<<<dim3((unsigned)cdiv(K, 256), (unsigned)ncols, 1), 256, 0, s>>>(
+  slice_b_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)ncols, 1), 256, 0, s>>>(
       K, Kp, w.brows, 0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
   count_launch();
   CUtensorMap ma, mb;
