@@ -90,6 +90,15 @@ __device__ bool converged_rule(double off, double fro, double off_prev) {
 
 // ------------------------------------------------- single-CTA batched version
 constexpr int SJ_MAX = 64, SJ_T = 256;
+// Eigenproblems of order up to kSmallFp64 run in FP64 in one CTA; its time grows
+// like n^3 (one SM has two DFMA a clock: 5 ms at n = 60, about 0.4 ms at 24), so
+// larger ones start in FP32 (0.3 ms in one CTA) and refine in FP64 on many SMs
+// (0.1 ms a step).
+constexpr int64_t kSmallFp64 = 24;
+// Largest order whose FP64 refinement multiplies on the CUDA cores: a product of
+// order 64 takes 20 us there and, with the digits of both operands, 60 us on the
+// tensor cores.
+constexpr int64_t kCoreRefine = 128;
 
 __global__ void __launch_bounds__(SJ_T)
     jacobi_small_kernel(int n, const double2* __restrict__ Gin, double* __restrict__ w,
@@ -770,6 +779,82 @@ __global__ void __launch_bounds__(BJ_IT)
     Rk[(e % m) + (e / m) * BJ_M] = R[(e % m) * BJ_LD + e / m];
 }
 
+// The FP32 stage of a matrix of order n <= 64 in one CTA: sweeps with the
+// stopping rule of run_block_jacobi32, eigenvectors written in FP64 (ld n). The
+// matrix is scaled by a power of two into FP32's range; *bad = 1 when it holds an
+// infinity or NaN.
+__global__ void __launch_bounds__(BJ_IT)
+    jacobi32_small_kernel(int n, const double2* __restrict__ G, int64_t ldg, int max_sweeps,
+                          double tol_conv, double tol_stag, double2* __restrict__ X,
+                          double* __restrict__ bad) {
+  extern __shared__ float2 bj_smem[];
+  float2* S = bj_smem;
+  float2* R = bj_smem + BJ_M * BJ_LD;
+  __shared__ Jrot rots[BJ_P];
+  __shared__ int2 pq[BJ_P];
+  __shared__ float red[BJ_IT / 32][2];
+  __shared__ int s_exp;  // largest exponent field
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) s_exp = 0;
+  __syncthreads();
+  int ex = 0;
+  for (int e = t; e < n * n; e += BJ_IT) {
+    const double2 v = G[e % n + e / n * ldg];
+    ex = max(ex, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+  }
+  atomicMax(&s_exp, ex);
+  __syncthreads();
+  const int sh = 1023 - s_exp;
+  if (t == 0) *bad = s_exp == 0x7ff ? 1.0 : 0.0;
+  for (int e = t; e < BJ_M * BJ_M; e += BJ_IT) {
+    const int a = e % BJ_M, c = e / BJ_M;
+    float2 g = make_float2(0.f, 0.f);
+    if (a < n && c < n) {
+      const double2 v = G[a + c * ldg];
+      g = make_float2((float)ldexp(v.x, sh), (float)ldexp(v.y, sh));
+    }
+    S[a * BJ_LD + c] = g;
+    R[a * BJ_LD + c] = make_float2(a == c ? 1.f : 0.f, 0.f);
+  }
+  double off_prev = 1e300;
+  for (int sw = 0; sw <= max_sweeps; ++sw) {
+    __syncthreads();
+    float o = 0.f, d = 0.f;
+    for (int e = t; e < BJ_M * BJ_M; e += BJ_IT) {
+      const int a = e % BJ_M, c = e / BJ_M;
+      const float2 g = S[a * BJ_LD + c];
+      const float v = fmaf(g.x, g.x, g.y * g.y);
+      if (a == c) d += v;
+      else o += v;
+    }
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+      o += __shfl_xor_sync(0xffffffffu, o, w);
+      d += __shfl_xor_sync(0xffffffffu, d, w);
+    }
+    if (lane == 0) {
+      red[warp][0] = o;
+      red[warp][1] = d;
+    }
+    __syncthreads();
+    double so = 0.0, sf = 0.0;
+#pragma unroll
+    for (int w = 0; w < BJ_IT / 32; ++w) {
+      so += red[w][0];
+      sf += red[w][1];
+    }
+    const double off = sqrt(so), fro = sqrt(so + sf);
+    if (off == 0.0 || off <= tol_conv * fro || (off <= tol_stag * fro && off > 0.25 * off_prev))
+      break;
+    off_prev = off;
+    if (sw < max_sweeps) bj_sweep(S, R, rots, pq);
+  }
+  for (int e = t; e < n * n; e += BJ_IT) {
+    const float2 r = R[(e % n) * BJ_LD + e / n];
+    X[e] = make_double2((double)r.x, (double)r.y);
+  }
+}
+
 // Columns of the pair: M(r0:r0+64, idx) <- M(r0:r0+64, idx) R for M = G and Z.
 __global__ void __launch_bounds__(BJ_T)
     bj_cols_kernel(int64_t n, int nb, int nbp, int round, float2* __restrict__ G,
@@ -916,6 +1001,16 @@ __global__ void bj_norms_kernel(int64_t n, const float2* __restrict__ G, double*
 }
 
 std::once_flag g_bj_attr[kMaxDevices];
+void set_bj_attrs() {
+  once_per_device(g_bj_attr, []() {
+    cudaFuncSetAttribute(bj_inner_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         BJ_INNER_SMEM);
+    cudaFuncSetAttribute(jacobi32_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         BJ_INNER_SMEM);
+    cudaFuncSetAttribute(bj_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
+    cudaFuncSetAttribute(bj_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
+  });
+}
 
 // Blocked FP32 Jacobi on G (n x n, destroyed) with eigenvectors into Z (starts
 // as I): sweeps until off(G) <= tol_conv ||G||_F, or <= tol_stag ||G||_F with
@@ -924,12 +1019,7 @@ std::once_flag g_bj_attr[kMaxDevices];
 int run_block_jacobi32(cudaStream_t s, int64_t n, float2* G, float2* Z, float2* Rbuf,
                        double* part, double* host_part, int max_sweeps, double tol_conv,
                        double tol_stag, int* sweeps, bool* conv) {
-  once_per_device(g_bj_attr, []() {
-    cudaFuncSetAttribute(bj_inner_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         BJ_INNER_SMEM);
-    cudaFuncSetAttribute(bj_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
-    cudaFuncSetAttribute(bj_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
-  });
+  set_bj_attrs();
   const int nb = (int)cdiv(n, BJ_B);
   const int nbp = nb + (nb & 1);
   const int npair = nbp / 2;
@@ -1029,7 +1119,10 @@ __global__ void oa_e_kernel(int64_t n, const double2* __restrict__ S,
       const double lj = lam[j], d = lj - lam[i];
       const double2 num = make_double2(fma(lj, r.x, sv.x), fma(lj, r.y, sv.y));
       const double an = sqrt(num.x * num.x + num.y * num.y);
-      if (an <= 1e-3 * fabs(d)) {
+      if (an == 0.0 && d == 0.0) {  // equal values without coupling: no pair to finish
+        e = make_double2(0.5 * r.x, 0.5 * r.y);
+        emax = 0.5 * sqrt(r.x * r.x + r.y * r.y);
+      } else if (an <= 1e-3 * fabs(d)) {
         e = make_double2(num.x / d, num.y / d);
         emax = an / fabs(d);
       } else {
@@ -1354,11 +1447,10 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
                 int* cluster_out) {
   if (cluster_out) cluster_out[0] = cluster_out[1] = cluster_out[2] = 0;
   if (n <= 0) return CHASE_OK;
-  cudaError_t e;
   int* status = reinterpret_cast<int*>(wk.red + 2 * kCoopMaxGrid + 8);
-  if (n <= SJ_MAX) {
-    // pack G (ld n) into Gw, run the single-CTA kernel into Zw, copy to Z.
-    e = cudaMemsetAsync(status, 0, sizeof(int), s);
+  // FP64 in one CTA: G (ld n) into Gw, the single-CTA kernel into Zw, copied to Z
+  auto small_fp64 = [&]() -> int {
+    cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), s);
     if (e != cudaSuccess) return CHASE_CUDA_FAIL();
     e = cudaMemcpy2DAsync(wk.Gw, n * sizeof(double2), G, ldg * sizeof(double2),
                           n * sizeof(double2), n, cudaMemcpyDeviceToDevice, s);
@@ -1374,35 +1466,45 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
     if (cudaStreamSynchronize(s) != cudaSuccess) return CHASE_CUDA_FAIL();
     if (sweeps_out) *sweeps_out = 0;
     return hs ? CHASE_ERR_HEEV_NOCONV : CHASE_OK;
-  }
+  };
+  if (n <= kSmallFp64) return small_fp64();
   // --- FP32 sweeps on the converted matrix
   const dim3 g2((unsigned)cdiv(n, 128), (unsigned)n, 1);
-  init32_kernel<<<g2, 128, 0, s>>>(n, G, ldg, wk.G32a, wk.Z32); count_launch();
   int sw32 = 0;
   bool conv32 = false;
   // stage caps: 30 FP32 sweeps, 8 refinement steps, kMaxSweeps FP64 sweeps, each
   // lowered to the caller's cap when one is set
   auto cap = [&](int def) { return wk.max_sweeps > 0 ? std::min(def, wk.max_sweeps) : def; };
-  // blocked FP32 Jacobi: G32a is G (in place), Rb the block rotations
-  if (jacobi_rot_elems(n) > wk.rb_elems) return CHASE_ERR_INVALID_ARG;
-  RC_(run_block_jacobi32(s, n, wk.G32a, wk.Z32, wk.Rb, wk.red, wk.host_part, cap(30), 4e-6, 1e-4,
-                         &sw32, &conv32));
+  constexpr double kTol32 = 4e-6, kStag32 = 1e-4;
+  double* out2 = wk.red + 2 * kCoopMaxGrid + 12;  // two maxima; [2]: non-finite input
+  if (n <= BJ_M) {
+    set_bj_attrs();
+    jacobi32_small_kernel<<<1, BJ_IT, BJ_INNER_SMEM, s>>>((int)n, G, ldg, cap(30), kTol32, kStag32,
+                                                          wk.Zw, out2 + 2);
+    count_launch();
+  } else {
+    init32_kernel<<<g2, 128, 0, s>>>(n, G, ldg, wk.G32a, wk.Z32); count_launch();
+    // blocked FP32 Jacobi: G32a is G (in place), Rb the block rotations
+    if (jacobi_rot_elems(n) > wk.rb_elems) return CHASE_ERR_INVALID_ARG;
+    RC_(run_block_jacobi32(s, n, wk.G32a, wk.Z32, wk.Rb, wk.red, wk.host_part, cap(30), kTol32,
+                           kStag32, &sw32, &conv32));
+    promote_kernel<<<g2, 128, 0, s>>>(n, wk.Z32, wk.Zw); count_launch();
+  }
   // --- FP64: refine the FP32 eigenvectors (Ogita-Aishima steps, FP64 GEMMs)
-  promote_kernel<<<g2, 128, 0, s>>>(n, wk.Z32, wk.Zw); count_launch();
   const unsigned gb = (unsigned)cdiv(n, 256);
   const int64_t nb = (int64_t)gb * n;  // partial slots (2 doubles each) of the E kernel
   double* lam = wk.params;             // n eigenvalue estimates (params is free here)
-  double* out2 = wk.red + 2 * kCoopMaxGrid + 12;
   double2* X = wk.Zw;
   double2* Xn = wk.Zw2;
   // scale of G for the cluster test
   frob2_kernel<<<dim3(gb, (unsigned)n, 1), 256, 0, s>>>(n, G, ldg, reinterpret_cast<double*>(wk.T));
   count_launch();
   max2_kernel<<<1, 256, 0, s>>>(nb, reinterpret_cast<double*>(wk.T), out2); count_launch();
-  if (cudaMemcpyAsync(wk.host_red, out2, 2 * sizeof(double), cudaMemcpyDeviceToHost, s) !=
+  if (cudaMemcpyAsync(wk.host_red, out2, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return CHASE_CUDA_FAIL();
+  if (n <= BJ_M && wk.host_red[2] != 0.0) return CHASE_ERR_HEEV_NOCONV;
   // sqrt(n) times the largest norm of a 256-row column segment: within a factor
   // sqrt(n) of ||G||_2 either way, enough for the 1e-14 cluster test below
   const double gscale = wk.host_red[0] * std::sqrt((double)n);
@@ -1417,7 +1519,8 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
   // rounding of the operands, a few 2^-48 of ||G||, like the CUDA-core FP64
   // products' sqrt(n) 2^-53), and so does the final orthogonalisation. Without
   // them, all products are the CUDA-core FP64 ones.
-  const bool tc = wk.gemm != nullptr;
+  // Up to order kCoreRefine those are the faster ones too.
+  const bool tc = wk.gemm != nullptr && n > kCoreRefine;
   bool fine = false;
   const int max_refine = cap(8);
   for (; refine < max_refine; ++refine) {  // 2-4 steps from FP32 accuracy; a slow start gets more
@@ -1491,7 +1594,10 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
   double2* Zfinal = X;
   double* wsrc = lam;
   bool clustered = false;
-  if (conv && cmax > 1e-14 * gscale) {
+  // couplings of pairs left together that are finished: below 64 columns the
+  // clusters cost little, and those of a close spectrum add up
+  const double cfinish = (n <= BJ_M ? 1e-16 : 1e-14) * gscale;
+  if (conv && cmax > cfinish) {
     // pairs the refinement could not separate: FP64 Jacobi on each cluster of
     // them alone (their couplings to every other vector are already at FP64
     // level); falls through to full FP64 sweeps when the clusters are too many
@@ -1507,7 +1613,8 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
       cluster_out[2] = cinfo[1];           // clusters (or recorded pairs if not used)
     }
   }
-  if (!conv || (cmax > 1e-14 * gscale && !clustered)) {
+  if (!conv || (cmax > cfinish && !clustered)) {
+    if (n <= SJ_MAX) return small_fp64();
     // pairs the refinement could not separate (or no convergence): FP64 Jacobi
     // sweeps on G' = X^H G X finish them; eigenvectors X Z'
     Epilogue ep{};
