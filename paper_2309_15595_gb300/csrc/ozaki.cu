@@ -75,6 +75,8 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr int KPAD = 128;                // K-half padding: 2 Np is a multiple of 256
 constexpr int HC = TN / 4;               // complex columns per epilogue warp half (16)
 constexpr int CT = TN / 2;               // complex columns per tile (32)
+constexpr int kEpiThreads = 256;         // epilogue warps' threads
+static_assert(2 * HC * kEpiThreads * 16 <= STAGES * STAGE_BYTES, "the sums fit the ring");
 constexpr unsigned long long kWaitLimitNs = 4000000000ull;
 constexpr unsigned kGroup = 8;           // row blocks per sweep of the column tiles
 
@@ -253,16 +255,103 @@ struct Params {
   const double* theta;        // resid
   double* partial;            // resid: [32-row tile + col * ceil(N / 32)]
   int* err;
+  int nrow, ncol;             // tiles
+  int split;                  // CTAs that share a tile's K range
 };
 
+// ------------------------------------------------------- cluster helpers
+// Cluster-wide barrier (release / acquire): every thread of every CTA arrives.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Rank in the cluster of part 0 of this CTA's tile.
+__device__ __forceinline__ unsigned cluster_base(int split, unsigned part) {
+  return split > 1 ? cluster_rank() - part : 0u;
+}
+// The same shared-memory variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t remote_smem(const void* p, unsigned rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ long long ld_cluster(uint32_t a, long long*) {
+  long long v;
+  asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a, float*) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
+// (acc 2^24 + low) 2^(e - 64), rounded to nearest even, in integer operations (the
+// FP64 pipe's conversions and adds took most of a tile's epilogue).
+__device__ __forceinline__ double fixed_to_double(long long acc, long long low, int e) {
+  acc += low >> 24;
+  unsigned lo = (unsigned)low & 0xffffffu;
+  const bool neg = acc < 0;
+  if (neg) {
+    acc = lo ? ~acc : -acc;
+    lo = lo ? (1u << 24) - lo : 0u;
+  }
+  const unsigned long long A = (unsigned long long)acc;
+  const int n = __clzll((long long)A);
+  unsigned long long W;
+  unsigned rest = 0;
+  int ex = e - 64;
+  if (n >= 24) {
+    W = (A << 24) | lo;
+  } else {
+    const int sh = 24 - n;
+    W = (A << n) | (lo >> sh);
+    rest = lo & ((1u << sh) - 1u);
+    ex += sh;
+  }
+  if (W == 0) return 0.0;
+  const int z = __clzll((long long)W);
+  W <<= z;
+  ex -= z;
+  unsigned long long m = W >> 11;  // 53 bits
+  const unsigned tail = (unsigned)W & 0x7ffu;
+  if (tail > 0x400u || (tail == 0x400u && (rest != 0 || (m & 1)))) ++m;
+  const int E = ex + 1086;
+  if (E < 1 || E > 2045) {
+    const double v = ldexp((double)m, ex + 11);
+    return neg ? -v : v;
+  }
+  return __longlong_as_double((long long)((((unsigned long long)E << 52) + (m - (1ull << 52))) |
+                                          ((unsigned long long)neg << 63)));
+}
+__device__ __forceinline__ long long low_fixed(long long v) { return v; }
+__device__ __forceinline__ long long low_fixed(float v) { return __float2ll_rn(v * 65536.0f); }
+
 // ---------------------------------------------------------------- kernel
-// One 128 x 64 output tile (row block rb, column tile ct of the active
-// columns); the per-problem kernel and the grouped kernel (the filter steps
-// of many problems in one launch) both run it.
+// CTA `local` of a product: tile local / split (128 x 64 outputs), part local %
+// split of its chunks; the per-problem kernel and the grouped kernel (the filter
+// steps of many problems in one launch) both run it. The CTAs of a tile are
+// consecutive ranks of a cluster: each leaves its sums in its own shared memory
+// and then adds up and finishes 1 / split of the tile's columns. clustered: the
+// launch has clusters of more than one CTA, all of which meet at the two cluster
+// barriers; CTAs past the last tile (padding of a group's problem) only do that.
 template <int LMAX>
 __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtensorMap* tmB,
-                                           const Params& P, unsigned rb, unsigned ct,
-                                           bool maps_in_global) {
+                                           const Params& P, unsigned local, bool maps_in_global,
+                                           bool clustered) {
+  const unsigned part = local % (unsigned)P.split;
+  if (local / (unsigned)P.split >= (unsigned)P.nrow * (unsigned)P.ncol) {
+    cluster_sync();
+    cluster_sync();
+    return;
+  }
+  unsigned rb, ct;  // row block and column tile (grouped raster order)
+  grouped_tile(local / (unsigned)P.split, (unsigned)P.nrow, (unsigned)P.ncol, kGroup, rb, ct);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
@@ -270,11 +359,18 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
   __shared__ int s_abort;
 
+  // the epilogue's sums, in the ring once that is free: [2 HC][kEpiThreads]
+  using Acc67 = typename std::conditional<LMAX == 8, long long, float>::type;
+  long long* acc_s = reinterpret_cast<long long*>(smem);
+  Acc67* low_s = reinterpret_cast<Acc67*>(acc_s + 2 * HC * kEpiThreads);
+
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t m0 = (int64_t)rb * TM;
   const int64_t tile = P.j0 / CT + ct;            // absolute CT-column tile
-  const int nkb = (int)((2 * P.Np) / TK);
-  const int nchunks = nkb / CHUNK_KB;
+  const int nchunks_all = (int)((2 * P.Np) / TK) / CHUNK_KB;
+  const int chunk0 = (int)part * nchunks_all / P.split;  // this CTA's chunks
+  const int nchunks = ((int)part + 1) * nchunks_all / P.split - chunk0;
+  const int nkb = nchunks * CHUNK_KB;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -298,6 +394,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
+  bool go = true;
   if (warp == 0) {
     if (lane == 0) {  // ------------------------------------ TMA producer
       if (maps_in_global) {  // tensor maps read from global memory by the TMA unit
@@ -318,7 +415,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
         const uint32_t full = smem_u32(&bars[s]);
         uint8_t* st = smem + s * STAGE_BYTES;
         mbar_expect_tx(full, STAGE_BYTES);
-        const int kx = kb * TK;
+        const int kx = (chunk0 * CHUNK_KB + kb) * TK;
 #pragma unroll
         for (int d = 0; d < OS; ++d) {
           // digit planes are stacked along rows: digit d of row r is row d * rows + r
@@ -359,7 +456,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
             // levels restart often enough to stay exact integers: see kDrain2, kDrain3
             const bool r = kc == 0 && kk == 0;
             digit_pairs<LMAX>(tmem, st + off, st + OS * A_TILE + off, r && c % kDrain2 == 0,
-                              r && c % kDrain3 == 0, r);
+                              r && c % kDrain3 == 0, r);  // c = 0 restarts all
           }
           umma_commit(smem_u32(&bars[STAGES + s]));
         }
@@ -374,7 +471,6 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
     // ------------------------------------------------------- epilogue warps
     const int q = warp & 3;                   // TMEM lane quarter
     const int h = (warp - 2) >> 2;            // complex column half: [h*24, h*24+24)
-    const int64_t row = m0 + q * 32 + lane;
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
     long long acc[2 * HC];                    // re[0..16), im[16..32): levels 2-5, weight 2^-40
     // levels 6-LMAX. In FP32 at weight 2^-48; in the extended variant in int64 at
@@ -382,15 +478,12 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
     // coherently (sum_k d_3(x_k)^2 grows like K), where FP32 sums over
     // K = 80000 lost about 2^-44 of the scale (orthogonality 2e-11 at
     // N = 40000 after CholeskyQR2); per chunk the values stay below 2^25.
-    using Acc67 = typename std::conditional<LMAX == 8, long long, float>::type;
-    constexpr double kW67 = LMAX == 8 ? 0x1p-64 : 0x1p-48;
     Acc67 acc67[2 * HC];
 #pragma unroll
     for (int j = 0; j < 2 * HC; ++j) {
       acc[j] = 0;
       acc67[j] = Acc67(0);
     }
-    bool go = true;
     for (int c = 0; c < nchunks; ++c) {
       const bool ok = mbar_wait(smem_u32(&bars[2 * STAGES]), (uint32_t)c & 1u, P.err, 15);
       go = __all_sync(0xffffffffu, ok && !*(volatile int*)&s_abort);
@@ -461,61 +554,110 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars[2 * STAGES + 1]));
     }
-    // ------------------------------------------------ FP64 result + update
-    double rsq[HC];
-    if (go && row < P.N) {
-      const double sa = ldexp(1.0, P.escale_a[row]);
-      const double2 dg = P.diag ? P.diag[row] : make_double2(0.0, 0.0);
+    // the ring is free: every MMA of this CTA has been waited for above
+    const int e = (warp - 2) * 32 + lane;
 #pragma unroll
-      for (int jj = 0; jj < HC; ++jj) {
-        const int64_t col = tile * CT + h * HC + jj;
-        rsq[jj] = 0.0;
-        if (col < P.j0 || col >= P.ncols) continue;
-        const double sc = sa * ldexp(1.0, P.escale_b[col]);
-        const double2 b = P.diag ? P.Bsrc[row + col * P.ldbs] : make_double2(0.0, 0.0);
-        const double lr = fma((double)acc[jj], 0x1p-40, (double)acc67[jj] * kW67);
-        const double li = fma((double)acc[HC + jj], 0x1p-40, (double)acc67[HC + jj] * kW67);
-        const double wr = fma(dg.x, b.x, fma(-dg.y, b.y, sc * lr));
-        const double wi = fma(dg.x, b.y, fma(dg.y, b.x, sc * li));
+    for (int j = 0; j < 2 * HC; ++j) {
+      acc_s[j * kEpiThreads + e] = acc[j];
+      low_s[j * kEpiThreads + e] = acc67[j];
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  __syncwarp();
+  if (clustered) cluster_sync();
+  if (warp >= 2 && go) {
+    // ------------------------------------------------ FP64 result + update
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    const int64_t row = m0 + q * 32 + lane;
+    const int e = (warp - 2) * 32 + lane;
+    const bool in_row = row < P.N;
+    const int ea = in_row ? P.escale_a[row] : 0;
+    const double2 dg = (in_row && P.diag) ? P.diag[row] : make_double2(0.0, 0.0);
+    // A_ii B_ij - gamma X_ij as one product where X is the right operand (gamma
+    // is the column's Ritz value in the residual)
+    const bool same = P.diag && P.mode != EPI_STORE && P.X == P.Bsrc && P.ldx == P.ldbs;
+    const double dgx = P.alpha * (dg.x - P.gamma), dgy = P.alpha * dg.y;
+    const double ag = P.alpha * P.gamma;
+    const unsigned base = cluster_base(P.split, part);
+    const int64_t nt32 = (P.N + 31) / 32, t32 = (int64_t)rb * 4 + q;
+    const int per = HC / P.split;
+#pragma unroll 2
+    for (int i = 0; i < per; ++i) {
+      const int jj = (int)part * per + i;
+      const int64_t col = tile * CT + h * HC + jj;
+      const bool in = in_row && col >= P.j0 && col < P.ncols;
+      double rsq = 0.0;
+      double2 x = make_double2(0.0, 0.0), y0 = x, b = x;
+      if (in) {
+        if (P.mode != EPI_STORE && (same || P.mode == EPI_RESID || P.gamma != 0.0))
+          x = P.X[row + col * P.ldx];
+        if (P.diag && !same) b = P.Bsrc[row + col * P.ldbs];
+        if (P.mode == EPI_FILTER && P.beta != 0.0) y0 = P.Y[row + col * P.ldy];
+        long long hr = acc_s[jj * kEpiThreads + e], hi = acc_s[(HC + jj) * kEpiThreads + e];
+        Acc67 lr = low_s[jj * kEpiThreads + e], li = low_s[(HC + jj) * kEpiThreads + e];
+        if (P.split > 1) {
+          hr = hi = 0;
+          lr = li = Acc67(0);
+          for (int p = 0; p < P.split; ++p) {
+            const unsigned rk = base + (unsigned)p;
+            hr += ld_cluster(remote_smem(acc_s + jj * kEpiThreads + e, rk), acc_s);
+            hi += ld_cluster(remote_smem(acc_s + (HC + jj) * kEpiThreads + e, rk), acc_s);
+            lr += ld_cluster(remote_smem(low_s + jj * kEpiThreads + e, rk), low_s);
+            li += ld_cluster(remote_smem(low_s + (HC + jj) * kEpiThreads + e, rk), low_s);
+          }
+        }
+        const int ex = ea + P.escale_b[col];
+        double wr = fixed_to_double(hr, low_fixed(lr), ex);
+        double wi = fixed_to_double(hi, low_fixed(li), ex);
+        if (P.diag && !same) {
+          wr = fma(dg.x, b.x, wr);
+          wi = fma(dg.x, b.y, wi);
+          if (dg.y != 0.0) {
+            wr = fma(-dg.y, b.y, wr);
+            wi = fma(dg.y, b.x, wi);
+          }
+        }
+        double2* yp = P.Y + row + col * P.ldy;
         if (P.mode == EPI_STORE) {
-          P.Y[row + col * P.ldy] = make_double2(wr, wi);
+          *yp = make_double2(wr, wi);
         } else if (P.mode == EPI_FILTER) {
-          const double2 x = P.X[row + col * P.ldx];
-          double2* yp = P.Y + row + col * P.ldy;
-          double vr = P.alpha * fma(-P.gamma, x.x, wr);
-          double vi = P.alpha * fma(-P.gamma, x.y, wi);
+          double vr = P.alpha * wr, vi = P.alpha * wi;
+          if (same) {
+            vr = fma(dgx, x.x, vr);
+            vi = fma(dgx, x.y, vi);
+            if (dgy != 0.0) {
+              vr = fma(-dgy, x.y, vr);
+              vi = fma(dgy, x.x, vi);
+            }
+          } else if (P.gamma != 0.0) {
+            vr = fma(-ag, x.x, vr);
+            vi = fma(-ag, x.y, vi);
+          }
           if (P.beta != 0.0) {
-            const double2 y0 = *yp;
             vr = fma(P.beta, y0.x, vr);
             vi = fma(P.beta, y0.y, vi);
           }
           *yp = make_double2(vr, vi);
         } else {
-          const double2 x = P.X[row + col * P.ldx];
           const double th = P.theta[col];
-          const double dx = fma(-th, x.x, wr), dy = fma(-th, x.y, wi);
-          rsq[jj] = fma(dx, dx, dy * dy);
+          const double f = same ? dg.x - th : -th;
+          double dx = fma(f, x.x, wr), dy = fma(f, x.y, wi);
+          if (same && dg.y != 0.0) {
+            dx = fma(-dg.y, x.y, dx);
+            dy = fma(dg.y, x.x, dy);
+          }
+          rsq = fma(dx, dx, dy * dy);
         }
       }
-    } else {
+      if (P.mode == EPI_RESID) {
+        // per column: sum over this warp's 32 rows, one partial per 32-row tile
 #pragma unroll
-      for (int jj = 0; jj < HC; ++jj) rsq[jj] = 0.0;
-    }
-    if (P.mode == EPI_RESID && go) {
-      // per column: sum over this warp's 32 rows, one partial per 32-row tile
-      const int64_t nt32 = (P.N + 31) / 32;
-      const int64_t t32 = (int64_t)rb * 4 + q;
-#pragma unroll
-      for (int jj = 0; jj < HC; ++jj) {
-        double v = rsq[jj];
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        const int64_t col = tile * CT + h * HC + jj;
-        if (lane == 0 && t32 < nt32 && col >= P.j0 && col < P.ncols) P.partial[t32 + col * nt32] = v;
+        for (int off = 16; off >= 1; off >>= 1) rsq += __shfl_xor_sync(0xffffffffu, rsq, off);
+        if (lane == 0 && t32 < nt32 && col >= P.j0 && col < P.ncols) P.partial[t32 + col * nt32] = rsq;
       }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
+  if (clustered) cluster_sync();  // the others have read this CTA's sums
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -529,9 +671,7 @@ template <int LMAX>
 __global__ void __launch_bounds__(NTHREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       Params P) {
-  unsigned rb, ct;  // row block and column tile of this CTA (grouped raster order)
-  grouped_tile(blockIdx.x + blockIdx.y * gridDim.x, gridDim.x, gridDim.y, kGroup, rb, ct);
-  ozaki_tile<LMAX>(&tmA, &tmB, P, rb, ct, false);
+  ozaki_tile<LMAX>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
 }
 
 // Many problems' filter steps in one launch: entry p of the table holds problem
@@ -542,11 +682,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 struct OzGroupEntry {  // aligned as its tensor maps
   CUtensorMap a, b;
   Params P;
-  int first, nrow, ncol, pad;
+  int first, pad;
 };
 
 __global__ void __launch_bounds__(NTHREADS, 1)
-    ozaki_filter_grouped_kernel(const OzGroupEntry* __restrict__ tab, int count) {
+    ozaki_filter_grouped_kernel(const OzGroupEntry* __restrict__ tab, int count, bool clustered) {
   const int id = (int)blockIdx.x;
   int lo = 0, hi = count - 1;
   while (lo < hi) {  // last entry with first <= id
@@ -556,9 +696,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   const OzGroupEntry* e = tab + lo;
   const Params P = e->P;
-  unsigned rb, ct;
-  grouped_tile((unsigned)(id - e->first), (unsigned)e->nrow, (unsigned)e->ncol, kGroup, rb, ct);
-  ozaki_tile<7>(&e->a, &e->b, P, rb, ct, true);
+  ozaki_tile<7>(&e->a, &e->b, P, (unsigned)(id - e->first), true, clustered);
 }
 
 // ------------------------------------------------------------ digit prep
@@ -853,6 +991,58 @@ struct Maps {
   CUtensorMap a, b;
 };
 
+// CTAs per tile. A tile costs its chunks plus about one chunk's time to start
+// and, undivided, one and a half to finish; a wave of tiles takes as long as its
+// slowest. Tiles that fill the chip several times over stay whole; a product of
+// few tiles (the 8 of a 512 x 60 block, the 30 of a 316 x 316 Gram over 9273
+// rows) is cut so that its parts fill one wave. A cut has to gain a tenth: parts
+// read the right operand no less often and meet at two cluster barriers. It
+// depends on the product alone, so a problem's result is the same in a group.
+constexpr int kMaxSplit = 8;
+int choose_split(int64_t tiles, int64_t Np) {
+  const int64_t nchunks = 2 * Np / (TK * CHUNK_KB), sms = num_sms();
+  int best = 1;
+  double best_cost = 1e300;
+  for (int s = 1; s <= kMaxSplit && s <= nchunks; s *= 2) {
+    const double cost =
+        (double)cdiv(tiles * s, sms) * ((double)cdiv(nchunks, s) + 1.0 + 1.5 / s);
+    if (cost < 0.9 * best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return best;
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned ctas, int cluster, cudaStream_t s,
+                            Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas, 1, 1);
+  cfg.blockDim = dim3(NTHREADS, 1, 1);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+cudaError_t launch_product(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b,
+                           const Params& P, bool extended) {
+  const unsigned ctas = (unsigned)P.nrow * (unsigned)P.ncol * (unsigned)P.split;
+  return launch_clusters(extended ? ozaki_gemm_kernel<8> : ozaki_gemm_kernel<7>, ctas, P.split, s,
+                         a, b, P);
+}
+void set_tiles(Params& P) {
+  P.nrow = (int)cdiv(P.N, TM);
+  P.ncol = (int)((P.ncols - 1) / CT - P.j0 / CT + 1);
+  P.split = choose_split((int64_t)P.nrow * P.ncol, P.Np);
+}
+
 // Launch parameters of A * B[:, j0:ncols_end] with epilogue ep (A's digits in w).
 Params product_params(const OzakiWork& w, int64_t ncols_end, int64_t j0, const double2* B,
                       int64_t ldb, const Epilogue& ep) {
@@ -879,6 +1069,7 @@ Params product_params(const OzakiWork& w, int64_t ncols_end, int64_t j0, const d
   P.theta = ep.theta;
   P.partial = ep.partial;
   P.err = w.err;
+  set_tiles(P);
   return P;
 }
 
@@ -964,10 +1155,7 @@ cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const doub
   count_launch();
   const Maps* maps = static_cast<const Maps*>(w.maps);
   const Params P = product_params(w, ncols_end, j0, B, ldb, ep);
-  const dim3 grid((unsigned)cdiv(N, TM), (unsigned)((ncols_end - 1) / CT - j0 / CT + 1), 1);
-  ozaki_gemm_kernel<7><<<grid, NTHREADS, SMEM_BYTES, s>>>(maps->a, maps->b, P);
-  count_launch();
-  return cudaGetLastError();
+  return launch_product(s, maps->a, maps->b, P, false);
 }
 
 cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const double2* X,
@@ -1037,13 +1225,8 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
   P.theta = ep.theta;
   P.partial = ep.partial;
   P.err = w.err;
-  const dim3 grid((unsigned)cdiv(M, TM), (unsigned)((ncols - 1) / CT + 1), 1);
-  if (extended)
-    ozaki_gemm_kernel<8><<<grid, NTHREADS, SMEM_BYTES, s>>>(ma, mb, P);
-  else
-    ozaki_gemm_kernel<7><<<grid, NTHREADS, SMEM_BYTES, s>>>(ma, mb, P);
-  count_launch();
-  return cudaGetLastError();
+  set_tiles(P);
+  return launch_product(s, ma, mb, P, extended);
 }
 
 cudaError_t ozaki_round_left(cudaStream_t s, int64_t M, int64_t K, double2* X, int64_t ldx,
@@ -1135,7 +1318,7 @@ int ozaki_filter_grouped(cudaStream_t s, int count, const OzakiGroupItem* items,
   OzGroupEntry* host = static_cast<OzGroupEntry*>(t.host);
   OzSliceEntry* shost = static_cast<OzSliceEntry*>(t.shost);
   std::vector<size_t> off(dmax_all + 2, 0);
-  std::vector<int> ctas(dmax_all + 1, 0), cols(dmax_all + 1, 0);
+  std::vector<int> ctas(dmax_all + 1, 0), cols(dmax_all + 1, 0), cluster(dmax_all + 1, 1);
   size_t n = 0;
   for (int i = 1; i <= dmax_all; ++i) {
     off[i] = n;
@@ -1175,12 +1358,15 @@ int ozaki_filter_grouped(cudaStream_t s, int count, const OzakiGroupItem* items,
       e.a = maps->a;
       e.b = maps->b;
       e.P = product_params(w, it.ncols, j0, buf[sp], ld[sp], ep);
-      e.nrow = (int)cdiv(it.N, TM);
-      e.ncol = (int)((it.ncols - 1) / CT - j0 / CT + 1);
-      e.first = first;
       e.pad = 0;
-      first += e.nrow * e.ncol;
+      cluster[i] = std::max(cluster[i], e.P.split);
       ++n;
+    }
+    // a cluster holds CTAs of one problem: each starts on a cluster boundary
+    for (size_t q = off[i]; q < n; ++q) {
+      host[q].first = first;
+      first += (int)cdiv((int64_t)host[q].P.nrow * host[q].P.ncol * host[q].P.split, cluster[i]) *
+               cluster[i];
     }
     ctas[i] = first;
     cols[i] = sfirst;
@@ -1203,9 +1389,8 @@ int ozaki_filter_grouped(cudaStream_t s, int count, const OzakiGroupItem* items,
     const int cnt = (int)(off[i + 1] - off[i]);
     slice_b_grouped_kernel<<<(unsigned)cols[i], 256, 0, s>>>(sdev + off[i], cnt);
     count_launch();
-    ozaki_filter_grouped_kernel<<<(unsigned)ctas[i], NTHREADS, SMEM_BYTES, s>>>(dev + off[i],
-                                                                               cnt);
-    count_launch();
+    launch_clusters(ozaki_filter_grouped_kernel, (unsigned)ctas[i], cluster[i], s, dev + off[i], cnt,
+                    cluster[i] > 1);
   }
   const cudaError_t ce = cudaStreamEndCapture(s, &graph);
   if (ce != cudaSuccess || !graph) return CHASE_CUDA_FAIL();
