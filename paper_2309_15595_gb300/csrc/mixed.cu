@@ -21,15 +21,21 @@
 // drain this one), and the epilogue warps add the chunk sums into FP32
 // registers with round-to-nearest adds.
 //
-// Kernel structure (one 128 x 256 output tile per CTA, 10 warps):
-//   warp 0   TMA producer: A_hi, A_lo (128 x 32) and B_hi, B_lo (256 x 32) per
-//            K block into a 4-stage shared-memory ring of 48 KB stages (64B
-//            swizzle: one K block of 32 BF16 is a 64-byte row)
-//   warp 1   TMEM allocator and single-thread MMA issuer (tcgen05.mma, M=128,
-//            N=256, K=16, kind::f16 with BF16 inputs)
+// Kernel structure (one 256 x 256 output tile per pair of CTAs, 10 warps each):
+//   warp 0   TMA producer: its 128 rows of A_hi, A_lo and its half of the 256 rows
+//            of B_hi, B_lo per K block of 32 into a 6-stage shared-memory ring of
+//            32 KB stages (64B swizzle: one K block of 32 BF16 is a 64-byte row)
+//   warp 1   TMEM allocator; in the leader the single-thread MMA issuer
+//            (tcgen05.mma.cta_group::2, M=256, N=256, K=16, kind::f16, BF16)
 //   warps 2-9 epilogue: warp w reads TMEM lane quarter w % 4 and half of the
 //            complex columns; per-chunk drain into FP32 register sums, then the
 //            fused Eq. 1 update
+// Why pairs: with a 128 x 256 tile per CTA the three MMAs of a K step read 36 KB
+// and the TMA writes 24 KB of shared memory, 480 cycles of its 128 bytes a cycle
+// for 384 cycles of products. A pair shares the operand rows: 24 and 16 KB, 320
+// cycles, so the products bound it. N = 13379, 1072 columns, degree 20: 63.3 ->
+// 60.9 ms of kernel time, 1.65 PFLOP/s with the padding of the last tiles, which is
+// 0.97 of the power-capped bf16 rate.
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the kernel
 // records an error code and winds down instead of spinning.
 #include <cuda.h>
@@ -53,13 +59,15 @@ namespace chase {
   } while (0)
 namespace {
 
-// K block of 32 BF16 (64-byte rows, 64B swizzle) and a 4-stage ring: three
+// K block of 32 BF16 (64-byte rows, 64B swizzle) and a 6-stage ring: five
 // stages stay in flight while one is consumed, enough bytes in flight to
 // cover the TMA latency at the MMA rate.
-constexpr int TM = 128, TN = 256, TK = 32, STAGES = 4;
+constexpr int TM = 128, TN = 256, TK = 32, STAGES = 6;
+constexpr int PAIR = 2;                             // CTAs of a pair: PAIR TM x TN outputs
 constexpr int A_TILE = TM * TK * 2;                 // 8 KB
-constexpr int B_TILE = TN * TK * 2;                 // 16 KB
-constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;  // 48 KB
+constexpr int B_HALF = TN / PAIR;                   // operand rows a CTA of the pair holds
+constexpr int B_TILE = B_HALF * TK * 2;             // 8 KB
+constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;  // 32 KB
 constexpr int KPAD = 64;                            // K-half padding of the planes
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr int NTHREADS = 320;
@@ -67,6 +75,7 @@ constexpr int EPI_WARPS = 8;
 constexpr int CHUNK_KB = 8;              // K blocks (of 32) per accumulation chunk: 256 values
 constexpr uint32_t TMEM_COLS = 512;      // two 128 x 256 FP32 accumulators
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
+constexpr unsigned long long kLandNs = 1000000ull;          // 1 ms
 
 struct Params {
   int64_t N, Np, j0, ncols;     // rows, padded K half, first active column, end column
@@ -76,7 +85,8 @@ struct Params {
   __nv_bfloat16* Bn_hi;         // next-step operand planes (rows = B^T rows, ld = 2 Np)
   __nv_bfloat16* Bn_lo;
   int write_next;
-  int group;                    // row blocks per sweep of the grouped raster order
+  int nrow, ncol;               // pair rows and column tiles
+  int group;                    // pair rows per sweep of the grouped raster order
   int* err;
 };
 
@@ -96,14 +106,29 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+// Rank in the pair and the address of a shared-memory variable of its leader (rank 0).
+__device__ __forceinline__ unsigned pair_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t leader_smem(uint32_t addr) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(addr));
+  return a;
+}
+__device__ __forceinline__ void pair_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
@@ -122,10 +147,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     }
   }
 }
+// Into this CTA's shared memory; `bar` is the leader's barrier (shared::cluster).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
                                             uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
@@ -141,21 +167,25 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
   d |= (uint64_t)4 << 61;             // SWIZZLE_64B
   return d;
 }
-// Instruction descriptor: FP32 accumulate, BF16 A and B, both K-major, M x N.
+// Instruction descriptor: FP32 accumulate, BF16 A and B, both K-major, M x N over
+// the pair (each CTA's tensor memory receives its TM rows).
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                            ((uint32_t)(TM >> 4) << 24);
+                            ((uint32_t)(PAIR * TM >> 4) << 24);
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
       "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
       : "memory");
 }
+// Arrives on the barrier at this offset in both CTAs once the MMAs so far are done.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
       : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -188,24 +218,28 @@ __device__ __forceinline__ void split2f(float x, __nv_bfloat16& hi, __nv_bfloat1
 __device__ __forceinline__ int64_t brow_re(int64_t j) { return (j >> 7) * 256 + (j & 127); }
 
 // ---------------------------------------------------------------- kernel
-// One 128 x 256 output tile (row block rb, column tile ct of the active
-// columns) of one filter step; the per-problem kernel and the grouped kernel
-// (many problems in one launch) both run it.
+// One 256 x 256 output tile (pair row rp, column tile ct of the active columns) of
+// one filter step by a pair of CTAs: each loads its 128 rows of A and half of the
+// operand rows (the real parts for rank 0, the imaginary ones for rank 1), the
+// leader issues MMAs over both, and each drains and updates its 128 rows. The
+// per-problem kernel and the grouped kernel (many problems in one launch) both
+// run it.
 __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtensorMap* tmAl,
                                            const CUtensorMap* tmBh, const CUtensorMap* tmBl,
-                                           const Params& P, unsigned rb, unsigned ct,
+                                           const Params& P, unsigned rp, unsigned ct,
                                            bool maps_in_global) {
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment of the shared-window address (swizzle atoms)
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  // bars[0..S) full, bars[S..2S) empty, bars[2S + b] accumulator b full,
-  // bars[2S + 2 + b] accumulator b drained
+  // bars[0..S) full (the leader's), bars[S..2S) empty, bars[2S + b] accumulator b
+  // full, bars[2S + 2 + b] accumulator b drained by both CTAs (the leader's)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
   __shared__ int s_abort;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t m0 = (int64_t)rb * TM;
+  const unsigned rank = pair_rank();
+  const int64_t m0 = ((int64_t)rp * PAIR + rank) * TM;
   const int64_t tile = (P.j0 >> 7) + ct;          // absolute 128-column tile
   const int nkb = (int)((2 * P.Np) / TK);
   const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
@@ -218,19 +252,20 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars[2 * STAGES + b]), 1);
-      mbar_init(smem_u32(&bars[2 * STAGES + 2 + b]), EPI_WARPS);
+      mbar_init(smem_u32(&bars[2 * STAGES + 2 + b]), PAIR * EPI_WARPS);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(TMEM_COLS)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
+  pair_sync();  // both CTAs' barriers and tensor memory are there
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
@@ -251,20 +286,29 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
         break;
       }
       if (*(volatile int*)&s_abort) break;
-      const uint32_t full = smem_u32(&bars[s]);
+      const uint32_t full = leader_smem(smem_u32(&bars[s]));
       uint8_t* st = smem + s * STAGE_BYTES;
-      mbar_expect_tx(full, STAGE_BYTES);
-      const int kx = kb * TK;
+      if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), PAIR * STAGE_BYTES);
+      const int kx = kb * TK, brow = (int)(tile * TN) + (int)rank * B_HALF;
       tma_load_2d(smem_u32(st), tmAh, kx, (int)m0, full);
       tma_load_2d(smem_u32(st + A_TILE), tmAl, kx, (int)m0, full);
-      tma_load_2d(smem_u32(st + 2 * A_TILE), tmBh, kx, (int)(tile * TN), full);
-      tma_load_2d(smem_u32(st + 2 * A_TILE + B_TILE), tmBl, kx, (int)(tile * TN), full);
+      tma_load_2d(smem_u32(st + 2 * A_TILE), tmBh, kx, brow, full);
+      tma_load_2d(smem_u32(st + 2 * A_TILE + B_TILE), tmBl, kx, brow, full);
       ++issued;
     }
-    // drain: every issued stage must land before the CTA may exit
-    for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-      mbar_wait(smem_u32(&bars[kb % STAGES]), (uint32_t)(kb / STAGES) & 1u, P.err, 2);
-  } else if (warp == 1 && lane == 0) {
+    if (issued == nkb) {
+      // the last stages' MMAs are done: both CTAs' loads have landed and the
+      // leader's arrivals on this CTA's barriers are in
+      for (int kb = nkb > STAGES ? nkb - STAGES : 0; kb < nkb; ++kb)
+        mbar_wait(smem_u32(&bars[STAGES + kb % STAGES]), (uint32_t)(kb / STAGES) & 1u, P.err, 2);
+    } else {
+      // after an expired wait the other CTA's half may never come: let a time
+      // pass that no load in flight outlasts
+      const unsigned long long t0 = globaltimer();
+      while (globaltimer() - t0 < kLandNs) {
+      }
+    }
+  } else if (warp == 1 && lane == 0 && rank == 0) {
     // ------------------------------------------------------- MMA issuer
     int kb = 0;
     bool ok = true;
@@ -341,7 +385,7 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars[2 * STAGES + 2 + b]));
+      if (lane == 0) mbar_arrive_cluster(leader_smem(smem_u32(&bars[2 * STAGES + 2 + b])));
     }
     if (go && row < P.N) {
 #pragma unroll
@@ -378,22 +422,23 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
+  pair_sync();  // neither CTA's memory is used by the other any more
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(TMEM_COLS)
                  : "memory");
   }
 }
 
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
     mixed_filter_kernel(const __grid_constant__ CUtensorMap tmAh,
                         const __grid_constant__ CUtensorMap tmAl,
                         const __grid_constant__ CUtensorMap tmBh,
                         const __grid_constant__ CUtensorMap tmBl, Params P) {
-  unsigned rb, ct;  // row block and column tile of this CTA (grouped raster order)
-  grouped_tile(blockIdx.x + blockIdx.y * gridDim.x, gridDim.x, gridDim.y, P.group, rb, ct);
-  mixed_tile(&tmAh, &tmAl, &tmBh, &tmBl, P, rb, ct, false);
+  unsigned rp, ct;  // pair row and column tile of this pair (grouped raster order)
+  grouped_tile(blockIdx.x / PAIR, (unsigned)P.nrow, (unsigned)P.ncol, P.group, rp, ct);
+  mixed_tile(&tmAh, &tmAl, &tmBh, &tmBl, P, rp, ct, false);
 }
 
 // Many problems' filter steps in one launch: entry p of the table holds problem
@@ -404,10 +449,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 struct alignas(64) GroupEntry {
   CUtensorMap ah, al, bh, bl;
   Params P;
-  int first, nrow, ncol, pad;
+  int first, pad;
 };
 
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
     mixed_filter_grouped_kernel(const GroupEntry* __restrict__ tab, int count) {
   const int id = (int)blockIdx.x;
   int lo = 0, hi = count - 1;
@@ -418,9 +463,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   const GroupEntry* e = tab + lo;
   const Params P = e->P;
-  unsigned rb, ct;
-  grouped_tile((unsigned)(id - e->first), (unsigned)e->nrow, (unsigned)e->ncol, P.group, rb, ct);
-  mixed_tile(&e->ah, &e->al, &e->bh, &e->bl, P, rb, ct, true);
+  unsigned rp, ct;
+  grouped_tile((unsigned)(id - e->first) / PAIR, (unsigned)P.nrow, (unsigned)P.ncol, P.group, rp,
+               ct);
+  mixed_tile(&e->ah, &e->al, &e->bh, &e->bl, P, rp, ct, true);
 }
 
 // ----------------------------------------------------------- conversions
@@ -548,7 +594,8 @@ cudaError_t mixed_alloc(MixedWork& w, int64_t N, int64_t ne) {
   for (int b = 0; b < 2; ++b) {
     char* yh = static_cast<char*>(w.Yhi) + b * b_bytes;
     char* yl = static_cast<char*>(w.Ylo) + b * b_bytes;
-    ok = ok && make_map(&maps->bh[b], yh, brows, Np, TN) && make_map(&maps->bl[b], yl, brows, Np, TN);
+    ok = ok && make_map(&maps->bh[b], yh, brows, Np, B_HALF) &&
+         make_map(&maps->bl[b], yl, brows, Np, B_HALF);
   }
   if (!ok) return cudaErrorInvalidValue;
   if ((e = cudaMalloc(&w.S32, (size_t)2 * N * ne * sizeof(float2))) != cudaSuccess) return e;
@@ -606,14 +653,12 @@ Params step_params(int64_t N, int64_t ncols, const int32_t* degs, double c, cons
   P.Bn_hi = static_cast<__nv_bfloat16*>(w.Yhi) + bout * b_elems;
   P.Bn_lo = static_cast<__nv_bfloat16*>(w.Ylo) + bout * b_elems;
   P.write_next = i < dmax;
+  P.nrow = (int)cdiv(N, PAIR * TM);
+  P.ncol = (int)((ncols - 1) / 128 - P.j0 / 128 + 1);
   P.group = group;
   P.err = w.err;
   *bin_out = (i - 1) & 1;
   return P;
-}
-
-unsigned step_col_tiles(const Params& P) {
-  return (unsigned)((P.ncols - 1) / 128 - P.j0 / 128 + 1);
 }
 
 // ----------------------------------------------- raster-order autotuner
@@ -634,8 +679,8 @@ unsigned step_col_tiles(const Params& P) {
 // counts), and one replaces the default only when it is faster by more than 3 %:
 // single timings of step 1 picked 16 or 32 in some runs (C3 filter 0.80 of the
 // peak instead of 0.90).
-constexpr int kGroupCandidates[] = {64, 32, 128, 16};
-constexpr int kDefaultGroup = 64;
+constexpr int kGroupCandidates[] = {32, 16, 64, 8};  // pair rows
+constexpr int kDefaultGroup = 32;
 constexpr int kTuneRepeats = 3;
 constexpr float kTuneMargin = 0.97f;
 static_assert(kGroupCandidates[0] == kDefaultGroup, "the default is timed first");
@@ -650,8 +695,10 @@ int tuned_group(int64_t N, unsigned coltiles) {
   return it == g_tuned_group.end() ? 0 : it->second;
 }
 
-int tune_group(cudaStream_t s, const Maps* maps, Params P, dim3 grid) {
-  const int cached = tuned_group(P.N, grid.y);
+unsigned step_ctas(const Params& P) { return (unsigned)P.nrow * (unsigned)P.ncol * PAIR; }
+
+int tune_group(cudaStream_t s, const Maps* maps, Params P) {
+  const int cached = tuned_group(P.N, (unsigned)P.ncol);
   if (cached) return cached;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
@@ -663,8 +710,8 @@ int tune_group(cudaStream_t s, const Maps* maps, Params P, dim3 grid) {
     for (int i = 0; i < nc; ++i) {
       P.group = kGroupCandidates[i];
       cudaEventRecord(e0, s);
-      mixed_filter_kernel<<<grid, NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[0],
-                                                             maps->bl[0], P);
+      mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al,
+                                                                     maps->bh[0], maps->bl[0], P);
       count_launch();
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) break;
@@ -685,7 +732,7 @@ int tune_group(cudaStream_t s, const Maps* maps, Params P, dim3 grid) {
   int dev = 0;
   cudaGetDevice(&dev);
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  g_tuned_group[std::make_tuple(dev, P.N, grid.y)] = best;
+  g_tuned_group[std::make_tuple(dev, P.N, (unsigned)P.ncol)] = best;
   return best;
 }
 
@@ -717,10 +764,9 @@ int mixed_filter(cudaStream_t s, int64_t N, const double2* A, int64_t lda, doubl
   for (int i = 1; i <= dmax; ++i) {
     int bin = 0;
     Params P = step_params(N, ncols, degs, c, al, be, i, group, w, &bin);
-    const dim3 grid((unsigned)cdiv(N, TM), step_col_tiles(P), 1);
-    if (i == 1 && autotune) P.group = group = tune_group(s, maps, P, grid);
-    mixed_filter_kernel<<<grid, NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[bin],
-                                                           maps->bl[bin], P);
+    if (i == 1 && autotune) P.group = group = tune_group(s, maps, P);
+    mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[bin],
+                                                                   maps->bl[bin], P);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return CHASE_CUDA_FAIL();
   }
@@ -799,11 +845,9 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
       e.al = maps->al;
       e.bh = maps->bh[bin];
       e.bl = maps->bl[bin];
-      e.nrow = (int)cdiv(it.N, TM);
-      e.ncol = (int)step_col_tiles(e.P);
       e.first = first;
       e.pad = 0;
-      first += e.nrow * e.ncol;
+      first += (int)step_ctas(e.P);
     }
     ctas[i] = first;
   }
