@@ -14,96 +14,105 @@ constexpr int NB = kNB;  // 64
 constexpr int FT = 256;  // threads
 
 // Unblocked Cholesky of the kb x kb diagonal block at (k0, k0) and the inverse
-// of the resulting upper-triangular block, in registers.
+// of the resulting upper-triangular block, in the registers of a cluster.
 //
 // The elimination that turns G into U turns an identity beside it into
 // V = U^-H, and the two fit one 64 x 64 array: U on and above the diagonal, V
 // below it. Step j subtracts conj(M(j, r)) M(j, c) / p_j from M(r, c) for all
 // r > j and c >= r (U) or c <= j (V); rows are divided by their sqrt(p) at the
-// end. Each of the 256 threads owns 16 entries, a warp an 8 x 4 patch of every
-// 16 x 16 block, so patches that a step does not touch cost nothing on the
-// FP64 pipe (2 DFMA a clock on this one SM: 85 us for the 87 thousand complex
-// multiply-adds, which is what bounds the kernel). The owner of the next pivot
-// takes its reciprocal square root while the others still update, and the row
-// buffer alternates, so a step has one barrier.
-__device__ __forceinline__ bool pivot_rsqrt(double p, double* rd) {
-  const bool ok = p > 0.0;  // false for NaN too
-  *rd = ok ? rsqrt(p) : 0.0;
-  return ok;
+// end. One SM's FP64 pipe (2 DFMA a clock) takes 85 us for the 87 thousand complex
+// multiply-adds (208 us measured with the patches' idle lanes), so the columns go
+// to the four CTAs of a cluster, 4 of every 16 each; a thread owns one row of its
+// CTA's columns, four entries. The owners of the next row write it into every CTA's
+// shared memory, the owner of the next pivot its reciprocal root, and a step ends
+// with one cluster barrier (the row buffer alternates).
+constexpr int PF_C = 4;
+__device__ __forceinline__ uint32_t remote_smem(const void* p, unsigned rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(a)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(FT)
+__global__ void __cluster_dims__(PF_C, 1, 1) __launch_bounds__(FT)
     potf2_kernel(double2* G, int64_t ldg, int64_t k0, int kb, double2* dinv_blk, int* info) {
   __shared__ double2 row_s[2][NB];  // raw row j of M, 1 at column j
-  __shared__ double rd_s[NB];       // 1 / sqrt(p_j)
-  __shared__ int ok_s[NB];
+  __shared__ double rd_s[NB];       // 1 / sqrt(p_j), 0 if p_j is not positive
   if (*info != 0) return;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int rl = (warp & 1) * 8 + (lane & 7), cl = (warp >> 1) * 4 + (lane >> 3);
-  double2 m[4][4];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, rank = blockIdx.x;
+  static_assert(FT / 32 * 8 == NB && PF_C * 4 * 4 == NB, "rows by warps, columns by CTAs");
+  const int r = warp * 8 + (lane & 7), c0 = 4 * rank + (lane >> 3);
+  double2 m[4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int b = 0; b < 4; ++b) {
+    const int c = 16 * b + c0;
+    m[b] = (r <= c && c < kb) ? G[(k0 + r) + (k0 + c) * ldg] : make_double2(0.0, 0.0);
+  }
+  auto publish = [&](int j) {
+    if (r != j) return;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      const int r = 16 * a + rl, c = 16 * b + cl;
-      m[a][b] = (r <= c && c < kb) ? G[(k0 + r) + (k0 + c) * ldg] : make_double2(0.0, 0.0);
-    }
-  // raw row j from its owners; the pivot's owner also takes its root
-  auto publish = [&](int j) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      if (16 * a + rl != j) continue;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = 16 * b + cl;
-        row_s[j & 1][c] = c == j ? make_double2(1.0, 0.0) : m[a][b];
-        if (c == j) ok_s[j] = pivot_rsqrt(m[a][b].x, &rd_s[j]);
+      const int c = 16 * b + c0;
+      const double2 v = c == j ? make_double2(1.0, 0.0) : m[b];
+      for (unsigned q = 0; q < PF_C; ++q)
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(
+                         remote_smem(&row_s[j & 1][c], q)),
+                     "d"(v.x), "d"(v.y)
+                     : "memory");
+      if (c == j) {
+        const double p = m[b].x, rd = p > 0.0 ? rsqrt(p) : 0.0;  // 0 for NaN too
+        for (unsigned q = 0; q < PF_C; ++q)
+          asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote_smem(&rd_s[j], q)), "d"(rd)
+                       : "memory");
       }
     }
   };
+  cluster_sync();  // every CTA has started
   publish(0);
-  __syncthreads();
+  cluster_sync();
   for (int j = 0; j < kb; ++j) {
-    if (!ok_s[j]) {
-      if (t == 0) *info = (int)(k0 + j + 1);
+    const double rd = rd_s[j];
+    if (rd == 0.0) {  // the same in every CTA
+      if (rank == 0 && t == 0) *info = (int)(k0 + j + 1);
       return;
     }
-    const double ip = rd_s[j] * rd_s[j];
-    const double2* w = row_s[j & 1];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int r = 16 * a + rl;
-      if (r <= j) continue;
-      const double2 f = cscale(-ip, conjz(w[r]));
+    if (r > j) {
+      const double2* w = row_s[j & 1];
+      const double2 f = cscale(-(rd * rd), conjz(w[r]));
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        const int c = 16 * b + cl;
-        if (c >= r || c <= j) cfma(m[a][b], f, w[c]);
+        const int c = 16 * b + c0;
+        if (c >= r || c <= j) cfma(m[b], f, w[c]);
       }
     }
-    if (j + 1 < kb) publish(j + 1);
-    __syncthreads();
+    if (j + 1 < kb) {
+      publish(j + 1);
+      cluster_sync();
+    }
   }
+  const double rd = r < kb ? rd_s[r] : 0.0;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int r = 16 * a + rl, c = 16 * b + cl;
-      const bool in = r < kb && c < kb;
-      const double rd = r < kb ? rd_s[r] : 0.0;
-      double2 u = make_double2(0.0, 0.0);  // U(r, c)
-      double2 v = make_double2(0.0, 0.0);  // V(r, c) = conj(U^-1(c, r))
-      if (in && r == c) {
-        u.x = sqrt(m[a][b].x);
-        v.x = rd;
-      } else if (in && r < c) {
-        u = cscale(rd, m[a][b]);
-      } else if (in) {
-        v = cscale(rd, m[a][b]);
-      }
-      if (in) G[(k0 + r) + (k0 + c) * ldg] = u;
-      dinv_blk[c + r * NB] = conjz(v);
+  for (int b = 0; b < 4; ++b) {
+    const int c = 16 * b + c0;
+    const bool in = r < kb && c < kb;
+    double2 u = make_double2(0.0, 0.0);  // U(r, c)
+    double2 v = make_double2(0.0, 0.0);  // V(r, c) = conj(U^-1(c, r))
+    if (in && r == c) {
+      u.x = sqrt(m[b].x);
+      v.x = rd;
+    } else if (in && r < c) {
+      u = cscale(rd, m[b]);
+    } else if (in) {
+      v = cscale(rd, m[b]);
     }
+    if (in) G[(k0 + r) + (k0 + c) * ldg] = u;
+    dinv_blk[c + r * NB] = conjz(v);
+  }
 }
 
 // Panel: U(k-block, j) = W^H G(k-block, j), PC columns per CTA (a 64 x 64 block
@@ -423,7 +432,7 @@ cudaError_t potrf_upper(cudaStream_t s, int64_t n, double2* G, int64_t ldg, doub
   if (e != cudaSuccess) return e;
   for (int64_t k0 = 0, b = 0; k0 < n; k0 += NB, ++b) {
     const int kb = (int)std::min<int64_t>(NB, n - k0);
-    potf2_kernel<<<1, FT, 0, s>>>(G, ldg, k0, kb, dinv + b * NB * NB, info); count_launch();
+    potf2_kernel<<<PF_C, FT, 0, s>>>(G, ldg, k0, kb, dinv + b * NB * NB, info); count_launch();
     const int64_t rest = n - k0 - kb;
     if (rest > 0) {
       panel_kernel<<<(unsigned)cdiv(rest, PC), FT, PANEL_SMEM, s>>>(n, G, ldg, k0, kb,
