@@ -205,9 +205,46 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void split2(double x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-  hi = __double2bfloat16(x);
-  lo = __double2bfloat16(x - (double)__bfloat162float(hi));
+// x in FP32, hi = bf16(x) and lo = bf16(x - hi) packed, the FP64 way (a call, so
+// that none of it runs ahead of the branch that needs it)
+__device__ __noinline__ uint2 split_fp64(double x) {
+  const __nv_bfloat16 hi = __double2bfloat16(x);
+  const __nv_bfloat16 lo = __double2bfloat16(x - (double)__bfloat162float(hi));
+  return make_uint2(__float_as_uint((float)x), (unsigned)__bfloat16_as_ushort(hi) |
+                                                   ((unsigned)__bfloat16_as_ushort(lo) << 16));
+}
+// hi, lo and the FP32 rounding of x in FP32 and integer operations (the FP64 pipe
+// and its conversions run at two operations a clock per SM). x is taken apart
+// into its upper 24 bits t, an exact float, and 29 lower ones; a float whose last
+// bit is set whenever something was cut off ("rounded to odd") rounds to BF16 as
+// the exact value does.
+__device__ __forceinline__ void split3(double x, float& f, __nv_bfloat16& hi, __nv_bfloat16& lo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & ~(1ull << 63);
+  const int E = (int)(b >> 52);
+  const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
+  const unsigned tb = b ? (unsigned)((b - (896ull << 52)) >> 29) : 0u;  // |x| truncated
+  const unsigned rest = (unsigned)b & 0x1fffffffu;
+  f = __uint_as_float((tb + (rest + 0x0fffffffu + (tb & 1u) >= 0x20000000u)) | sign);
+  const __nv_bfloat16 h = __float2bfloat16_rn(__uint_as_float(tb | (rest != 0)));
+  const float u = __uint_as_float(tb) - __bfloat162float(h);  // exact
+  // parts that are not all normal in FP32, and a rest that u would cancel to
+  // (once in 2^15 entries): the FP64 way
+  if (b != 0 && (E < 1023 - 70 || E > 1023 + 100 ||
+                 (rest != 0 && fabsf(u) <= __uint_as_float((unsigned)(E - 919) << 23)))) {
+    const uint2 r = split_fp64(x);
+    f = __uint_as_float(r.x);
+    hi = __ushort_as_bfloat16((unsigned short)(r.y & 0xffffu));
+    lo = __ushort_as_bfloat16((unsigned short)(r.y >> 16));
+    return;
+  }
+  const float t2 = (float)((rest >> 5) | ((rest & 31u) != 0)) *
+                   __uint_as_float((unsigned)(E - 943) << 23);  // the rest, odd
+  const float s = __fadd_rz(u, t2);
+  const float l = __uint_as_float(__float_as_uint(s) | ((u - s) + t2 != 0.f ? 1u : 0u));
+  const unsigned flip = sign >> 16;
+  hi = __ushort_as_bfloat16((unsigned short)(__bfloat16_as_ushort(h) ^ flip));
+  const unsigned short lb = __bfloat16_as_ushort(__float2bfloat16_rn(l));
+  lo = __ushort_as_bfloat16((unsigned short)(lb ? lb ^ flip : 0));
 }
 __device__ __forceinline__ void split2f(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
   hi = __float2bfloat16_rn(x);
@@ -470,30 +507,48 @@ __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
 }
 
 // ----------------------------------------------------------- conversions
-// A (column-major complex) -> row-major planes [Ar | Ai], K half padded to Np.
-__global__ void split_a_kernel(int64_t N, int64_t Np, const double2* __restrict__ A, int64_t lda,
-                               __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-  __shared__ double2 tile[32][33];
-  const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
+// A (column-major complex) -> row-major planes [Ar | Ai], K half padded to Np. A
+// warp writes 64 entries of a row, two per lane: 128 bytes of each plane row. The
+// entries are taken apart before they are transposed. N = 4000: 87 us, 5.9 TB/s
+// (250 us with FP64 splits of single entries).
+constexpr int SA_K = 64;
+__device__ __forceinline__ unsigned bf_pair(__nv_bfloat16 a, __nv_bfloat16 b) {
+  return (unsigned)__bfloat16_as_ushort(a) | ((unsigned)__bfloat16_as_ushort(b) << 16);
+}
+__global__ void __launch_bounds__(256)
+    split_a_kernel(int64_t N, int64_t Np, const double2* __restrict__ A, int64_t lda,
+                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+  __shared__ uint2 tile[SA_K][33];  // (hi, lo) of the real part, of the imaginary part
+  const int64_t i0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * SA_K;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t i = i0 + tx, k = k0 + r;
-    tile[r][tx] = (i < N && k < N) ? A[i + k * lda] : make_double2(0.0, 0.0);
+  double2 a[SA_K / 8];
+#pragma unroll
+  for (int r = 0; r < SA_K / 8; ++r) {
+    const int64_t i = i0 + tx, k = k0 + ty + 8 * r;
+    a[r] = (i < N && k < N) ? A[i + k * lda] : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int r = 0; r < SA_K / 8; ++r) {
+    float f;
+    __nv_bfloat16 rh, rl, ih, il;
+    split3(a[r].x, f, rh, rl);
+    split3(a[r].y, f, ih, il);
+    tile[ty + 8 * r][tx] = make_uint2(bf_pair(rh, rl), bf_pair(ih, il));
   }
   __syncthreads();
   const int64_t ld = 2 * Np;
+  const int64_t k = k0 + 2 * tx;  // k + 1 may be N: a zero of the padding
+  if (k >= N) return;
+#pragma unroll
   for (int r = ty; r < 32; r += 8) {
-    const int64_t i = i0 + r, k = k0 + tx;
-    if (i < N && k < N) {
-      const double2 a = tile[tx][r];
-      __nv_bfloat16 h, l;
-      split2(a.x, h, l);
-      hi[i * ld + k] = h;
-      lo[i * ld + k] = l;
-      split2(a.y, h, l);
-      hi[i * ld + Np + k] = h;
-      lo[i * ld + Np + k] = l;
-    }
+    const int64_t i = i0 + r;
+    if (i >= N) continue;
+    const uint2 x = tile[2 * tx][r], y = tile[2 * tx + 1][r];
+    const int64_t o = i * ld + k;
+    *reinterpret_cast<unsigned*>(hi + o) = __byte_perm(x.x, y.x, 0x5410);
+    *reinterpret_cast<unsigned*>(lo + o) = __byte_perm(x.x, y.x, 0x7632);
+    *reinterpret_cast<unsigned*>(hi + o + Np) = __byte_perm(x.y, y.y, 0x5410);
+    *reinterpret_cast<unsigned*>(lo + o + Np) = __byte_perm(x.y, y.y, 0x7632);
   }
 }
 
@@ -502,24 +557,31 @@ __global__ void split_a_kernel(int64_t N, int64_t Np, const double2* __restrict_
 __global__ void split_y_kernel(int64_t N, int64_t Np, int64_t j0, const double2* __restrict__ Y,
                                int64_t ldy, __nv_bfloat16* __restrict__ hi,
                                __nv_bfloat16* __restrict__ lo, float2* __restrict__ S) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t j = j0 + blockIdx.y;
   if (k >= N) return;
-  const double2 y = Y[k + j * ldy];
-  S[k + j * N] = make_float2((float)y.x, (float)y.y);
-  __nv_bfloat16 rh, rl, ih, il, nh, nl;
-  split2(y.x, rh, rl);
-  split2(y.y, ih, il);
-  split2(-y.y, nh, nl);
-  const int64_t br = brow_re(j), bi = br + 128, ld = 2 * Np;
-  hi[br * ld + k] = rh;
-  lo[br * ld + k] = rl;
-  hi[br * ld + Np + k] = nh;
-  lo[br * ld + Np + k] = nl;
-  hi[bi * ld + k] = ih;
-  lo[bi * ld + k] = il;
-  hi[bi * ld + Np + k] = rh;
-  lo[bi * ld + Np + k] = rl;
+  const bool two = k + 1 < N;
+  const double2 a = Y[k + j * ldy], b = two ? Y[k + 1 + j * ldy] : make_double2(0.0, 0.0);
+  float2 fa, fb;
+  __nv_bfloat16 arh, arl, aih, ail, brh, brl, bih, bil;
+  split3(a.x, fa.x, arh, arl);
+  split3(a.y, fa.y, aih, ail);
+  split3(b.x, fb.x, brh, brl);
+  split3(b.y, fb.y, bih, bil);
+  S[k + j * N] = fa;
+  if (two) S[k + 1 + j * N] = fb;
+  const int64_t ld = 2 * Np, re = brow_re(j) * ld + k, im = re + 128 * ld;
+  auto put = [](__nv_bfloat16* p, unsigned v) { *reinterpret_cast<unsigned*>(p) = v; };
+  const unsigned rh = bf_pair(arh, brh), rl = bf_pair(arl, brl);
+  const unsigned ih = bf_pair(aih, bih), il = bf_pair(ail, bil);
+  put(hi + re, rh);
+  put(lo + re, rl);
+  put(hi + re + Np, ih ^ 0x80008000u);
+  put(lo + re + Np, il ^ 0x80008000u);
+  put(hi + im, ih);
+  put(lo + im, il);
+  put(hi + im + Np, rh);
+  put(lo + im + Np, rl);
 }
 
 // FP32 state -> FP64 columns of V.
@@ -621,10 +683,10 @@ namespace {
 void mixed_prologue(cudaStream_t s, int64_t N, const double2* A, int64_t lda, const double2* V,
                     int64_t ldv, int64_t ncols, MixedWork& w) {
   const int64_t Np = cdiv(N, KPAD) * KPAD;
-  split_a_kernel<<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, 32), 1), dim3(32, 8, 1), 0, s>>>(
+  split_a_kernel<<<dim3((unsigned)cdiv(N, SA_K), (unsigned)cdiv(N, 32), 1), dim3(32, 8, 1), 0, s>>>(
       N, Np, A, lda, static_cast<__nv_bfloat16*>(w.Ahi), static_cast<__nv_bfloat16*>(w.Alo));
   count_launch();
-  split_y_kernel<<<dim3((unsigned)cdiv(N, 256), (unsigned)ncols, 1), 256, 0, s>>>(
+  split_y_kernel<<<dim3((unsigned)cdiv(N, 512), (unsigned)ncols, 1), 256, 0, s>>>(
       N, Np, 0, V, ldv, static_cast<__nv_bfloat16*>(w.Yhi), static_cast<__nv_bfloat16*>(w.Ylo),
       static_cast<float2*>(w.S32));
   count_launch();
