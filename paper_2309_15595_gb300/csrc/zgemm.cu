@@ -350,16 +350,18 @@ cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2
   const int64_t tiles = hermitian ? tm * (tm + 1) / 2 : tm * tn;
   // split-K factor: the one (up to the workspace and K / 64) for which the most
   // loaded SM has the fewest k steps, a tile counting 16 more for its start and
-  // its partial (a 96 x 64 Gram over 2048 rows is 24 tiles: split 25 ways it
-  // takes 0.1 ms, in 4 pieces 0.9 ms); ties to fewer splits
+  // its partial. A tile has two warps, so one CTA on an SM drives half of its FP64
+  // pipe and shows all its latencies: fewer than three CTAs an SM count more (a
+  // 64 x 64 Gram over 2048 rows, 16 tiles: split 9 ways 142 us); ties to fewer splits
   const int64_t sms = num_sms();
   const int64_t smax = std::max<int64_t>(
       1, std::min<int64_t>(K / 64, (int64_t)(ws_elems / ((size_t)m * n))));
   int64_t splits = 1;
-  int64_t best = -1;
+  double best = 0.0;
   for (int64_t sp = 1; sp <= smax && tiles * (sp - 1) < 8 * sms; ++sp) {
-    const int64_t load = cdiv(tiles * sp, sms) * (cdiv(K, sp) + 16);
-    if (best < 0 || load < best) {
+    const int64_t r = cdiv(tiles * sp, sms);
+    const double load = (double)(r * (cdiv(K, sp) + 16)) * (r >= 3 ? 1.0 : r == 2 ? 1.2 : 2.2);
+    if (sp == 1 || load < best) {
       best = load;
       splits = sp;
     }
