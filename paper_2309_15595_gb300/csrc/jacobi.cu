@@ -633,7 +633,6 @@ constexpr int BJ_B = 32;          // block width
 constexpr int BJ_M = 2 * BJ_B;    // order of a block pair
 constexpr int BJ_T = 256;
 constexpr int BJ_ROWS = 64;       // rows (or columns) of G per CTA in the update kernels
-constexpr int BJ_UPD_SMEM = (BJ_M * (BJ_M + 1) + BJ_ROWS * (BJ_M + 1)) * (int)sizeof(float2);
 
 __device__ __forceinline__ void bj_pair(int64_t n, int nb, int nbp, int round, int k, int64_t& i0,
                                         int& ni, int64_t& j0, int& nj) {
@@ -659,11 +658,50 @@ constexpr int BJ_P = BJ_M / 2;       // rotations of a round
 constexpr int BJ_LD = BJ_M + 1;
 constexpr int BJ_INNER_SMEM = 2 * BJ_M * BJ_LD * (int)sizeof(float2);
 
-// J = [[c, u], [-conj(u), c]] with u = s phi
+// J = [[c, u], [-conj(u), c]] with u = s phi for the pair p < q; pq = p | q << 8,
+// and bit 16 where the rotation is not the identity
 struct Jrot {
   float c, ux, uy;
-  int on;
+  int pq;
 };
+// The rotation of make_rot_t for a sweep, with approximate square roots and
+// quotients (two units in the last place) and a Newton step on c and on 1 / |b|,
+// so that J is unitary to FP32 rounding: this chain is a third of a round's
+// latency, and the annihilated entry need only be small beside the FP32 rounding
+// of the others.
+__device__ __forceinline__ Jrot fast_rot(float a, float d, float2 b, float& app, float& aqq) {
+  Jrot r;
+  float bb = fmaf(b.x, b.x, b.y * b.y), back = 1.f;
+  if (bb < 1e-30f) {  // squares near FP32's smallest: the rotation of 2^50 times the block
+    a *= 0x1p50f;
+    d *= 0x1p50f;
+    b.x *= 0x1p50f;
+    b.y *= 0x1p50f;
+    bb = fmaf(b.x, b.x, b.y * b.y);
+    back = 0x1p-50f;
+  }
+  if (!(bb > 1e-30f) || bb <= Cx<float>::eps * Cx<float>::eps * fabsf(a) * fabsf(d)) {
+    r.c = 1.f; r.ux = 0.f; r.uy = 0.f; r.pq = 0; app = a * back; aqq = d * back;
+    return r;
+  }
+  float ri = rsqrtf(bb);
+  ri = ri * fmaf(-0.5f * bb, ri * ri, 1.5f);
+  const float ab = bb * ri, tau = 0.5f * (d - a) * ri, at = fabsf(tau);
+  const float q = fmaf(tau, tau, 1.f);
+  const float t = copysignf(at > 1e15f ? __fdividef(0.5f, at) : __fdividef(1.f, at + q * rsqrtf(q)),
+                            tau);
+  const float w = fmaf(t, t, 1.f);
+  float c = rsqrtf(w);
+  c = c * fmaf(-0.5f * w, c * c, 1.5f);
+  const float sr = t * c * ri;
+  r.c = c;
+  r.ux = sr * b.x;
+  r.uy = sr * b.y;
+  r.pq = 1 << 16;
+  app = fmaf(-t, ab, a) * back;
+  aqq = fmaf(t, ab, d) * back;
+  return r;
+}
 
 // One cyclic sweep on S (64 x 64, Hermitian, ld BJ_LD in shared memory; a
 // smaller matrix is padded with zeros, which no rotation touches), its rotations
@@ -673,8 +711,9 @@ struct Jrot {
 // two), its mirror image is written and not computed, the pairs' own blocks are
 // set exactly by the threads that compute the rotations. Warp w takes the blocks
 // of pair w and of pair 31 - w, together one per lane, and rows w, w + 16, .. of
-// R, a lane per pair.
-__device__ __forceinline__ void bj_sweep(float2* S, float2* R, Jrot* rots, int2* pq) {
+// R, a lane per pair. Bound by the 128 bytes a cycle of shared memory (8 KB of R and
+// S's blocks a round, read and written).
+__device__ __forceinline__ void bj_sweep(float2* S, float2* R, Jrot* rots) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   static_assert(BJ_P == 32 && BJ_IT / 32 == BJ_P / 2, "one pair per lane, two per warp");
   // the off-diagonal block of this lane: pairs k < l
@@ -685,29 +724,25 @@ __device__ __forceinline__ void bj_sweep(float2* S, float2* R, Jrot* rots, int2*
     if (t < BJ_P) {
       int p, q;
       rr_pair(BJ_M, rd, t, p, q);
-      const RotT<float> r =
-          make_rot_t<float>(S[p * BJ_LD + p].x, S[q * BJ_LD + q].x, S[p * BJ_LD + q]);
-      Jrot j;
-      j.c = r.c;
-      j.ux = r.s * r.px;
-      j.uy = r.s * r.py;
-      j.on = r.s != 0.f;
-      rots[t] = j;
-      pq[t] = make_int2(p, q);
-      if (j.on) {  // the rotated 2 x 2 block exactly (no other thread reads it)
-        S[p * BJ_LD + p] = make_float2(r.app, 0.f);
-        S[q * BJ_LD + q] = make_float2(r.aqq, 0.f);
+      float app, aqq;
+      Jrot r = fast_rot(S[p * BJ_LD + p].x, S[q * BJ_LD + q].x, S[p * BJ_LD + q], app, aqq);
+      if (r.pq) {  // the rotated 2 x 2 block exactly (no other thread reads it)
+        S[p * BJ_LD + p] = make_float2(app, 0.f);
+        S[q * BJ_LD + q] = make_float2(aqq, 0.f);
         S[p * BJ_LD + q] = make_float2(0.f, 0.f);
         S[q * BJ_LD + p] = make_float2(0.f, 0.f);
       }
+      r.pq |= p | q << 8;
+      rots[t] = r;
     }
     __syncthreads();
     const Jrot jm = rots[lane];
-    const int2 pm = pq[lane];
+    const int2 pm = make_int2(jm.pq & 255, (jm.pq >> 8) & 255);
     if (k != l) {  // B <- J_k^H B J_l
       const Jrot jk = rots[k], jl = rots[l];
-      if (jk.on | jl.on) {
-        const int2 pk = pq[k], pl = pq[l];
+      if ((jk.pq | jl.pq) >> 16) {
+        const int2 pk = make_int2(jk.pq & 255, (jk.pq >> 8) & 255);
+        const int2 pl = make_int2(jl.pq & 255, (jl.pq >> 8) & 255);
         float2 b00 = S[pk.x * BJ_LD + pl.x], b01 = S[pk.x * BJ_LD + pl.y];
         float2 b10 = S[pk.y * BJ_LD + pl.x], b11 = S[pk.y * BJ_LD + pl.y];
         auto cols = [](float2& x, float2& y, const Jrot& j) {
@@ -738,7 +773,7 @@ __device__ __forceinline__ void bj_sweep(float2* S, float2* R, Jrot* rots, int2*
         S[pl.y * BJ_LD + pk.y] = make_float2(b11.x, -b11.y);
       }
     }
-    if (jm.on) {
+    if (jm.pq >> 16) {
 #pragma unroll
       for (int h = 0; h < BJ_M / (BJ_IT / 32); ++h) {
         float2* row = R + (warp + h * (BJ_IT / 32)) * BJ_LD;
@@ -760,7 +795,6 @@ __global__ void __launch_bounds__(BJ_IT)
   float2* S = bj_smem;
   float2* R = bj_smem + BJ_M * BJ_LD;
   __shared__ Jrot rots[BJ_P];
-  __shared__ int2 pq[BJ_P];  // a round's index pairs
   const int t = threadIdx.x;
   int64_t i0, j0;
   int ni, nj;
@@ -773,7 +807,7 @@ __global__ void __launch_bounds__(BJ_IT)
                            : make_float2(0.f, 0.f);
     R[a * BJ_LD + c] = make_float2(a == c ? 1.f : 0.f, 0.f);
   }
-  bj_sweep(S, R, rots, pq);
+  bj_sweep(S, R, rots);
   float2* Rk = Rbuf + (int64_t)blockIdx.x * BJ_M * BJ_M;
   for (int e = t; e < m * m; e += BJ_IT)
     Rk[(e % m) + (e / m) * BJ_M] = R[(e % m) * BJ_LD + e / m];
@@ -791,7 +825,6 @@ __global__ void __launch_bounds__(BJ_IT)
   float2* S = bj_smem;
   float2* R = bj_smem + BJ_M * BJ_LD;
   __shared__ Jrot rots[BJ_P];
-  __shared__ int2 pq[BJ_P];
   __shared__ float red[BJ_IT / 32][2];
   __shared__ int s_exp;  // largest exponent field
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -847,7 +880,7 @@ __global__ void __launch_bounds__(BJ_IT)
     if (off == 0.0 || off <= tol_conv * fro || (off <= tol_stag * fro && off > 0.25 * off_prev))
       break;
     off_prev = off;
-    if (sw < max_sweeps) bj_sweep(S, R, rots, pq);
+    if (sw < max_sweeps) bj_sweep(S, R, rots);
   }
   for (int e = t; e < n * n; e += BJ_IT) {
     const float2 r = R[(e % n) * BJ_LD + e / n];
@@ -855,103 +888,34 @@ __global__ void __launch_bounds__(BJ_IT)
   }
 }
 
-// Columns of the pair: M(r0:r0+64, idx) <- M(r0:r0+64, idx) R for M = G and Z.
-__global__ void __launch_bounds__(BJ_T)
-    bj_cols_kernel(int64_t n, int nb, int nbp, int round, float2* __restrict__ G,
-                   float2* __restrict__ Z, const float2* __restrict__ Rbuf) {
-  extern __shared__ float2 bj_smem[];
-  float2* R = bj_smem;                      // [BJ_M][BJ_M + 1]
-  float2* T = bj_smem + BJ_M * (BJ_M + 1);  // [BJ_ROWS][BJ_M + 1]
-  const int k = blockIdx.y, t = threadIdx.x;
-  int64_t i0, j0;
-  int ni, nj;
-  bj_pair(n, nb, nbp, round, k, i0, ni, j0, nj);
-  const int m = ni + nj;
-  if (m == 0) return;
-  const float2* Rk = Rbuf + (int64_t)k * BJ_M * BJ_M;
-  for (int e = t; e < m * m; e += BJ_T) R[(e % m) * (BJ_M + 1) + e / m] = Rk[(e % m) + (e / m) * BJ_M];
-  const int64_t r0 = (int64_t)blockIdx.x * BJ_ROWS;
-  const int tx = t & 15, ty = t >> 4;  // columns tx + 16 c, rows ty + 16 r
-  for (int mat = 0; mat < 2; ++mat) {
-    float2* M = mat == 0 ? G : Z;
-    __syncthreads();
-    for (int e = t; e < BJ_ROWS * m; e += BJ_T) {
-      const int i = e % BJ_ROWS, a = e / BJ_ROWS;
-      const int64_t row = r0 + i;
-      T[i * (BJ_M + 1) + a] =
-          row < n ? M[row + bj_gidx(a, i0, ni, j0) * n] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    float2 o[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) o[r][c] = make_float2(0.f, 0.f);
-    for (int a = 0; a < m; ++a) {
-      float2 x[4], y[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) x[r] = T[(ty + 16 * r) * (BJ_M + 1) + a];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) y[c] = R[a * (BJ_M + 1) + tx + 16 * c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          o[r][c].x = fmaf(x[r].x, y[c].x, fmaf(-x[r].y, y[c].y, o[r][c].x));
-          o[r][c].y = fmaf(x[r].x, y[c].y, fmaf(x[r].y, y[c].x, o[r][c].y));
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int64_t row = r0 + ty + 16 * r;
-      if (row >= n) continue;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int cc = tx + 16 * c;
-        if (cc < m) M[row + bj_gidx(cc, i0, ni, j0) * n] = o[r][c];
-      }
-    }
-  }
-}
+// After a round's inner sweeps: G <- R^H G R and Z <- Z R with the block-diagonal R
+// of all pairs, 64 x 64 tiles, one CTA each, one launch. The tile of G where pairs
+// k <= l meet is multiplied from both sides and written with its conjugate
+// transpose (half the tiles, and G stays Hermitian); tiles of Z take one product.
+// Bound by FP32 FMAs and the shared-memory reads that feed them. n = 1072: separate
+// column and row passes over all of G took 73 us a round.
+constexpr int BJ_TILE = BJ_M * BJ_LD;
+constexpr int BJ_UPD_SMEM = 3 * BJ_TILE * (int)sizeof(float2);
 
-// Rows of the pair: G(idx, c0:c0+64) <- R^H G(idx, c0:c0+64).
-__global__ void __launch_bounds__(BJ_T)
-    bj_rows_kernel(int64_t n, int nb, int nbp, int round, float2* __restrict__ G,
-                   const float2* __restrict__ Rbuf) {
-  extern __shared__ float2 bj_smem[];
-  float2* R = bj_smem;                      // [BJ_M][BJ_M + 1]
-  float2* T = bj_smem + BJ_M * (BJ_M + 1);  // [BJ_M][BJ_ROWS + 1] (rows of the pair x columns)
-  const int k = blockIdx.y, t = threadIdx.x;
-  int64_t i0, j0;
-  int ni, nj;
-  bj_pair(n, nb, nbp, round, k, i0, ni, j0, nj);
-  const int m = ni + nj;
-  if (m == 0) return;
-  const float2* Rk = Rbuf + (int64_t)k * BJ_M * BJ_M;
-  for (int e = t; e < m * m; e += BJ_T) R[(e % m) * (BJ_M + 1) + e / m] = Rk[(e % m) + (e / m) * BJ_M];
-  const int64_t c0 = (int64_t)blockIdx.x * BJ_ROWS;
-  for (int e = t; e < m * BJ_ROWS; e += BJ_T) {
-    const int a = e % m, j = e / m;
-    const int64_t col = c0 + j;
-    T[a * (BJ_ROWS + 1) + j] = col < n ? G[bj_gidx(a, i0, ni, j0) + col * n] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  const int tx = t & 15, ty = t >> 4;  // columns tx + 16 c, pair rows ty + 16 r
-  float2 o[4][4];
+// o(r, c) = sum_a X(r, a) Y(a, c) for rows tx + 16 r and columns ty + 16 c; X is T
+// row-major, or conj(R)^T for CONJT
+template <bool CONJT>
+__device__ __forceinline__ void bj_product(const float2* X, const float2* Y, int tx, int ty,
+                                           float2 (&o)[4][4]) {
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 4; ++c) o[r][c] = make_float2(0.f, 0.f);
-  for (int b = 0; b < m; ++b) {
+#pragma unroll 4
+  for (int a = 0; a < BJ_M; ++a) {
     float2 x[4], y[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int a = ty + 16 * r;  // (R^H)(a, b) = conj(R(b, a))
-      const float2 rv = a < m ? R[b * (BJ_M + 1) + a] : make_float2(0.f, 0.f);
-      x[r] = make_float2(rv.x, -rv.y);
+      x[r] = CONJT ? X[a * BJ_LD + tx + 16 * r] : X[(tx + 16 * r) * BJ_LD + a];
+      if (CONJT) x[r].y = -x[r].y;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) y[c] = T[b * (BJ_ROWS + 1) + tx + 16 * c];
+    for (int c = 0; c < 4; ++c) y[c] = Y[a * BJ_LD + ty + 16 * c];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -960,20 +924,92 @@ __global__ void __launch_bounds__(BJ_T)
         o[r][c].y = fmaf(x[r].x, y[c].y, fmaf(x[r].y, y[c].x, o[r][c].y));
       }
   }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int a = ty + 16 * r;
-    if (a >= m) continue;
+}
+// R of a pair (order m, column-major, ld 64) row-major into shared memory, zero padded
+__device__ __forceinline__ void bj_load_r(float2* R, const float2* __restrict__ src, int m) {
+  for (int e = threadIdx.x; e < BJ_M * BJ_M; e += BJ_T) {
+    const int a = e % BJ_M, c = e / BJ_M;
+    R[a * BJ_LD + c] = (a < m && c < m) ? src[a + c * BJ_M] : make_float2(0.f, 0.f);
+  }
+}
+
+__global__ void __launch_bounds__(BJ_T)
+    bj_update_kernel(int64_t n, int nb, int nbp, int round, int ng, float2* __restrict__ G,
+                     float2* __restrict__ Z, const float2* __restrict__ Rbuf) {
+  extern __shared__ float2 bj_smem[];
+  float2* T = bj_smem;
+  float2* Rl = bj_smem + BJ_TILE;
+  float2* Rk = bj_smem + 2 * BJ_TILE;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4, npair = nbp / 2;
+  const bool in_g = (int)blockIdx.x < ng;
+  int k = 0, l;
+  int64_t r0 = 0;
+  if (in_g) {  // tile number l (l + 1) / 2 + k
+    l = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while (l * (l + 1) / 2 > (int)blockIdx.x) --l;
+    while ((l + 1) * (l + 2) / 2 <= (int)blockIdx.x) ++l;
+    k = (int)blockIdx.x - l * (l + 1) / 2;
+  } else {
+    l = ((int)blockIdx.x - ng) % npair;
+    r0 = (int64_t)(((int)blockIdx.x - ng) / npair) * BJ_ROWS;
+  }
+  int64_t li0, lj0, ki0 = 0, kj0 = 0;
+  int lni, lnj, kni = 0, knj = 0;
+  bj_pair(n, nb, nbp, round, l, li0, lni, lj0, lnj);
+  const int ml = lni + lnj;
+  int mk = 0;
+  if (in_g) {
+    bj_pair(n, nb, nbp, round, k, ki0, kni, kj0, knj);
+    mk = kni + knj;
+  } else {
+    mk = (int)min((int64_t)BJ_ROWS, n - r0);
+  }
+  if (ml == 0 || mk <= 0) return;
+  float2* M = in_g ? G : Z;
+  auto row = [&](int a) { return in_g ? bj_gidx(a, ki0, kni, kj0) : r0 + a; };
+  bj_load_r(Rl, Rbuf + (int64_t)l * BJ_M * BJ_M, ml);
+  if (in_g) bj_load_r(Rk, Rbuf + (int64_t)k * BJ_M * BJ_M, mk);
+  for (int e = t; e < BJ_M * BJ_M; e += BJ_T) {
+    const int a = e % BJ_M, c = e / BJ_M;
+    T[a * BJ_LD + c] = (a < mk && c < ml) ? M[row(a) + bj_gidx(c, li0, lni, lj0) * n]
+                                          : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  float2 o[4][4];
+  bj_product<false>(T, Rl, tx, ty, o);
+  if (!in_g) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const int64_t col = c0 + tx + 16 * c;
-      if (col < n) G[bj_gidx(a, i0, ni, j0) + col * n] = o[r][c];
+      const int cc = ty + 16 * c;
+      if (cc >= ml) continue;
+      const int64_t col = bj_gidx(cc, li0, lni, lj0);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (tx + 16 * r < mk) M[r0 + tx + 16 * r + col * n] = o[r][c];
+    }
+    return;
+  }
+  auto keep = [&]() {
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) T[(tx + 16 * r) * BJ_LD + ty + 16 * c] = o[r][c];
+    __syncthreads();
+  };
+  keep();
+  bj_product<true>(Rk, T, tx, ty, o);
+  keep();
+  for (int e = t; e < BJ_M * BJ_M; e += BJ_T) {
+    const int a = e % BJ_M, c = e / BJ_M;
+    if (a < mk && c < ml) G[row(a) + bj_gidx(c, li0, lni, lj0) * n] = T[a * BJ_LD + c];
+    if (k != l && a < ml && c < mk) {  // the mirror image
+      const float2 v = T[c * BJ_LD + a];
+      G[bj_gidx(a, li0, lni, lj0) + row(c) * n] = make_float2(v.x, -v.y);
     }
   }
 }
 
-// Off-diagonal and total squared Frobenius norms of G (n x n, FP32): one
-// partial pair per block, summed on the host in a fixed order.
 __global__ void bj_norms_kernel(int64_t n, const float2* __restrict__ G, double* __restrict__ part) {
   __shared__ double so[256], sf[256];
   double o = 0.0, f = 0.0;
@@ -1007,8 +1043,8 @@ void set_bj_attrs() {
                          BJ_INNER_SMEM);
     cudaFuncSetAttribute(jacobi32_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          BJ_INNER_SMEM);
-    cudaFuncSetAttribute(bj_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
-    cudaFuncSetAttribute(bj_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BJ_UPD_SMEM);
+    cudaFuncSetAttribute(bj_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         BJ_UPD_SMEM);
   });
 }
 
@@ -1024,6 +1060,7 @@ int run_block_jacobi32(cudaStream_t s, int64_t n, float2* G, float2* Z, float2* 
   const int nbp = nb + (nb & 1);
   const int npair = nbp / 2;
   const unsigned gt = (unsigned)cdiv(n, BJ_ROWS);
+  const int ng = npair * (npair + 1) / 2;  // tiles of G on and above the diagonal
   constexpr int kNormBlocks = 256;
   double off_prev = 1e300;
   *conv = false;
@@ -1049,11 +1086,8 @@ int run_block_jacobi32(cudaStream_t s, int64_t n, float2* G, float2* Z, float2* 
     if (sw == max_sweeps) break;
     for (int rd = 0; rd < nbp - 1; ++rd) {
       bj_inner_kernel<<<npair, BJ_IT, BJ_INNER_SMEM, s>>>(n, nb, nbp, rd, G, Rbuf);
-      bj_cols_kernel<<<dim3(gt, (unsigned)npair, 1), BJ_T, BJ_UPD_SMEM, s>>>(n, nb, nbp, rd, G, Z,
-                                                                          Rbuf);
-      bj_rows_kernel<<<dim3(gt, (unsigned)npair, 1), BJ_T, BJ_UPD_SMEM, s>>>(n, nb, nbp, rd, G,
-                                                                          Rbuf);
-      count_launch();
+      bj_update_kernel<<<(unsigned)(ng + npair * (int)gt), BJ_T, BJ_UPD_SMEM, s>>>(n, nb, nbp, rd,
+                                                                                ng, G, Z, Rbuf);
       count_launch();
       count_launch();
     }
