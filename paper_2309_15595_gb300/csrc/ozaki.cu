@@ -61,6 +61,7 @@ namespace {
 
 constexpr int OS = 6;                    // digits per operand
 static_assert(OS == 6, "the epilogue keeps levels 2-5 exact and levels 6-7 in FP32");
+constexpr int OS7 = 7;                   // digits of the fine product
 constexpr int TM = 128, TN = 64, TK = 32, STAGES = 3;
 constexpr int CHUNK_KB = 8;              // K blocks per exact chunk (256 values)
 // a chunk's sum of level L is an integer of at most (L - 1) 2^22, so level 2 may
@@ -69,6 +70,10 @@ constexpr int kDrain2 = 4, kDrain3 = 2;
 constexpr int A_TILE = TM * TK * 2;      // 8 KB per digit
 constexpr int B_TILE = TN * TK * 2;      // 4 KB per digit
 constexpr int STAGE_BYTES = OS * (A_TILE + B_TILE);  // 72 KB
+// ring: three stages of six digits or two of seven
+constexpr int stages(int ns) { return ns == OS ? STAGES : 2; }
+constexpr int stage_bytes(int ns) { return ns * (A_TILE + B_TILE); }
+static_assert(stages(OS7) * stage_bytes(OS7) <= STAGES * STAGE_BYTES, "one shared-memory size");
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr int NTHREADS = 320;
 constexpr uint32_t TMEM_COLS = 512;
@@ -173,7 +178,7 @@ template <> struct Slots<8> {
 // atoms). 36 filter steps with N = 9273 and up to 316 columns: 132 ms with 21
 // MMAs of N = 64 and every level drained per chunk, 99 ms so.
 // r2, r3, r: this step restarts levels 2, 3 and the others.
-template <int LMAX>
+template <int LMAX, int NS>
 __device__ __forceinline__ void digit_pairs(uint32_t tmem, uint32_t sa, uint32_t sb, bool r2,
                                             bool r3, bool r) {
   using S = Slots<LMAX>;
@@ -203,7 +208,7 @@ __device__ __forceinline__ void digit_pairs(uint32_t tmem, uint32_t sa, uint32_t
   one(S::L7b, 6, 1, r);
   if constexpr (LMAX == 8) {
 #pragma unroll
-    for (int s = 2; s <= 6; ++s) one(S::L8, s, 8 - s, r && s == 2);
+    for (int s = 8 - NS; s <= NS; ++s) one(S::L8, s, 8 - s, r && s == 8 - NS);
   }
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -340,7 +345,7 @@ __device__ __forceinline__ long long low_fixed(float v) { return __float2ll_rn(v
 // and then adds up and finishes 1 / split of the tile's columns. clustered: the
 // launch has clusters of more than one CTA, all of which meet at the two cluster
 // barriers; CTAs past the last tile (padding of a group's problem) only do that.
-template <int LMAX>
+template <int LMAX, int NS>
 __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtensorMap* tmB,
                                            const Params& P, unsigned local, bool maps_in_global,
                                            bool clustered) {
@@ -352,11 +357,12 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   }
   unsigned rb, ct;  // row block and column tile (grouped raster order)
   grouped_tile(local / (unsigned)P.split, (unsigned)P.nrow, (unsigned)P.ncol, kGroup, rb, ct);
+  constexpr int kStages = stages(NS), kStage = stage_bytes(NS);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
   // [0,S) full, [S,2S) empty, [2S] accumulators full, [2S+1] accumulators empty
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 2);
   __shared__ int s_abort;
 
   // the epilogue's sums, in the ring once that is free: [2 HC][kEpiThreads]
@@ -374,12 +380,12 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
 
   if (threadIdx.x == 0) {
     s_abort = 0;
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&bars[s]), 1);
-      mbar_init(smem_u32(&bars[STAGES + s]), 1);
+      mbar_init(smem_u32(&bars[kStages + s]), 1);
     }
-    mbar_init(smem_u32(&bars[2 * STAGES]), 1);
-    mbar_init(smem_u32(&bars[2 * STAGES + 1]), 8);
+    mbar_init(smem_u32(&bars[2 * kStages]), 1);
+    mbar_init(smem_u32(&bars[2 * kStages + 1]), 8);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -405,66 +411,66 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
       }
       int issued = 0;
       for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-        if (!mbar_wait(smem_u32(&bars[STAGES + s]), ph ^ 1u, P.err, 11)) {
+        const int s = kb % kStages;
+        const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
+        if (!mbar_wait(smem_u32(&bars[kStages + s]), ph ^ 1u, P.err, 11)) {
           s_abort = 1;
           break;
         }
         if (*(volatile int*)&s_abort) break;
         const uint32_t full = smem_u32(&bars[s]);
-        uint8_t* st = smem + s * STAGE_BYTES;
-        mbar_expect_tx(full, STAGE_BYTES);
+        uint8_t* st = smem + s * kStage;
+        mbar_expect_tx(full, kStage);
         const int kx = (chunk0 * CHUNK_KB + kb) * TK;
 #pragma unroll
-        for (int d = 0; d < OS; ++d) {
+        for (int d = 0; d < NS; ++d) {
           // digit planes are stacked along rows: digit d of row r is row d * rows + r
           tma_load_2d(smem_u32(st + d * A_TILE), tmA, kx, (int)(d * P.arows + m0), full);
         }
 #pragma unroll
-        for (int d = 0; d < OS; ++d) {
-          tma_load_2d(smem_u32(st + OS * A_TILE + d * B_TILE), tmB, kx,
+        for (int d = 0; d < NS; ++d) {
+          tma_load_2d(smem_u32(st + NS * A_TILE + d * B_TILE), tmB, kx,
                       (int)(d * P.brows + tile * TN), full);
         }
         ++issued;
       }
-      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-        mbar_wait(smem_u32(&bars[kb % STAGES]), (uint32_t)(kb / STAGES) & 1u, P.err, 12);
+      for (int kb = issued > kStages ? issued - kStages : 0; kb < issued; ++kb)
+        mbar_wait(smem_u32(&bars[kb % kStages]), (uint32_t)(kb / kStages) & 1u, P.err, 12);
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ------------------------------------ MMA issuer
       int kb = 0;
       bool ok = true;
       for (int c = 0; c < nchunks && ok; ++c) {
-        if (c > 0 && !mbar_wait(smem_u32(&bars[2 * STAGES + 1]), (uint32_t)(c - 1) & 1u, P.err, 13)) {
+        if (c > 0 && !mbar_wait(smem_u32(&bars[2 * kStages + 1]), (uint32_t)(c - 1) & 1u, P.err, 13)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int kc = 0; kc < CHUNK_KB; ++kc, ++kb) {
-          const int s = kb % STAGES;
-          const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
+          const int s = kb % kStages;
+          const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
           if (!mbar_wait(smem_u32(&bars[s]), ph, P.err, 14) || *(volatile int*)&s_abort) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t st = smem_u32(smem + s * STAGE_BYTES);
+          const uint32_t st = smem_u32(smem + s * kStage);
 #pragma unroll
           for (int kk = 0; kk < TK / 16; ++kk) {
             const uint32_t off = kk * 32;
             // levels restart often enough to stay exact integers: see kDrain2, kDrain3
             const bool r = kc == 0 && kk == 0;
-            digit_pairs<LMAX>(tmem, st + off, st + OS * A_TILE + off, r && c % kDrain2 == 0,
+            digit_pairs<LMAX, NS>(tmem, st + off, st + NS * A_TILE + off, r && c % kDrain2 == 0,
                               r && c % kDrain3 == 0, r);  // c = 0 restarts all
           }
-          umma_commit(smem_u32(&bars[STAGES + s]));
+          umma_commit(smem_u32(&bars[kStages + s]));
         }
-        umma_commit(smem_u32(&bars[2 * STAGES]));  // chunk c ready
+        umma_commit(smem_u32(&bars[2 * kStages]));  // chunk c ready
       }
       if (!ok) {
         s_abort = 1;
-        umma_commit(smem_u32(&bars[2 * STAGES]));
+        umma_commit(smem_u32(&bars[2 * kStages]));
       }
     }
   } else {
@@ -485,7 +491,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
       acc67[j] = Acc67(0);
     }
     for (int c = 0; c < nchunks; ++c) {
-      const bool ok = mbar_wait(smem_u32(&bars[2 * STAGES]), (uint32_t)c & 1u, P.err, 15);
+      const bool ok = mbar_wait(smem_u32(&bars[2 * kStages]), (uint32_t)c & 1u, P.err, 15);
       go = __all_sync(0xffffffffu, ok && !*(volatile int*)&s_abort);
       if (!go) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -552,7 +558,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars[2 * STAGES + 1]));
+      if (lane == 0) mbar_arrive(smem_u32(&bars[2 * kStages + 1]));
     }
     // the ring is free: every MMA of this CTA has been waited for above
     const int e = (warp - 2) * 32 + lane;
@@ -667,11 +673,11 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   }
 }
 
-template <int LMAX>
+template <int LMAX, int NS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       Params P) {
-  ozaki_tile<LMAX>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
+  ozaki_tile<LMAX, NS>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
 }
 
 // Many problems' filter steps in one launch: entry p of the table holds problem
@@ -696,7 +702,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   const OzGroupEntry* e = tab + lo;
   const Params P = e->P;
-  ozaki_tile<7>(&e->a, &e->b, P, (unsigned)(id - e->first), true, clustered);
+  ozaki_tile<7, OS>(&e->a, &e->b, P, (unsigned)(id - e->first), true, clustered);
 }
 
 // ------------------------------------------------------------ digit prep
@@ -713,29 +719,34 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // through the bit pattern of 2^23 + b. A BF16 digit is the upper half of that
 // float. (With FP64 scaling and one conversion per digit and format, slicing a
 // 20000-row matrix took 8.8 ms, 2.9 of the copy bandwidth's 6.8 TB/s.)
-__device__ __forceinline__ long long fixed48(double x, int e) {  // rint(x 2^(48 - e))
+template <int BITS>
+__device__ __forceinline__ long long fixed(double x, int e) {  // rint(x 2^(BITS - e))
   const long long b = __double_as_longlong(x);
   const int E = (int)(b >> 52) & 0x7ff;
   const long long m = (b & 0xfffffffffffffll) | (E ? 1ll << 52 : 0);
-  const int sh = 1027 - (E ? E : 1) + e;
-  if (E == 0x7ff || sh < 1) return __double2ll_rn(x * ldexp(1.0, -e) * 0x1p48);
+  const int sh = 1075 - BITS - (E ? E : 1) + e;
+  if (E == 0x7ff || sh < 48 - BITS - 2) return __double2ll_rn(ldexp(x * ldexp(1.0, -e), BITS));
   if (sh > 53) return 0;
+  if (sh < 1) return b < 0 ? -(m << -sh) : m << -sh;  // more bits than x has
   const long long X = (m + (1ll << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh;
   return b < 0 ? -X : X;
 }
+template <int NS>
 struct Digits {
-  float d[OS];  // leading digit first
+  float d[NS];  // leading digit first
 };
-__device__ __forceinline__ Digits digits_of(double x, int e) {
-  const unsigned long long X = (unsigned long long)fixed48(x, e) + 0x8080808080ull;
+template <int NS>
+__device__ __forceinline__ Digits<NS> digits_of(double x, int e) {
+  const unsigned long long X = (unsigned long long)fixed<8 * NS>(x, e) +
+                               (NS == OS ? 0x8080808080ull : 0x808080808080ull);
   const unsigned lo = (unsigned)X, hi = (unsigned)(X >> 32);
-  Digits r;
+  Digits<NS> r;
 #pragma unroll
-  for (int s = 0; s < OS - 1; ++s) {  // byte s of X: digit OS - 1 - s
+  for (int s = 0; s < NS - 1; ++s) {  // byte s of X: digit NS - 1 - s
     const unsigned f = __byte_perm(s < 4 ? lo : hi, 0x4b000000u, 0x7440u | (unsigned)(s & 3));
-    r.d[OS - 1 - s] = __uint_as_float(f) - 8388736.0f;  // 2^23 + 128
+    r.d[NS - 1 - s] = __uint_as_float(f) - 8388736.0f;  // 2^23 + 128
   }
-  r.d[0] = (float)((int)hi >> 8);
+  r.d[0] = (float)((int)hi >> (8 * (NS - OS + 1)));
   return r;
 }
 // BF16 of two digits, the first one in the lower half. Digits of finite values
@@ -793,6 +804,7 @@ __global__ void exps_kernel(int64_t n, const unsigned long long* __restrict__ mx
 // [Ar | Ai]), stacked; skip_diag leaves the diagonal out (square A). A warp
 // writes a row of 64 entries, two per lane: 128 bytes of each of its 12 rows.
 constexpr int SA_K = 64;
+template <int NS>
 __global__ void __launch_bounds__(256)
     slice_a_kernel(int64_t M, int64_t K, int64_t Np, bool skip_diag,
                    const double2* __restrict__ A, int64_t lda, const int* __restrict__ ea,
@@ -816,11 +828,11 @@ __global__ void __launch_bounds__(256)
     if (i >= M) continue;
     const double2 a0 = tile[2 * tx][r], a1 = tile[2 * tx + 1][r];
     const int e = ea[i];
-    const Digits r0 = digits_of(a0.x, e), r1 = digits_of(a1.x, e);
-    const Digits c0 = digits_of(a0.y, e), c1 = digits_of(a1.y, e);
+    const Digits<NS> r0 = digits_of<NS>(a0.x, e), r1 = digits_of<NS>(a1.x, e);
+    const Digits<NS> c0 = digits_of<NS>(a0.y, e), c1 = digits_of<NS>(a1.y, e);
     __nv_bfloat16* o = out + i * ld + k;
 #pragma unroll
-    for (int d = 0; d < OS; ++d) {
+    for (int d = 0; d < NS; ++d) {
       *reinterpret_cast<unsigned*>(o + d * plane) = pack_digits(r0.d[d], r1.d[d]);
       *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
     }
@@ -837,8 +849,8 @@ __global__ void round_left_kernel(int64_t M, int64_t K, double2* __restrict__ X,
   const double2 x = X[i + k * ldx];
   const int e = ea[i];
   // exact: 48 bits below the scale
-  X[i + k * ldx] = make_double2(ldexp((double)fixed48(x.x, e), e - 48),
-                                ldexp((double)fixed48(x.y, e), e - 48));
+  X[i + k * ldx] = make_double2(ldexp((double)fixed<48>(x.x, e), e - 48),
+                                ldexp((double)fixed<48>(x.y, e), e - 48));
 }
 
 // Left operand X^H for X (K x M, column-major): row i of X^H is conj(X[:, i]),
@@ -853,8 +865,8 @@ __global__ void slice_ct_kernel(int64_t M, int64_t K, int64_t Np, const double2*
   const double2 x0 = X[k + i * ldx];
   const double2 x1 = k + 1 < K ? X[k + 1 + i * ldx] : make_double2(0.0, 0.0);
   const int e = ea[i];
-  const Digits r0 = digits_of(x0.x, e), r1 = digits_of(x1.x, e);
-  const Digits c0 = digits_of(-x0.y, e), c1 = digits_of(-x1.y, e);
+  const Digits<OS> r0 = digits_of<OS>(x0.x, e), r1 = digits_of<OS>(x1.x, e);
+  const Digits<OS> c0 = digits_of<OS>(-x0.y, e), c1 = digits_of<OS>(-x1.y, e);
   const int64_t ld = 2 * Np;
   const size_t plane = (size_t)M * ld;
   __nv_bfloat16* o = out + i * ld + k;
@@ -897,16 +909,17 @@ __global__ void __launch_bounds__(256)
 
 // Digits of entries k, k + 1 (zero past N) of one column of the right operand
 // into its rows of B^T. Real row: [Yr | -Yi]; imaginary row: [Yi | Yr].
+template <int NS>
 __device__ __forceinline__ void slice_b_pair(int64_t N, int64_t Np, size_t plane, int64_t k,
                                              const double2* __restrict__ Y, int e,
                                              __nv_bfloat16* __restrict__ re,
                                              __nv_bfloat16* __restrict__ im) {
   const double2 y0 = Y[k];
   const double2 y1 = k + 1 < N ? Y[k + 1] : make_double2(0.0, 0.0);
-  const Digits r0 = digits_of(y0.x, e), r1 = digits_of(y1.x, e);
-  const Digits c0 = digits_of(y0.y, e), c1 = digits_of(y1.y, e);
+  const Digits<NS> r0 = digits_of<NS>(y0.x, e), r1 = digits_of<NS>(y1.x, e);
+  const Digits<NS> c0 = digits_of<NS>(y0.y, e), c1 = digits_of<NS>(y1.y, e);
 #pragma unroll
-  for (int d = 0; d < OS; ++d) {
+  for (int d = 0; d < NS; ++d) {
     const unsigned r = pack_digits(r0.d[d], r1.d[d]), c = pack_digits(c0.d[d], c1.d[d]);
     *reinterpret_cast<unsigned*>(re + d * plane + k) = r;
     *reinterpret_cast<unsigned*>(re + d * plane + Np + k) = c ^ 0x80008000u;
@@ -917,6 +930,7 @@ __device__ __forceinline__ void slice_b_pair(int64_t N, int64_t Np, size_t plane
 
 // Y columns -> OS digit planes of B^T (rows: 32-column tiles of 64 rows), stacked
 // with `brows` rows per plane; two entries per thread.
+template <int NS>
 __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
                                const double2* __restrict__ Y, int64_t ldy, const int* __restrict__ eb,
                                __nv_bfloat16* __restrict__ out) {
@@ -924,7 +938,7 @@ __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
   const int64_t j = j0 + blockIdx.y;
   if (k >= N) return;
   const int64_t ld = 2 * Np, br = brow_re(j);
-  slice_b_pair(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], out + br * ld,
+  slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], out + br * ld,
                out + (br + CT) * ld);
 }
 
@@ -957,7 +971,7 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) e.eb[j] = ex;
   const int64_t ld = 2 * e.Np, br = brow_re(j);
   for (int64_t k = 2 * threadIdx.x; k < N; k += 512)
-    slice_b_pair(N, e.Np, (size_t)e.brows * ld, k, Y, ex, e.out + br * ld, e.out + (br + CT) * ld);
+    slice_b_pair<OS>(N, e.Np, (size_t)e.brows * ld, k, Y, ex, e.out + br * ld, e.out + (br + CT) * ld);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 lookup_encoder() {
@@ -1031,11 +1045,14 @@ cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned ctas, int cluster
   count_launch();
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+enum Pairs { PAIRS_21, PAIRS_26, PAIRS_28 };
 cudaError_t launch_product(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b,
-                           const Params& P, bool extended) {
+                           const Params& P, Pairs pairs) {
   const unsigned ctas = (unsigned)P.nrow * (unsigned)P.ncol * (unsigned)P.split;
-  return launch_clusters(extended ? ozaki_gemm_kernel<8> : ozaki_gemm_kernel<7>, ctas, P.split, s,
-                         a, b, P);
+  auto* k = pairs == PAIRS_21   ? ozaki_gemm_kernel<7, OS>
+            : pairs == PAIRS_26 ? ozaki_gemm_kernel<8, OS>
+                                : ozaki_gemm_kernel<8, OS7>;
+  return launch_clusters(k, ctas, P.split, s, a, b, P);
 }
 void set_tiles(Params& P) {
   P.nrow = (int)cdiv(P.N, TM);
@@ -1091,14 +1108,14 @@ cudaError_t ozaki_alloc(OzakiWork& w, int64_t N, int64_t ne) {
   if ((e = cudaMemset(w.Ad, 0, a_elems * 2)) != cudaSuccess) return e;
   if ((e = cudaMemset(w.Bd, 0, b_elems * 2)) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.ea, N * sizeof(int))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&w.eb, ne * sizeof(int))) != cudaSuccess) return e;
+  if ((e = cudaMalloc(&w.eb, std::max(N, ne) * sizeof(int))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.amax, N * sizeof(unsigned long long))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.diag, N * sizeof(double2))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.err, sizeof(int))) != cudaSuccess) return e;
   if ((e = cudaMemset(w.err, 0, sizeof(int))) != cudaSuccess) return e;
   // general left operands of the N x n^2 products: X^H (ne x N) or Q (N x ne)
   const int64_t npe = ozaki_np(ne);
-  w.l_elems = (size_t)OS * std::max((size_t)ne * 2 * w.Np, (size_t)N * 2 * npe);
+  w.l_elems = (size_t)OS7 * std::max((size_t)ne * 2 * w.Np, (size_t)N * 2 * npe);
   if ((e = cudaMalloc(&w.Ld, w.l_elems * 2)) != cudaSuccess) return e;
   if ((e = cudaMemset(w.Ld, 0, w.l_elems * 2)) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.el, std::max(N, ne) * sizeof(int))) != cudaSuccess) return e;
@@ -1109,11 +1126,11 @@ cudaError_t ozaki_alloc(OzakiWork& w, int64_t N, int64_t ne) {
   if (!make_map(&maps->a, w.Ad, (int64_t)OS * N, w.Np, TM) ||
       !make_map(&maps->b, w.Bd, (int64_t)OS * w.brows, w.Np, TN))
     return cudaErrorInvalidValue;
-  if ((e = cudaFuncSetAttribute(ozaki_gemm_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_BYTES)) != cudaSuccess)
-    return e;
-  return cudaFuncSetAttribute(ozaki_gemm_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              SMEM_BYTES);
+  for (auto k : {ozaki_gemm_kernel<7, OS>, ozaki_gemm_kernel<8, OS>, ozaki_gemm_kernel<8, OS7>})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) !=
+        cudaSuccess)
+      return e;
+  return cudaSuccess;
 }
 
 void ozaki_free(OzakiWork& w) {
@@ -1135,7 +1152,7 @@ cudaError_t ozaki_prepare_a(cudaStream_t s, const double2* A, int64_t lda, Ozaki
   count_launch();
   diag_kernel<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(N, A, lda, w.diag);
   count_launch();
-  slice_a_kernel<<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
+  slice_a_kernel<OS><<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
       N, N, w.Np, true, A, lda, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
   count_launch();
   w.A_ready = A;
@@ -1150,62 +1167,59 @@ cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const doub
   // digits of the active columns of B
   colexp_kernel<<<(unsigned)n, 256, 0, s>>>(N, j0, B, ldb, w.eb);
   count_launch();
-  slice_b_kernel<<<dim3((unsigned)cdiv(N, 512), (unsigned)n, 1), 256, 0, s>>>(
+  slice_b_kernel<OS><<<dim3((unsigned)cdiv(N, 512), (unsigned)n, 1), 256, 0, s>>>(
       N, w.Np, w.brows, j0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
   count_launch();
   const Maps* maps = static_cast<const Maps*>(w.maps);
   const Params P = product_params(w, ncols_end, j0, B, ldb, ep);
-  return launch_product(s, maps->a, maps->b, P, false);
+  return launch_product(s, maps->a, maps->b, P, PAIRS_21);
 }
 
-cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const double2* X,
-                               int64_t ldx, bool conj_trans, int64_t ncols, const double2* B,
-                               int64_t ldb, const Epilogue& ep, OzakiWork& w, bool extended) {
-  if (M <= 0 || ncols <= 0 || K <= 0) return cudaSuccess;
-  const int64_t Kp = ozaki_np(K);
-  if (Kp > w.Np || ncols > w.ne || (size_t)OS * M * 2 * Kp > w.l_elems)
-    return cudaErrorInvalidValue;
-  __nv_bfloat16* L = static_cast<__nv_bfloat16*>(w.Ld);
-  // The K padding of the left planes must be zero (the right operand's padding
-  // then only has to be finite, which digits always are). The slicing writes
-  // k < K only, so the planes are cleared whenever their layout changes.
-  cudaError_t e;
-  if (M != w.l_M || K != w.l_K) {
-    if ((e = cudaMemsetAsync(L, 0, (size_t)OS * M * 2 * Kp * 2, s)) != cudaSuccess) return e;
-    w.l_M = M;
-    w.l_K = K;
-  }
-  if (conj_trans) {  // left = X^H, X is K x M
-    colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
-    count_launch();
-    slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(M, K, Kp, X, ldx,
-                                                                                 w.el, L);
-    count_launch();
-  } else {           // left = X, M x K
-    if ((e = cudaMemsetAsync(w.amax, 0, M * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    rowmax_kernel<<<dim3((unsigned)cdiv(M, 256), (unsigned)cdiv(K, 256), 1), 256, 0, s>>>(
-        M, K, false, X, ldx, w.amax);
-    count_launch();
-    exps_kernel<<<(unsigned)cdiv(M, 256), 256, 0, s>>>(M, w.amax, w.el);
-    count_launch();
-    slice_a_kernel<<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
-        M, K, Kp, false, X, ldx, w.el, L);
-    count_launch();
-  }
-  // right operand digits, K rows
+namespace {
+// Digits of the left operand X (M x K) into w.Ld, row exponents into w.el.
+template <int NS>
+cudaError_t slice_left(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
+                       OzakiWork& w) {
+  const cudaError_t e = cudaMemsetAsync(w.amax, 0, M * sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  rowmax_kernel<<<dim3((unsigned)cdiv(M, 256), (unsigned)cdiv(K, 256), 1), 256, 0, s>>>(
+      M, K, false, X, ldx, w.amax);
+  count_launch();
+  exps_kernel<<<(unsigned)cdiv(M, 256), 256, 0, s>>>(M, w.amax, w.el);
+  count_launch();
+  slice_a_kernel<NS><<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, SA_K), 1), dim3(32, 8, 1), 0,
+                       s>>>(M, K, ozaki_np(K), false, X, ldx, w.el,
+                            static_cast<__nv_bfloat16*>(w.Ld));
+  count_launch();
+  return cudaGetLastError();
+}
+// The K padding of the left planes must be zero (the right operand's padding then
+// only has to be finite, which digits always are). The slicing writes k < K only,
+// so the planes are cleared whenever their layout changes.
+cudaError_t clear_left(cudaStream_t s, int64_t M, int64_t K, int ns, OzakiWork& w) {
+  if (M == w.l_M && K == w.l_K && ns == w.l_ns) return cudaSuccess;
+  w.l_M = M;
+  w.l_K = K;
+  w.l_ns = ns;
+  return cudaMemsetAsync(w.Ld, 0, (size_t)ns * M * 2 * ozaki_np(K) * 2, s);
+}
+// Digits of the columns of B (K x ncols) into w.Bd (`brows` rows a plane).
+template <int NS>
+void slice_right(cudaStream_t s, int64_t K, int64_t ncols, const double2* B, int64_t ldb,
+                 int64_t brows, OzakiWork& w) {
   colexp_kernel<<<(unsigned)ncols, 256, 0, s>>>(K, 0, B, ldb, w.eb);
   count_launch();
-  slice_b_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)ncols, 1), 256, 0, s>>>(
-      K, Kp, w.brows, 0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
+  slice_b_kernel<NS><<<dim3((unsigned)cdiv(K, 512), (unsigned)ncols, 1), 256, 0, s>>>(
+      K, ozaki_np(K), brows, 0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
   count_launch();
-  CUtensorMap ma, mb;
-  if (!make_map(&ma, L, (int64_t)OS * M, Kp, TM) ||
-      !make_map(&mb, w.Bd, (int64_t)OS * w.brows, Kp, TN))
-    return cudaErrorInvalidValue;
+}
+// Parameters of a product with the left planes in w.Ld (no diagonal split).
+Params general_params(int64_t M, int64_t K, int64_t ncols, const double2* B, int64_t ldb,
+                      int64_t brows, const Epilogue& ep, OzakiWork& w) {
   Params P;
   P.N = M;
-  P.Np = Kp;
-  P.brows = w.brows;
+  P.Np = ozaki_np(K);
+  P.brows = brows;
   P.arows = M;
   P.j0 = 0;
   P.ncols = ncols;
@@ -1226,7 +1240,70 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
   P.partial = ep.partial;
   P.err = w.err;
   set_tiles(P);
-  return launch_product(s, ma, mb, P, extended);
+  return P;
+}
+}  // namespace
+
+cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const double2* X,
+                               int64_t ldx, bool conj_trans, int64_t ncols, const double2* B,
+                               int64_t ldb, const Epilogue& ep, OzakiWork& w, bool extended) {
+  if (M <= 0 || ncols <= 0 || K <= 0) return cudaSuccess;
+  const int64_t Kp = ozaki_np(K);
+  if (Kp > w.Np || ncols > w.ne || (size_t)OS * M * 2 * Kp > w.l_elems)
+    return cudaErrorInvalidValue;
+  cudaError_t e = clear_left(s, M, K, OS, w);
+  if (e != cudaSuccess) return e;
+  if (conj_trans) {  // left = X^H, X is K x M
+    colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
+    count_launch();
+    slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(
+        M, K, Kp, X, ldx, w.el, static_cast<__nv_bfloat16*>(w.Ld));
+    count_launch();
+  } else if ((e = slice_left<OS>(s, M, K, X, ldx, w)) != cudaSuccess) {  // left = X, M x K
+    return e;
+  }
+  slice_right<OS>(s, K, ncols, B, ldb, w.brows, w);
+  CUtensorMap ma, mb;
+  if (!make_map(&ma, w.Ld, (int64_t)OS * M, Kp, TM) ||
+      !make_map(&mb, w.Bd, (int64_t)OS * w.brows, Kp, TN))
+    return cudaErrorInvalidValue;
+  const Params P = general_params(M, K, ncols, B, ldb, w.brows, ep, w);
+  return launch_product(s, ma, mb, P, extended ? PAIRS_26 : PAIRS_21);
+}
+
+int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M) {
+  const int64_t left = (int64_t)(w.l_elems / ((size_t)OS7 * M * 2)) / KPAD * KPAD;
+  // one column tile of the right operand has to fit too
+  const int64_t right = OS * w.brows * w.Np / (OS7 * TN) / KPAD * KPAD;
+  return std::min(left, right);
+}
+
+cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
+                            int64_t ncols, const double2* B, int64_t ldb, const Epilogue& ep,
+                            OzakiWork& w) {
+  if (M <= 0 || ncols <= 0 || K <= 0) return cudaSuccess;
+  const int64_t Kp = ozaki_np(K);
+  if (M > w.N || Kp > ozaki_fine_inner(w, M)) return cudaErrorInvalidValue;
+  cudaError_t e = clear_left(s, M, K, OS7, w);
+  if (e != cudaSuccess || (e = slice_left<OS7>(s, M, K, X, ldx, w)) != cudaSuccess) return e;
+  // as many columns at a time as the right operand's planes hold, in whole tiles
+  const int64_t fit = OS * w.brows * w.Np / (OS7 * Kp) / TN * CT;
+  const int64_t block = std::min({ncols, fit, std::max(w.N, w.ne)});
+  const int64_t brows = cdiv(block, CT) * TN;
+  CUtensorMap ma, mb;
+  if (!make_map(&ma, w.Ld, (int64_t)OS7 * M, Kp, TM) ||
+      !make_map(&mb, w.Bd, (int64_t)OS7 * brows, Kp, TN))
+    return cudaErrorInvalidValue;
+  for (int64_t c0 = 0; c0 < ncols; c0 += block) {
+    const int64_t nc = std::min(block, ncols - c0);
+    slice_right<OS7>(s, K, nc, B + c0 * ldb, ldb, brows, w);
+    Epilogue ec = ep;
+    if (ec.X) ec.X += c0 * ec.ldx;
+    if (ec.Y) ec.Y += c0 * ec.ldy;
+    const Params P = general_params(M, K, nc, B + c0 * ldb, ldb, brows, ec, w);
+    if ((e = launch_product(s, ma, mb, P, PAIRS_28)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t ozaki_round_left(cudaStream_t s, int64_t M, int64_t K, double2* X, int64_t ldx,

@@ -20,6 +20,7 @@ struct OzakiWork {
   size_t l_elems = 0;
   int* el = nullptr;            // row exponents of the general left operand
   int64_t l_M = 0, l_K = 0;     // layout of the planes in Ld (0: not yet written)
+  int l_ns = 0;
   int64_t N = 0, ne = 0, Np = 0, brows = 0;
 };
 
@@ -43,6 +44,14 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
                                int64_t ldx, bool conj_trans, int64_t ncols, const double2* B,
                                int64_t ldb, const Epilogue& ep, OzakiWork& w,
                                bool extended = false);
+// P = X * B (M x K times K x ncols, any ncols) from seven digits of each operand, 28
+// digit pairs: an error of about sqrt(2K) 2^-57 of the row and column maxima, which
+// is FP64's. ep: EPI_STORE or EPI_FILTER. K at most ozaki_fine_inner, which is at
+// least ne for M = N.
+cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
+                            int64_t ncols, const double2* B, int64_t ldb, const Epilogue& ep,
+                            OzakiWork& w);
+int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M);
 // X (M x K, column-major, M <= N) <- the digits it has as the left
 // operand of ozaki_gemm_general (rows scaled by powers of two, six digits), so
 // that such a product takes X exactly: a change of at most 2^-49 of each row's
