@@ -201,9 +201,10 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
 // Batched small Jacobi (n <= 64) on `batch` column-major n x n matrices with
 // stride n*n; eigenvalues ascending (w: batch x n), eigenvectors Z; *status
 // (device) set to 1 when a sweep cap is hit.
-// max_sweeps > 0 lowers the sweep cap (default 40).
+// max_sweeps > 0 lowers the sweep cap (default 40). real: the matrices are real
+// (their imaginary parts are not read).
 cudaError_t jacobi_small_batched(cudaStream_t s, int n, int batch, const double2* G, double* w,
-                                 double2* Z, int* status, int max_sweeps = 0);
+                                 double2* Z, int* status, int max_sweeps = 0, bool real = false);
 
 // -------------------------------------------------------------- vector ops
 cudaError_t copy_cols(cudaStream_t s, int64_t m, int64_t n, const double2* src, int64_t lds,

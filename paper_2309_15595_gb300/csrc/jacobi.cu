@@ -32,50 +32,6 @@ namespace {
 constexpr int kMaxSweeps = 40;
 constexpr int kCoopMaxGrid = 2048;  // reduction scratch holds 2 * kCoopMaxGrid partials
 
-struct Rot {
-  double c, s, px, py, app, aqq;  // px + i py = phi
-};
-
-__device__ __forceinline__ Rot make_rot(double a, double d, double2 b) {
-  Rot r;
-  const double ab = sqrt(cabs2(b));
-  if (!(ab > 1e-300)) {
-    r.c = 1.0; r.s = 0.0; r.px = 1.0; r.py = 0.0; r.app = a; r.aqq = d;
-    return r;
-  }
-  r.px = b.x / ab;
-  r.py = b.y / ab;
-  const double tau = (d - a) / (2.0 * ab);
-  double t;
-  if (fabs(tau) > 1e150) {
-    t = 0.5 / tau;
-  } else {
-    t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-  }
-  r.c = 1.0 / sqrt(1.0 + t * t);
-  r.s = t * r.c;
-  r.app = a - t * ab;
-  r.aqq = d + t * ab;
-  return r;
-}
-
-// (x_p, x_q) <- (x_p, x_q) J  (column rotation)
-__device__ __forceinline__ void rot_cols(double2& xp, double2& xq, const Rot& r) {
-  const double2 phi = make_double2(r.px, r.py);
-  const double2 np_ = csub(cscale(r.c, xp), cscale(r.s, cmul(xq, conjz(phi))));
-  const double2 nq = cadd(cscale(r.s, cmul(xp, phi)), cscale(r.c, xq));
-  xp = np_;
-  xq = nq;
-}
-// (y_p; y_q) <- J^H (y_p; y_q)  (row rotation)
-__device__ __forceinline__ void rot_rows(double2& yp, double2& yq, const Rot& r) {
-  const double2 phi = make_double2(r.px, r.py);
-  const double2 np_ = csub(cscale(r.c, yp), cscale(r.s, cmul(phi, yq)));
-  const double2 nq = cadd(cscale(r.s, cmul(conjz(phi), yp)), cscale(r.c, yq));
-  yp = np_;
-  yq = nq;
-}
-
 __device__ __forceinline__ void rr_pair(int m, int round, int k, int& p, int& q) {
   auto pos = [&](int i) { return i == 0 ? 0 : 1 + (i - 1 + round) % (m - 1); };
   p = pos(k);
@@ -100,35 +56,106 @@ constexpr int64_t kSmallFp64 = 24;
 // tensor cores.
 constexpr int64_t kCoreRefine = 128;
 
+// A whole FP64 Jacobi in one CTA, n <= 64 (one SM: two DFMA a clock, so FP64
+// operations are what a round costs). The matrix is scaled by a power of two to
+// entries of at most 1 and padded to an even order. Per round: the rotations, with
+// the angle from FP32 and the cosine (and phase) made exact to FP64, so that the
+// rotated entry is small and not zero (a sweep still gains seven digits at the
+// least); then each 2 x 2 block where two pairs meet is rotated from both sides at
+// once and mirrored, and Z by columns. REAL: a real symmetric matrix (the Lanczos
+// tridiagonals), a quarter of the operations. n = 25, four matrices: 1.1 ms with FP64
+// angles, separate passes over columns and rows and complex arithmetic.
+template <bool REAL> struct Sj;
+template <> struct Sj<true> {
+  using C = double;
+  static __device__ __forceinline__ C mk(double x, double) { return x; }
+  static __device__ __forceinline__ double re(C a) { return a; }
+  static __device__ __forceinline__ double abs2(C a) { return a * a; }
+  static __device__ __forceinline__ C conj(C a) { return a; }
+  // c x - w y  and  c x + w y
+  static __device__ __forceinline__ C sub(double c, C x, C w, C y) { return fma(c, x, -(w * y)); }
+  static __device__ __forceinline__ C add(double c, C x, C w, C y) { return fma(c, x, w * y); }
+  static __device__ __forceinline__ double2 z(C a) { return make_double2(a, 0.0); }
+};
+template <> struct Sj<false> {
+  using C = double2;
+  static __device__ __forceinline__ C mk(double x, double y) { return make_double2(x, y); }
+  static __device__ __forceinline__ double re(C a) { return a.x; }
+  static __device__ __forceinline__ double abs2(C a) { return cabs2(a); }
+  static __device__ __forceinline__ C conj(C a) { return conjz(a); }
+  static __device__ __forceinline__ C sub(double c, C x, C w, C y) {
+    return make_double2(fma(c, x.x, fma(-w.x, y.x, w.y * y.y)),
+                        fma(c, x.y, -fma(w.x, y.y, w.y * y.x)));
+  }
+  static __device__ __forceinline__ C add(double c, C x, C w, C y) {
+    return make_double2(fma(c, x.x, fma(w.x, y.x, -(w.y * y.y))),
+                        fma(c, x.y, fma(w.x, y.y, w.y * y.x)));
+  }
+  static __device__ __forceinline__ double2 z(C a) { return a; }
+};
+// 1 / sqrt(w) for w in FP32's normal range: an FP32 seed and two Newton steps
+__device__ __forceinline__ double rsqrt_seeded(double w, float wf) {
+  double y = (double)rsqrtf(wf);
+  const double h = 0.5 * w;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = fma(y, fma(-h * y, y, 0.5), y);
+  return y;
+}
+
+constexpr int SJ_LD = SJ_MAX + 1;
+constexpr double kSjSkip = 1e-18;  // entries this far below the largest one stay
+
+template <bool REAL>
 __global__ void __launch_bounds__(SJ_T)
     jacobi_small_kernel(int n, const double2* __restrict__ Gin, double* __restrict__ w,
                         double2* __restrict__ Zout, int* status, int max_sweeps) {
+  using O = Sj<REAL>;
+  using C = typename O::C;
+  struct SjRot {
+    double c;
+    C u;  // s phi
+    int p, q, on;
+  };
   extern __shared__ double2 sm[];
-  double2* G = sm;                    // n x n, ld SJ_MAX
-  double2* Z = sm + SJ_MAX * SJ_MAX;  // n x n
-  __shared__ Rot rots[SJ_MAX / 2 + 1];
+  C* G = reinterpret_cast<C*>(sm);  // m x m, ld SJ_LD
+  C* Z = G + SJ_MAX * SJ_LD;
+  __shared__ SjRot rots[SJ_MAX / 2];
   __shared__ double red[SJ_T], red2[SJ_T];
-  __shared__ int rank_s[SJ_MAX];
+  __shared__ int rank_s[SJ_MAX], s_exp;
   const int t = threadIdx.x;
   const double2* Gb = Gin + (size_t)blockIdx.x * n * n;
+  const int m = n + (n & 1), npairs = m / 2, nblocks = npairs * (npairs - 1) / 2;
+  if (t == 0) s_exp = 0;
+  __syncthreads();
+  int ex = 0;
   for (int e = t; e < n * n; e += SJ_T) {
-    const int r = e % n, c = e / n;
+    const double2 v = Gb[e];
+    ex = max(ex, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+  }
+  atomicMax(&s_exp, ex);
+  __syncthreads();
+  // 2^sh G has entries below 1; nothing is scaled where that leaves FP64's range
+  const int sh = s_exp > 0 && s_exp < 2040 ? 1022 - s_exp : 0;
+  for (int e = t; e < m * m; e += SJ_T) {
+    const int r = e % m, c = e / m;
     // Hermitian part of the input (inputs formed as X^H (G X) are Hermitian
     // only up to rounding)
-    const double2 a = Gb[e], b = Gb[c + r * n];
-    G[r + c * SJ_MAX] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-    Z[r + c * SJ_MAX] = make_double2(r == c ? 1.0 : 0.0, 0.0);
+    C g = O::mk(0.0, 0.0);
+    if (r < n && c < n) {
+      const double2 a = Gb[r + c * n], b = Gb[c + r * n];
+      g = O::mk(ldexp(0.5 * a.x + 0.5 * b.x, sh), ldexp(0.5 * a.y - 0.5 * b.y, sh));
+    }
+    G[r + c * SJ_LD] = g;
+    Z[r + c * SJ_LD] = O::mk(r == c ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
-  const int m = n + (n & 1);
-  const int npairs = m / 2;
   double off_prev = 1e300;
   bool conv = false;
   for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
     double so = 0.0, sf = 0.0;
-    for (int e = t; e < n * n; e += SJ_T) {
-      const int r = e % n, c = e / n;
-      const double v = cabs2(G[r + c * SJ_MAX]);
+    for (int e = t; e < m * m; e += SJ_T) {
+      const int r = e % m, c = e / m;
+      const double v = O::abs2(G[r + c * SJ_LD]);
       sf += v;
       if (r != c) so += v;
     }
@@ -149,41 +176,78 @@ __global__ void __launch_bounds__(SJ_T)
     if (sweep == max_sweeps) break;
     for (int round = 0; round < m - 1; ++round) {
       if (t < npairs) {
-        int p, q;
-        rr_pair(m, round, t, p, q);
-        if (q < n) {
-          rots[t] = make_rot(G[p + p * SJ_MAX].x, G[q + q * SJ_MAX].x, G[p + q * SJ_MAX]);
-        } else {
-          rots[t] = make_rot(0.0, 0.0, make_double2(0.0, 0.0));
+        SjRot r;
+        rr_pair(m, round, t, r.p, r.q);
+        C* gp = G + r.p * SJ_LD;
+        C* gq = G + r.q * SJ_LD;
+        const double a = O::re(gp[r.p]), d = O::re(gq[r.q]), delta = d - a;
+        const C b = gq[r.p];  // G(p, q)
+        const double bb = O::abs2(b);
+        r.c = 1.0;
+        r.u = O::mk(0.0, 0.0);
+        r.on = bb > kSjSkip * kSjSkip;
+        if (r.on) {
+          const float bf = (float)bb, rf = rsqrtf(bf);
+          const float tau = 0.5f * (float)delta * rf;
+          const float tf = copysignf(
+              __fdividef(1.f, fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f))), tau);
+          const double tt = (double)tf, ww = fma(tt, tt, 1.0);
+          r.c = rsqrt_seeded(ww, (float)ww);
+          const double sn = tt * r.c, ri = REAL ? 0.0 : rsqrt_seeded(bb, bf);
+          const double ab = REAL ? fabs(O::re(b)) : bb * ri;
+          const double s2 = sn * sn, cs = r.c * sn;
+          const double v = fma(s2, delta, -2.0 * cs * ab);
+          const double no = fma(fma(r.c, r.c, -s2), ab, -cs * delta);  // what is left of |b|
+          if constexpr (REAL) {
+            const double sg = O::re(b) < 0.0 ? -1.0 : 1.0;
+            r.u = sg * sn;
+            gq[r.p] = gp[r.q] = sg * no;
+          } else {
+            const double2 ph = cscale(ri, b);
+            r.u = cscale(sn, ph);
+            gq[r.p] = cscale(no, ph);
+            gp[r.q] = conjz(gq[r.p]);
+          }
+          gp[r.p] = O::mk(a + v, 0.0);
+          gq[r.q] = O::mk(d - v, 0.0);
         }
+        rots[t] = r;
       }
       __syncthreads();
-      for (int e = t; e < npairs * n; e += SJ_T) {  // column rotations of G and Z
-        const int k = e / n, i = e % n;
-        int p, q;
-        rr_pair(m, round, k, p, q);
-        if (q >= n) continue;
-        rot_cols(G[i + p * SJ_MAX], G[i + q * SJ_MAX], rots[k]);
-        rot_cols(Z[i + p * SJ_MAX], Z[i + q * SJ_MAX], rots[k]);
+      for (int e = t; e < nblocks; e += SJ_T) {  // block (k, l), k < l: number l (l-1)/2 + k
+        int l = (int)((1.f + sqrtf(8.f * (float)e + 1.f)) * 0.5f);
+        while (l * (l - 1) / 2 > e) --l;
+        while (l * (l + 1) / 2 <= e) ++l;
+        const SjRot& jk = rots[e - l * (l - 1) / 2];
+        const SjRot& jl = rots[l];
+        if (!(jk.on | jl.on)) continue;
+        const int pk = jk.p, qk = jk.q, pl = jl.p, ql = jl.q;
+        const double ck = jk.c, cl = jl.c;
+        const C uk = jk.u, ul = jl.u, uck = O::conj(uk), ucl = O::conj(ul);
+        const C x0 = G[pk + pl * SJ_LD], x1 = G[pk + ql * SJ_LD];
+        const C x2 = G[qk + pl * SJ_LD], x3 = G[qk + ql * SJ_LD];
+        // columns of pair l, then rows of pair k
+        const C y0 = O::sub(cl, x0, ucl, x1), y1 = O::add(cl, x1, ul, x0);
+        const C y2 = O::sub(cl, x2, ucl, x3), y3 = O::add(cl, x3, ul, x2);
+        const C z0 = O::sub(ck, y0, uk, y2), z2 = O::add(ck, y2, uck, y0);
+        const C z1 = O::sub(ck, y1, uk, y3), z3 = O::add(ck, y3, uck, y1);
+        G[pk + pl * SJ_LD] = z0;
+        G[pk + ql * SJ_LD] = z1;
+        G[qk + pl * SJ_LD] = z2;
+        G[qk + ql * SJ_LD] = z3;
+        G[pl + pk * SJ_LD] = O::conj(z0);
+        G[ql + pk * SJ_LD] = O::conj(z1);
+        G[pl + qk * SJ_LD] = O::conj(z2);
+        G[ql + qk * SJ_LD] = O::conj(z3);
       }
-      __syncthreads();
-      for (int e = t; e < npairs * n; e += SJ_T) {  // row rotations of G
-        const int k = e / n, j = e % n;
-        int p, q;
-        rr_pair(m, round, k, p, q);
-        if (q >= n) continue;
-        rot_rows(G[p + j * SJ_MAX], G[q + j * SJ_MAX], rots[k]);
-      }
-      __syncthreads();
-      if (t < npairs) {
-        int p, q;
-        rr_pair(m, round, t, p, q);
-        if (q < n && rots[t].s != 0.0) {
-          G[p + q * SJ_MAX] = make_double2(0.0, 0.0);
-          G[q + p * SJ_MAX] = make_double2(0.0, 0.0);
-          G[p + p * SJ_MAX] = make_double2(rots[t].app, 0.0);
-          G[q + q * SJ_MAX] = make_double2(rots[t].aqq, 0.0);
-        }
+      for (int e = t; e < npairs * n; e += SJ_T) {
+        const SjRot& r = rots[e / n];
+        if (!r.on) continue;
+        C* zp = Z + r.p * SJ_LD + e % n;
+        C* zq = Z + r.q * SJ_LD + e % n;
+        const C x = *zp, y = *zq;
+        *zp = O::sub(r.c, x, O::conj(r.u), y);
+        *zq = O::add(r.c, y, r.u, x);
       }
       __syncthreads();
     }
@@ -191,10 +255,10 @@ __global__ void __launch_bounds__(SJ_T)
   if (t == 0 && !conv) *status = 1;
   // rank sort of the diagonal (ties by index)
   if (t < n) {
-    const double v = G[t + t * SJ_MAX].x;
+    const double v = O::re(G[t + t * SJ_LD]);
     int rk = 0;
     for (int j = 0; j < n; ++j) {
-      const double u = G[j + j * SJ_MAX].x;
+      const double u = O::re(G[j + j * SJ_LD]);
       rk += (u < v) || (u == v && j < t);
     }
     rank_s[t] = rk;
@@ -202,10 +266,10 @@ __global__ void __launch_bounds__(SJ_T)
   __syncthreads();
   double* wb = w + (size_t)blockIdx.x * n;
   double2* Zb = Zout + (size_t)blockIdx.x * n * n;
-  if (t < n) wb[rank_s[t]] = G[t + t * SJ_MAX].x;
+  if (t < n) wb[rank_s[t]] = ldexp(O::re(G[t + t * SJ_LD]), -sh);
   for (int e = t; e < n * n; e += SJ_T) {
     const int r = e % n, c = e / n;
-    Zb[r + rank_s[c] * n] = Z[r + c * SJ_MAX];
+    Zb[r + rank_s[c] * n] = O::z(Z[r + c * SJ_LD]);
   }
 }
 
@@ -1221,8 +1285,10 @@ __global__ void max2_kernel(int64_t nb, const double* __restrict__ partial, doub
   }
 }
 // Block S_c = X_c^H (G X_c) of each cluster c of size k (clusters of one size,
-// consecutive in XI / TI): one CTA per cluster, one warp per output entry at a
-// time, lanes over rows, fixed-order reduction. Output k x k column-major.
+// consecutive in XI / TI): CTAs (x: cluster, y: share of its entries) of 8 warps, one
+// warp per output entry at a time, lanes over rows, fixed-order reduction. Output
+// k x k column-major. (A CTA per cluster left it to a few SMs' FP64 pipes: 0.4 ms for
+// clusters of 20 columns of 1072.)
 __global__ void cluster_gram_kernel(int64_t n, int k, const double2* __restrict__ XI,
                                     const double2* __restrict__ TI, int64_t ld,
                                     double2* __restrict__ Sout) {
@@ -1230,7 +1296,7 @@ __global__ void cluster_gram_kernel(int64_t n, int k, const double2* __restrict_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double2* X = XI + (int64_t)c * k * ld;
   const double2* T = TI + (int64_t)c * k * ld;
-  for (int e = warp; e < k * k; e += blockDim.x >> 5) {
+  for (int e = warp + 8 * blockIdx.y; e < k * k; e += 8 * gridDim.y) {
     const int a = e % k, b = e / k;
     double2 acc = make_double2(0.0, 0.0);
     for (int64_t r = lane; r < n; r += 32) acc = cadd(acc, cmulc(X[r + a * ld], T[r + b * ld]));
@@ -1344,15 +1410,21 @@ size_t jacobi_rot_elems(int64_t n) {
 size_t jacobi_params_elems(int64_t n) { return (size_t)8 * (n / 2 + 2) + 8 + n; }
 
 cudaError_t jacobi_small_batched(cudaStream_t s, int n, int batch, const double2* G, double* w,
-                                 double2* Z, int* status, int max_sweeps) {
+                                 double2* Z, int* status, int max_sweeps, bool real) {
   if (n > SJ_MAX || n < 1) return cudaErrorInvalidValue;
-  const size_t smem = 2 * SJ_MAX * SJ_MAX * sizeof(double2);
-  once_per_device(g_small_attr, [smem]() {
-    cudaFuncSetAttribute(jacobi_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  constexpr size_t elems = 2 * SJ_MAX * SJ_LD;
+  once_per_device(g_small_attr, []() {
+    cudaFuncSetAttribute(jacobi_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(elems * sizeof(double2)));
+    cudaFuncSetAttribute(jacobi_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(elems * sizeof(double)));
   });
   const int cap = max_sweeps > 0 ? std::min(max_sweeps, kMaxSweeps) : kMaxSweeps;
-  jacobi_small_kernel<<<batch, SJ_T, smem, s>>>(n, G, w, Z, status, cap); count_launch();
+  if (real)
+    jacobi_small_kernel<true><<<batch, SJ_T, elems * sizeof(double), s>>>(n, G, w, Z, status, cap);
+  else
+    jacobi_small_kernel<false><<<batch, SJ_T, elems * sizeof(double2), s>>>(n, G, w, Z, status, cap);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -1457,7 +1529,8 @@ int cluster_finish(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, dou
       }
       continue;
     }
-    cluster_gram_kernel<<<g.count, 256, 0, s>>>(n, g.k, XI + off * n, wk.T + off * n, n, wk.Gw);
+    cluster_gram_kernel<<<dim3((unsigned)g.count, (unsigned)std::min<int64_t>(64, cdiv(g.k * g.k, 8)), 1),
+                          256, 0, s>>>(n, g.k, XI + off * n, wk.T + off * n, n, wk.Gw);
     count_launch();
     if (jacobi_small_batched(s, g.k, g.count, wk.Gw, wz + off, wk.Gw2, status, wk.max_sweeps) !=
         cudaSuccess)

@@ -213,7 +213,7 @@ cudaError_t lanczos_bounds(cudaStream_t s, int64_t N, const double2* A, int64_t 
     if (e != cudaSuccess) return e;
   }
   lz_build_t_kernel<<<nvec, 256, 0, s>>>(nvec, k, kmax, w.ab, w.T); count_launch();
-  e = jacobi_small_batched(s, k, nvec, w.T, w.theta, w.Z, w.status);
+  e = jacobi_small_batched(s, k, nvec, w.T, w.theta, w.Z, w.status, 0, true);
   if (e != cudaSuccess) return e;
   lz_bounds_kernel<<<1, 256, 0, s>>>(nvec, k, kmax, w.ab, w.theta, w.Z, (double)ne / (double)N,
                                      w.out4); count_launch();
