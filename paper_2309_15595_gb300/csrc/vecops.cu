@@ -29,18 +29,39 @@ __global__ void gather_cols_kernel(int64_t m, const double2* src, int64_t lds, c
 // mode 0: |Q0_i|^2            (start-vector norms)
 // mode 1: W_i -= beta_prev Qp_i; partial Re(conj(Q_i) W_i)
 // mode 2: W_i -= alpha Q_i;  partial |W_i|^2
+// Modes 2 and lz_scale_kernel add up the partial sums of the kernel before them in
+// every block (128 values, a fixed order), which saves the chain a launch of one
+// thread's 128 dependent loads each time; the first block keeps the scalar.
+__device__ __forceinline__ double sum_partials(const double* __restrict__ p, double* red) {
+  const int t = threadIdx.x;
+  static_assert(RB == 128, "four partials a lane");
+  if (t < 32) {
+    double s = (p[t] + p[t + 32]) + (p[t + 64] + p[t + 96]);
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (t == 0) red[0] = s;
+  }
+  __syncthreads();
+  const double s = red[0];
+  __syncthreads();
+  return s;
+}
+
 __global__ void lz_partial_kernel(int mode, int64_t N, int nvec, const double2* Q0, int64_t ldq,
-                                  const double2* Q, const double2* Qp, double2* W, const double* ab,
-                                  int step, int kmax, double* partial) {
+                                  const double2* Q, const double2* Qp, double2* W, double* ab,
+                                  int step, int kmax, const double* prev, double* partial) {
   __shared__ double red[VT];
   const int r = blockIdx.y;
   const int t = threadIdx.x;
   double s = 0.0;
-  const double* alpha = ab;               // [r * kmax + step]
+  double* alpha = ab;                     // [r * kmax + step]
   const double* beta = ab + 8 * kmax;     // [r * kmax + step]
   double bprev = 0.0, al = 0.0;
   if (mode == 1 && step > 0) bprev = beta[r * kmax + step - 1];
-  if (mode == 2) al = alpha[r * kmax + step];
+  if (mode == 2) {
+    al = sum_partials(prev + r * RB, red);
+    if (blockIdx.x == 0 && t == 0) alpha[r * kmax + step] = al;
+  }
   for (int64_t i = (int64_t)blockIdx.x * VT + t; i < N; i += (int64_t)RB * VT) {
     if (mode == 0) {
       s += cabs2(Q0[i + r * ldq]);
@@ -82,13 +103,16 @@ __global__ void lz_final_kernel(int nvec, const double* partial, double* dst, in
   dst[r * kmax + step] = take_sqrt ? sqrt(s) : s;
 }
 
-// out[:, r] = in[:, r] * (1 / scale[r * kmax + step])
+// scale[r * kmax + step] = sqrt(sum_b partial[b + r RB]), out[:, r] = in[:, r] / scale
 __global__ void lz_scale_kernel(int64_t N, int nvec, const double2* in, int64_t ldi, double2* out,
-                                const double* scale, int kmax, int step) {
+                                const double* partial, double* scale, int kmax, int step) {
+  __shared__ double red[1];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int r = blockIdx.y;
+  const double norm = sqrt(sum_partials(partial + r * RB, red));
+  if (i == 0) scale[r * kmax + step] = norm;
   if (i >= N) return;
-  const double inv = 1.0 / scale[r * kmax + step];
+  const double inv = 1.0 / norm;
   out[i + r * N] = cscale(inv, in[i + r * ldi]);
 }
 
@@ -186,11 +210,12 @@ cudaError_t lanczos_bounds(cudaStream_t s, int64_t N, const double2* A, int64_t 
   double* norms = w.ab + 16 * kmax;  // scratch row for start norms: [r * kmax + 0]
   const dim3 gp(RB, (unsigned)nvec, 1);
   const dim3 ge((unsigned)cdiv(N, 256), (unsigned)nvec, 1);
+  double* pa = w.red;            // partial sums of alpha
+  double* pb = w.red + 8 * RB;   // partial sums of norms and betas
   // q = q0 / ||q0||
   lz_partial_kernel<<<gp, VT, 0, s>>>(0, N, nvec, Q0, ldq, nullptr, nullptr, nullptr, w.ab, 0,
-                                      kmax, w.red); count_launch();
-  lz_final_kernel<<<1, 32, 0, s>>>(nvec, w.red, norms, kmax, 0, 1); count_launch();
-  lz_scale_kernel<<<ge, 256, 0, s>>>(N, nvec, Q0, ldq, Q, norms, kmax, 0); count_launch();
+                                      kmax, nullptr, pb); count_launch();
+  lz_scale_kernel<<<ge, 256, 0, s>>>(N, nvec, Q0, ldq, Q, pb, norms, kmax, 0); count_launch();
   lz_zero_kernel<<<(unsigned)cdiv(N * 8, 256), 256, 0, s>>>(N * 8, Qp); count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -199,15 +224,17 @@ cudaError_t lanczos_bounds(cudaStream_t s, int64_t N, const double2* A, int64_t 
                  : zgemm_skinny(s, N, nvec, A, lda, Q, N, W, N, w.ws);
     if (e != cudaSuccess) return e;
     // W -= beta_{j-1} q_prev ; alpha_j = Re(q^H W)
-    lz_partial_kernel<<<gp, VT, 0, s>>>(1, N, nvec, nullptr, 0, Q, Qp, W, w.ab, j, kmax, w.red); count_launch();
-    lz_final_kernel<<<1, 32, 0, s>>>(nvec, w.red, w.ab, kmax, j, 0); count_launch();
+    lz_partial_kernel<<<gp, VT, 0, s>>>(1, N, nvec, nullptr, 0, Q, Qp, W, w.ab, j, kmax, nullptr,
+                                        pa); count_launch();
     // W -= alpha_j q ; beta_j = ||W||
-    lz_partial_kernel<<<gp, VT, 0, s>>>(2, N, nvec, nullptr, 0, Q, Qp, W, w.ab, j, kmax, w.red); count_launch();
-    lz_final_kernel<<<1, 32, 0, s>>>(nvec, w.red, w.ab + 8 * kmax, kmax, j, 1); count_launch();
+    lz_partial_kernel<<<gp, VT, 0, s>>>(2, N, nvec, nullptr, 0, Q, Qp, W, w.ab, j, kmax, pa,
+                                        pb); count_launch();
     if (j + 1 < k) {
       // q_prev <- q ; q <- W / beta_j  (the old q_prev buffer receives the new q)
-      lz_scale_kernel<<<ge, 256, 0, s>>>(N, nvec, W, N, Qp, w.ab + 8 * kmax, kmax, j); count_launch();
+      lz_scale_kernel<<<ge, 256, 0, s>>>(N, nvec, W, N, Qp, pb, w.ab + 8 * kmax, kmax, j); count_launch();
       std::swap(Qp, Q);
+    } else {
+      lz_final_kernel<<<1, 32, 0, s>>>(nvec, pb, w.ab + 8 * kmax, kmax, j, 1); count_launch();
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
