@@ -339,7 +339,7 @@ __device__ __forceinline__ long long low_fixed(float v) { return __float2ll_rn(v
 
 // ---------------------------------------------------------------- kernel
 // CTA `local` of a product: tile local / split (128 x 64 outputs), part local %
-// split of its chunks; the per-problem kernel and the grouped kernel (the filter
+// split of its K blocks; the per-problem kernel and the grouped kernel (the filter
 // steps of many problems in one launch) both run it. The CTAs of a tile are
 // consecutive ranks of a cluster: each leaves its sums in its own shared memory
 // and then adds up and finishes 1 / split of the tile's columns. clustered: the
@@ -373,10 +373,10 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t m0 = (int64_t)rb * TM;
   const int64_t tile = P.j0 / CT + ct;            // absolute CT-column tile
-  const int nchunks_all = (int)((2 * P.Np) / TK) / CHUNK_KB;
-  const int chunk0 = (int)part * nchunks_all / P.split;  // this CTA's chunks
-  const int nchunks = ((int)part + 1) * nchunks_all / P.split - chunk0;
-  const int nkb = nchunks * CHUNK_KB;
+  const int nkb_all = (int)((2 * P.Np) / TK);
+  const int kb0 = (int)part * nkb_all / P.split;  // this CTA's K blocks, its chunks from there
+  const int nkb = ((int)part + 1) * nkb_all / P.split - kb0;
+  const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -421,7 +421,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
         const uint32_t full = smem_u32(&bars[s]);
         uint8_t* st = smem + s * kStage;
         mbar_expect_tx(full, kStage);
-        const int kx = (chunk0 * CHUNK_KB + kb) * TK;
+        const int kx = (kb0 + kb) * TK;
 #pragma unroll
         for (int d = 0; d < NS; ++d) {
           // digit planes are stacked along rows: digit d of row r is row d * rows + r
@@ -447,7 +447,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int kc = 0; kc < CHUNK_KB; ++kc, ++kb) {
+        for (int kc = 0; kc < CHUNK_KB && kb < nkb; ++kc, ++kb) {
           const int s = kb % kStages;
           const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
           if (!mbar_wait(smem_u32(&bars[s]), ph, P.err, 14) || *(volatile int*)&s_abort) {
@@ -773,6 +773,13 @@ __device__ __forceinline__ int scale_exp(double mx) {
   return E + 1;   // mx 2^-(E+1) in [0.25, 0.5)
 }
 
+// the same from the bit pattern of a maximum
+__device__ __forceinline__ int exp_of_bits(unsigned long long b) {
+  const int f = (int)(b >> 52);
+  if (f == 0 || f == 0x7ff) return scale_exp(__longlong_as_double((long long)b));
+  return f - 1021;
+}
+
 // Row maxima of A (column-major): amax[i] = max_k max(|Re A_ik|, |Im A_ik|),
 // as the bit pattern of a non-negative double (monotone in unsigned order).
 __global__ void rowmax_kernel(int64_t M, int64_t K, bool skip_diag, const double2* __restrict__ A,
@@ -801,13 +808,15 @@ __global__ void exps_kernel(int64_t n, const unsigned long long* __restrict__ mx
 }
 
 // A (M x K, column-major) -> OS digit planes, each M rows x 2 Np (row-major
-// [Ar | Ai]), stacked; skip_diag leaves the diagonal out (square A). A warp
+// [Ar | Ai]), stacked, and the rows' exponents from their maxima; skip_diag leaves the
+// diagonal out (square A). A warp
 // writes a row of 64 entries, two per lane: 128 bytes of each of its 12 rows.
 constexpr int SA_K = 64;
 template <int NS>
 __global__ void __launch_bounds__(256)
     slice_a_kernel(int64_t M, int64_t K, int64_t Np, bool skip_diag,
-                   const double2* __restrict__ A, int64_t lda, const int* __restrict__ ea,
+                   const double2* __restrict__ A, int64_t lda,
+                   const unsigned long long* __restrict__ amax, int* __restrict__ ea,
                    __nv_bfloat16* __restrict__ out) {
   __shared__ double2 tile[SA_K][33];
   const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * SA_K;
@@ -827,7 +836,8 @@ __global__ void __launch_bounds__(256)
     const int64_t i = i0 + r;
     if (i >= M) continue;
     const double2 a0 = tile[2 * tx][r], a1 = tile[2 * tx + 1][r];
-    const int e = ea[i];
+    const int e = exp_of_bits(amax[i]);
+    if (k0 == 0 && tx == 0) ea[i] = e;
     const Digits<NS> r0 = digits_of<NS>(a0.x, e), r1 = digits_of<NS>(a1.x, e);
     const Digits<NS> c0 = digits_of<NS>(a0.y, e), c1 = digits_of<NS>(a1.y, e);
     __nv_bfloat16* o = out + i * ld + k;
@@ -854,27 +864,28 @@ __global__ void round_left_kernel(int64_t M, int64_t K, double2* __restrict__ X,
 }
 
 // Left operand X^H for X (K x M, column-major): row i of X^H is conj(X[:, i]),
-// contiguous, so no transpose is needed. Exponents per row come from colexp.
-// Two entries per thread.
+// contiguous, so no transpose is needed. Exponents per row come from colexp. Entries
+// k, k + 1 (zero past K) of a row.
+__device__ __forceinline__ void slice_ct_pair(int64_t K, int64_t Np, size_t plane, int64_t k,
+                                              const double2* __restrict__ X, int e,
+                                              __nv_bfloat16* __restrict__ row) {
+  const double2 x0 = X[k];
+  const double2 x1 = k + 1 < K ? X[k + 1] : make_double2(0.0, 0.0);
+  const Digits<OS> r0 = digits_of<OS>(x0.x, e), r1 = digits_of<OS>(x1.x, e);
+  const Digits<OS> c0 = digits_of<OS>(-x0.y, e), c1 = digits_of<OS>(-x1.y, e);
+#pragma unroll
+  for (int d = 0; d < OS; ++d) {
+    *reinterpret_cast<unsigned*>(row + d * plane + k) = pack_digits(r0.d[d], r1.d[d]);
+    *reinterpret_cast<unsigned*>(row + d * plane + Np + k) = pack_digits(c0.d[d], c1.d[d]);
+  }
+}
 __global__ void slice_ct_kernel(int64_t M, int64_t K, int64_t Np, const double2* __restrict__ X,
                                 int64_t ldx, const int* __restrict__ ea,
                                 __nv_bfloat16* __restrict__ out) {
   const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t i = blockIdx.y;
   if (k >= K) return;
-  const double2 x0 = X[k + i * ldx];
-  const double2 x1 = k + 1 < K ? X[k + 1 + i * ldx] : make_double2(0.0, 0.0);
-  const int e = ea[i];
-  const Digits<OS> r0 = digits_of<OS>(x0.x, e), r1 = digits_of<OS>(x1.x, e);
-  const Digits<OS> c0 = digits_of<OS>(-x0.y, e), c1 = digits_of<OS>(-x1.y, e);
-  const int64_t ld = 2 * Np;
-  const size_t plane = (size_t)M * ld;
-  __nv_bfloat16* o = out + i * ld + k;
-#pragma unroll
-  for (int d = 0; d < OS; ++d) {
-    *reinterpret_cast<unsigned*>(o + d * plane) = pack_digits(r0.d[d], r1.d[d]);
-    *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
-  }
+  slice_ct_pair(K, Np, (size_t)M * 2 * Np, k, X + i * ldx, ea[i], out + i * 2 * Np);
 }
 
 // Column maxima of Y (complex columns j0 .. j0 + gridDim.x): one CTA per column.
@@ -942,6 +953,46 @@ __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
                out + (br + CT) * ld);
 }
 
+// Maximum, exponent and digits of one column of the right operand by one CTA of 256
+// threads (the second reading comes from the caches). A separate pass for the
+// exponents costs a launch: 4.3 us against 2 + 2.3 us and the gap between them for 60
+// columns of 512 rows. Longer columns, which one CTA reads too slowly (64 of 2048
+// rows: 10.4 against 5.5 us), take the two passes.
+constexpr int64_t kOnePass = 1024;
+template <int NS>
+__device__ __forceinline__ void slice_b_column(int64_t N, int64_t Np, int64_t brows, int64_t j,
+                                               const double2* __restrict__ Y,
+                                               int* __restrict__ eb, __nv_bfloat16* __restrict__ out,
+                                               unsigned long long* red) {
+  const int ex = scale_exp(__longlong_as_double((long long)column_max(N, Y, red)));
+  if (threadIdx.x == 0) eb[j] = ex;
+  const int64_t ld = 2 * Np, br = brow_re(j);
+  for (int64_t k = 2 * threadIdx.x; k < N; k += 512)
+    slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y, ex, out + br * ld, out + (br + CT) * ld);
+}
+template <int NS>
+__global__ void __launch_bounds__(256)
+    slice_b_column_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
+                          const double2* __restrict__ Y, int64_t ldy, int* __restrict__ eb,
+                          __nv_bfloat16* __restrict__ out) {
+  __shared__ unsigned long long red[8];
+  const int64_t j = j0 + blockIdx.x;
+  slice_b_column<NS>(N, Np, brows, j, Y + j * ldy, eb, out, red);
+}
+// The same for the left operand X^H: row i is the conjugate of X's column i.
+__global__ void __launch_bounds__(256)
+    slice_ct_column_kernel(int64_t M, int64_t K, int64_t Np, const double2* __restrict__ X,
+                           int64_t ldx, int* __restrict__ el, __nv_bfloat16* __restrict__ out) {
+  __shared__ unsigned long long red[8];
+  const int64_t i = blockIdx.x;
+  const double2* Xi = X + i * ldx;
+  const int ex = scale_exp(__longlong_as_double((long long)column_max(K, Xi, red)));
+  if (threadIdx.x == 0) el[i] = ex;
+  const int64_t ld = 2 * Np;
+  for (int64_t k = 2 * threadIdx.x; k < K; k += 512)
+    slice_ct_pair(K, Np, (size_t)M * ld, k, Xi, ex, out + i * ld);
+}
+
 // The right-operand digits of many problems' filter steps in one launch: one
 // CTA (256 threads) per active column of every problem. It forms the column's
 // maximum with the reduction of colexp_kernel, then the column's digits as
@@ -967,11 +1018,7 @@ __global__ void __launch_bounds__(256)
   const OzSliceEntry& e = tab[lo];
   const int64_t N = e.N, j = e.j0 + (id - e.first);
   const double2* __restrict__ Y = e.B + j * e.ldb;
-  const int ex = scale_exp(__longlong_as_double((long long)column_max(N, Y, red)));
-  if (threadIdx.x == 0) e.eb[j] = ex;
-  const int64_t ld = 2 * e.Np, br = brow_re(j);
-  for (int64_t k = 2 * threadIdx.x; k < N; k += 512)
-    slice_b_pair<OS>(N, e.Np, (size_t)e.brows * ld, k, Y, ex, e.out + br * ld, e.out + (br + CT) * ld);
+  slice_b_column<OS>(N, e.Np, e.brows, j, Y, e.eb, e.out, red);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 lookup_encoder() {
@@ -1014,12 +1061,12 @@ struct Maps {
 // depends on the product alone, so a problem's result is the same in a group.
 constexpr int kMaxSplit = 8;
 int choose_split(int64_t tiles, int64_t Np) {
-  const int64_t nchunks = 2 * Np / (TK * CHUNK_KB), sms = num_sms();
+  const int64_t nkb = 2 * Np / TK, sms = num_sms();
   int best = 1;
   double best_cost = 1e300;
-  for (int s = 1; s <= kMaxSplit && s <= nchunks; s *= 2) {
-    const double cost =
-        (double)cdiv(tiles * s, sms) * ((double)cdiv(nchunks, s) + 1.0 + 1.5 / s);
+  for (int s = 1; s <= kMaxSplit && 4 * s <= nkb; s *= 2) {  // at least half a chunk each
+    const double cost = (double)cdiv(tiles * s, sms) *
+                        ((double)cdiv(nkb, s) / CHUNK_KB + 1.0 + 1.5 / s);
     if (cost < 0.9 * best_cost) {
       best_cost = cost;
       best = s;
@@ -1148,28 +1195,41 @@ cudaError_t ozaki_prepare_a(cudaStream_t s, const double2* A, int64_t lda, Ozaki
   rowmax_kernel<<<dim3((unsigned)cdiv(N, 256), (unsigned)cdiv(N, 256), 1), 256, 0, s>>>(
       N, N, true, A, lda, w.amax);
   count_launch();
-  exps_kernel<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(N, w.amax, w.ea);
-  count_launch();
   diag_kernel<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(N, A, lda, w.diag);
   count_launch();
   slice_a_kernel<OS><<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
-      N, N, w.Np, true, A, lda, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
+      N, N, w.Np, true, A, lda, w.amax, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
   count_launch();
   w.A_ready = A;
   return cudaGetLastError();
 }
+
+namespace {
+// Digits of columns j0 .. j0 + n of B (K rows) into w.Bd (`brows` rows a plane).
+template <int NS>
+void slice_right(cudaStream_t s, int64_t K, int64_t j0, int64_t n, const double2* B, int64_t ldb,
+                 int64_t brows, OzakiWork& w) {
+  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w.Bd);
+  count_launch();
+  if (K <= kOnePass) {
+    slice_b_column_kernel<NS><<<(unsigned)n, 256, 0, s>>>(K, ozaki_np(K), brows, j0, B, ldb, w.eb,
+                                                          out);
+    return;
+  }
+  colexp_kernel<<<(unsigned)n, 256, 0, s>>>(K, j0, B, ldb, w.eb);
+  slice_b_kernel<NS><<<dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, 0, s>>>(
+      K, ozaki_np(K), brows, j0, B, ldb, w.eb, out);
+  count_launch();
+}
+
+}  // namespace
 
 cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const double2* B,
                        int64_t ldb, const Epilogue& ep, OzakiWork& w) {
   const int64_t N = w.N;
   const int64_t n = ncols_end - j0;
   if (n <= 0) return cudaSuccess;
-  // digits of the active columns of B
-  colexp_kernel<<<(unsigned)n, 256, 0, s>>>(N, j0, B, ldb, w.eb);
-  count_launch();
-  slice_b_kernel<OS><<<dim3((unsigned)cdiv(N, 512), (unsigned)n, 1), 256, 0, s>>>(
-      N, w.Np, w.brows, j0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
-  count_launch();
+  slice_right<OS>(s, N, j0, n, B, ldb, w.brows, w);
   const Maps* maps = static_cast<const Maps*>(w.maps);
   const Params P = product_params(w, ncols_end, j0, B, ldb, ep);
   return launch_product(s, maps->a, maps->b, P, PAIRS_21);
@@ -1185,10 +1245,8 @@ cudaError_t slice_left(cudaStream_t s, int64_t M, int64_t K, const double2* X, i
   rowmax_kernel<<<dim3((unsigned)cdiv(M, 256), (unsigned)cdiv(K, 256), 1), 256, 0, s>>>(
       M, K, false, X, ldx, w.amax);
   count_launch();
-  exps_kernel<<<(unsigned)cdiv(M, 256), 256, 0, s>>>(M, w.amax, w.el);
-  count_launch();
   slice_a_kernel<NS><<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, SA_K), 1), dim3(32, 8, 1), 0,
-                       s>>>(M, K, ozaki_np(K), false, X, ldx, w.el,
+                       s>>>(M, K, ozaki_np(K), false, X, ldx, w.amax, w.el,
                             static_cast<__nv_bfloat16*>(w.Ld));
   count_launch();
   return cudaGetLastError();
@@ -1202,16 +1260,6 @@ cudaError_t clear_left(cudaStream_t s, int64_t M, int64_t K, int ns, OzakiWork& 
   w.l_K = K;
   w.l_ns = ns;
   return cudaMemsetAsync(w.Ld, 0, (size_t)ns * M * 2 * ozaki_np(K) * 2, s);
-}
-// Digits of the columns of B (K x ncols) into w.Bd (`brows` rows a plane).
-template <int NS>
-void slice_right(cudaStream_t s, int64_t K, int64_t ncols, const double2* B, int64_t ldb,
-                 int64_t brows, OzakiWork& w) {
-  colexp_kernel<<<(unsigned)ncols, 256, 0, s>>>(K, 0, B, ldb, w.eb);
-  count_launch();
-  slice_b_kernel<NS><<<dim3((unsigned)cdiv(K, 512), (unsigned)ncols, 1), 256, 0, s>>>(
-      K, ozaki_np(K), brows, 0, B, ldb, w.eb, static_cast<__nv_bfloat16*>(w.Bd));
-  count_launch();
 }
 // Parameters of a product with the left planes in w.Ld (no diagonal split).
 Params general_params(int64_t M, int64_t K, int64_t ncols, const double2* B, int64_t ldb,
@@ -1254,15 +1302,20 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
   cudaError_t e = clear_left(s, M, K, OS, w);
   if (e != cudaSuccess) return e;
   if (conj_trans) {  // left = X^H, X is K x M
-    colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
+    __nv_bfloat16* L = static_cast<__nv_bfloat16*>(w.Ld);
     count_launch();
-    slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(
-        M, K, Kp, X, ldx, w.el, static_cast<__nv_bfloat16*>(w.Ld));
-    count_launch();
+    if (K <= kOnePass) {
+      slice_ct_column_kernel<<<(unsigned)M, 256, 0, s>>>(M, K, Kp, X, ldx, w.el, L);
+    } else {
+      colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
+      slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(M, K, Kp, X, ldx,
+                                                                                   w.el, L);
+      count_launch();
+    }
   } else if ((e = slice_left<OS>(s, M, K, X, ldx, w)) != cudaSuccess) {  // left = X, M x K
     return e;
   }
-  slice_right<OS>(s, K, ncols, B, ldb, w.brows, w);
+  slice_right<OS>(s, K, 0, ncols, B, ldb, w.brows, w);
   CUtensorMap ma, mb;
   if (!make_map(&ma, w.Ld, (int64_t)OS * M, Kp, TM) ||
       !make_map(&mb, w.Bd, (int64_t)OS * w.brows, Kp, TN))
@@ -1296,7 +1349,7 @@ cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2*
     return cudaErrorInvalidValue;
   for (int64_t c0 = 0; c0 < ncols; c0 += block) {
     const int64_t nc = std::min(block, ncols - c0);
-    slice_right<OS7>(s, K, nc, B + c0 * ldb, ldb, brows, w);
+    slice_right<OS7>(s, K, 0, nc, B + c0 * ldb, ldb, brows, w);
     Epilogue ec = ep;
     if (ec.X) ec.X += c0 * ec.ldx;
     if (ec.Y) ec.Y += c0 * ec.ldy;
