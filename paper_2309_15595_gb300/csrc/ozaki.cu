@@ -264,6 +264,21 @@ struct Params {
   int split;                  // CTAs that share a tile's K range
 };
 
+// ------------------------------------------------- dependent launches
+// The kernels of a product (column exponents, digits, MMAs) follow each other in the
+// stream by the dozen and are short, so each may be launched while its predecessor
+// still runs (programmatic stream serialization): its CTAs get onto free SMs, the
+// product kernel sets up its barriers and tensor memory, and then every thread waits
+// here until the predecessor has finished and its writes are visible. Every kernel
+// of the chain waits before its first access, so finishing implies that all before
+// it have finished too. 20 filter steps with 512 rows: 0.57 -> 0.49 ms.
+__device__ __forceinline__ void wait_for_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void let_successor_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------------- cluster helpers
 // Cluster-wide barrier (release / acquire): every thread of every CTA arrives.
 __device__ __forceinline__ void cluster_sync() {
@@ -399,6 +414,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  wait_for_predecessor();
 
   bool go = true;
   if (warp == 0) {
@@ -677,6 +693,7 @@ template <int LMAX, int NS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       Params P) {
+  let_successor_start();
   ozaki_tile<LMAX, NS>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
 }
 
@@ -914,6 +931,8 @@ __global__ void __launch_bounds__(256)
                   int* __restrict__ eb) {
   __shared__ unsigned long long red[8];
   const int64_t j = j0 + blockIdx.x;
+  let_successor_start();
+  wait_for_predecessor();
   const unsigned long long m = column_max(N, Y + j * ldy, red);
   if (threadIdx.x == 0) eb[j] = scale_exp(__longlong_as_double((long long)m));
 }
@@ -947,6 +966,8 @@ __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
                                __nv_bfloat16* __restrict__ out) {
   const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t j = j0 + blockIdx.y;
+  let_successor_start();
+  wait_for_predecessor();
   if (k >= N) return;
   const int64_t ld = 2 * Np, br = brow_re(j);
   slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], out + br * ld,
@@ -977,6 +998,8 @@ __global__ void __launch_bounds__(256)
                           __nv_bfloat16* __restrict__ out) {
   __shared__ unsigned long long red[8];
   const int64_t j = j0 + blockIdx.x;
+  let_successor_start();
+  wait_for_predecessor();
   slice_b_column<NS>(N, Np, brows, j, Y + j * ldy, eb, out, red);
 }
 // The same for the left operand X^H: row i is the conjugate of X's column i.
@@ -1076,19 +1099,26 @@ int choose_split(int64_t tiles, int64_t Np) {
 }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned ctas, int cluster, cudaStream_t s,
-                            Args... args) {
+cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned ctas, int cluster, bool early,
+                            cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(ctas, 1, 1);
   cfg.blockDim = dim3(NTHREADS, 1, 1);
   cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)cluster;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  cudaLaunchAttribute at[2]{};
+  if (cluster > 1) {
+    cudaLaunchAttribute& c = at[cfg.numAttrs++];
+    c.id = cudaLaunchAttributeClusterDimension;
+    c.val.clusterDim.x = (unsigned)cluster;
+    c.val.clusterDim.y = c.val.clusterDim.z = 1;
+  }
+  if (early) {
+    cudaLaunchAttribute& e = at[cfg.numAttrs++];
+    e.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    e.val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = at;
   count_launch();
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
@@ -1099,7 +1129,7 @@ cudaError_t launch_product(cudaStream_t s, const CUtensorMap& a, const CUtensorM
   auto* k = pairs == PAIRS_21   ? ozaki_gemm_kernel<7, OS>
             : pairs == PAIRS_26 ? ozaki_gemm_kernel<8, OS>
                                 : ozaki_gemm_kernel<8, OS7>;
-  return launch_clusters(k, ctas, P.split, s, a, b, P);
+  return launch_clusters(k, ctas, P.split, true, s, a, b, P);
 }
 void set_tiles(Params& P) {
   P.nrow = (int)cdiv(P.N, TM);
@@ -1205,21 +1235,36 @@ cudaError_t ozaki_prepare_a(cudaStream_t s, const double2* A, int64_t lda, Ozaki
 }
 
 namespace {
+// Launch that may begin while its predecessor in the stream still runs; the kernel
+// waits for it (wait_for_predecessor).
+template <typename... KArgs, typename... Args>
+void launch_early(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  count_launch();
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);  // the caller checks
+}
 // Digits of columns j0 .. j0 + n of B (K rows) into w.Bd (`brows` rows a plane).
 template <int NS>
 void slice_right(cudaStream_t s, int64_t K, int64_t j0, int64_t n, const double2* B, int64_t ldb,
                  int64_t brows, OzakiWork& w) {
   __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w.Bd);
-  count_launch();
+  const int64_t Kp = ozaki_np(K);
   if (K <= kOnePass) {
-    slice_b_column_kernel<NS><<<(unsigned)n, 256, 0, s>>>(K, ozaki_np(K), brows, j0, B, ldb, w.eb,
-                                                          out);
+    launch_early(slice_b_column_kernel<NS>, dim3((unsigned)n, 1, 1), 256, s, K, Kp, brows, j0, B,
+                 ldb, w.eb, out);
     return;
   }
-  colexp_kernel<<<(unsigned)n, 256, 0, s>>>(K, j0, B, ldb, w.eb);
-  slice_b_kernel<NS><<<dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, 0, s>>>(
-      K, ozaki_np(K), brows, j0, B, ldb, w.eb, out);
-  count_launch();
+  launch_early(colexp_kernel, dim3((unsigned)n, 1, 1), 256, s, K, j0, B, ldb, w.eb);
+  launch_early(slice_b_kernel<NS>, dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, s, K, Kp,
+               brows, j0, B, ldb, (const int*)w.eb, out);
 }
 
 }  // namespace
@@ -1519,7 +1564,7 @@ int ozaki_filter_grouped(cudaStream_t s, int count, const OzakiGroupItem* items,
     const int cnt = (int)(off[i + 1] - off[i]);
     slice_b_grouped_kernel<<<(unsigned)cols[i], 256, 0, s>>>(sdev + off[i], cnt);
     count_launch();
-    launch_clusters(ozaki_filter_grouped_kernel, (unsigned)ctas[i], cluster[i], s, dev + off[i], cnt,
+    launch_clusters(ozaki_filter_grouped_kernel, (unsigned)ctas[i], cluster[i], false, s, dev + off[i], cnt,
                     cluster[i] > 1);
   }
   const cudaError_t ce = cudaStreamEndCapture(s, &graph);
