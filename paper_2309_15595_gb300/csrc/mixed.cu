@@ -21,7 +21,8 @@
 // drain this one), and the epilogue warps add the chunk sums into FP32
 // registers with round-to-nearest adds.
 //
-// Kernel structure (one 256 x 256 output tile per pair of CTAs, 10 warps each):
+// Kernel structure (one 256 x 2 W output tile per pair of CTAs, W = 32, 64 or 128
+// complex columns, 10 warps each; figures for W = 128):
 //   warp 0   TMA producer: its 128 rows of A_hi, A_lo and its half of the 256 rows
 //            of B_hi, B_lo per K block of 32 into a 6-stage shared-memory ring of
 //            32 KB stages (64B swizzle: one K block of 32 BF16 is a 64-byte row)
@@ -63,13 +64,17 @@ namespace {
 // stages stay in flight while one is consumed, enough bytes in flight to
 // cover the TMA latency at the MMA rate.
 constexpr int TM = 128, TN = 256, TK = 32, STAGES = 6;
-constexpr int PAIR = 2;                             // CTAs of a pair: PAIR TM x TN outputs
+constexpr int PAIR = 2;                             // CTAs of a pair: PAIR TM x 2 W outputs
+// Complex columns W of a tile (2 W real ones, TN at the most; the pair's MMA takes
+// multiples of 32): see choose_width.
+constexpr int kWidths[] = {32, 64, 128};
+constexpr int kNumWidths = (int)(sizeof(kWidths) / sizeof(int));
+constexpr int kMaxWidth = TN / 2;
 constexpr int A_TILE = TM * TK * 2;                 // 8 KB
-constexpr int B_HALF = TN / PAIR;                   // operand rows a CTA of the pair holds
-constexpr int B_TILE = B_HALF * TK * 2;             // 8 KB
-constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;  // 32 KB
+constexpr int b_tile(int w) { return w * TK * 2; }  // W operand rows per CTA: 8 KB at most
+constexpr int stage_bytes(int w) { return 2 * A_TILE + 2 * b_tile(w); }  // 32 KB at most
 constexpr int KPAD = 64;                            // K-half padding of the planes
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int SMEM_BYTES = STAGES * stage_bytes(kMaxWidth) + 1024 + 256;
 constexpr int NTHREADS = 320;
 constexpr int EPI_WARPS = 8;
 constexpr int CHUNK_KB = 8;              // K blocks (of 32) per accumulation chunk: 256 values
@@ -85,6 +90,7 @@ struct Params {
   __nv_bfloat16* Bn_hi;         // next-step operand planes (rows = B^T rows, ld = 2 Np)
   __nv_bfloat16* Bn_lo;
   int write_next;
+  int width;                    // complex columns of a tile
   int nrow, ncol;               // pair rows and column tiles
   int group;                    // pair rows per sweep of the grouped raster order
   int* err;
@@ -169,15 +175,18 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
 }
 // Instruction descriptor: FP32 accumulate, BF16 A and B, both K-major, M x N over
 // the pair (each CTA's tensor memory receives its TM rows).
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                            ((uint32_t)(PAIR * TM >> 4) << 24);
+constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) |
+         ((uint32_t)(PAIR * TM >> 4) << 24);
+}
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
+                                          uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
+      "l"(a), "l"(b), "r"(id), "r"(acc)
       : "memory");
 }
 // Arrives on the barrier at this offset in both CTAs once the MMAs so far are done.
@@ -188,21 +197,21 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
       "h"((uint16_t)3)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
+// 16 consecutive TMEM columns of this warp's 32 lanes (no wait).
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+  uint32_t r[16];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
-      "%28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_wait_ld() {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // x in FP32, hi = bf16(x) and lo = bf16(x - hi) packed, the FP64 way (a call, so
@@ -251,24 +260,26 @@ __device__ __forceinline__ void split2f(float x, __nv_bfloat16& hi, __nv_bfloat1
   lo = __float2bfloat16_rn(x - __bfloat162float(hi));
 }
 
-// B^T row of complex column j: tile j/128 holds 256 rows, real parts first.
-__device__ __forceinline__ int64_t brow_re(int64_t j) { return (j >> 7) * 256 + (j & 127); }
+// B^T row of complex column j: tile j / W holds 2 W rows, real parts first.
+__device__ __forceinline__ int64_t brow_re(int64_t j, int w) { return j / w * 2 * w + j % w; }
 
 // ---------------------------------------------------------------- kernel
-// One 256 x 256 output tile (pair row rp, column tile ct of the active columns) of
+// One 256 x 2 W output tile (pair row rp, column tile ct of the active columns) of
 // one filter step by a pair of CTAs: each loads its 128 rows of A and half of the
 // operand rows (the real parts for rank 0, the imaginary ones for rank 1), the
 // leader issues MMAs over both, and each drains and updates its 128 rows. The
 // per-problem kernel and the grouped kernel (many problems in one launch) both
 // run it.
+template <int W>
 __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtensorMap* tmAl,
                                            const CUtensorMap* tmBh, const CUtensorMap* tmBl,
                                            const Params& P, unsigned rp, unsigned ct,
                                            bool maps_in_global) {
+  constexpr int kStage = stage_bytes(W), kBTile = b_tile(W), HALF = W / 2;
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment of the shared-window address (swizzle atoms)
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * kStage);
   // bars[0..S) full (the leader's), bars[S..2S) empty, bars[2S + b] accumulator b
   // full, bars[2S + 2 + b] accumulator b drained by both CTAs (the leader's)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
@@ -277,7 +288,7 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned rank = pair_rank();
   const int64_t m0 = ((int64_t)rp * PAIR + rank) * TM;
-  const int64_t tile = (P.j0 >> 7) + ct;          // absolute 128-column tile
+  const int64_t tile = P.j0 / W + ct;             // absolute W-column tile
   const int nkb = (int)((2 * P.Np) / TK);
   const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
 
@@ -324,13 +335,13 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
       }
       if (*(volatile int*)&s_abort) break;
       const uint32_t full = leader_smem(smem_u32(&bars[s]));
-      uint8_t* st = smem + s * STAGE_BYTES;
-      if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), PAIR * STAGE_BYTES);
-      const int kx = kb * TK, brow = (int)(tile * TN) + (int)rank * B_HALF;
+      uint8_t* st = smem + s * kStage;
+      if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), PAIR * kStage);
+      const int kx = kb * TK, brow = (int)(tile * 2 * W) + (int)rank * W;
       tma_load_2d(smem_u32(st), tmAh, kx, (int)m0, full);
       tma_load_2d(smem_u32(st + A_TILE), tmAl, kx, (int)m0, full);
       tma_load_2d(smem_u32(st + 2 * A_TILE), tmBh, kx, brow, full);
-      tma_load_2d(smem_u32(st + 2 * A_TILE + B_TILE), tmBl, kx, brow, full);
+      tma_load_2d(smem_u32(st + 2 * A_TILE + kBTile), tmBl, kx, brow, full);
       ++issued;
     }
     if (issued == nkb) {
@@ -369,16 +380,16 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t st = smem_u32(smem + s * STAGE_BYTES);
-        const uint32_t ah = st, al = st + A_TILE, bh = st + 2 * A_TILE, bl = bh + B_TILE;
+        const uint32_t st = smem_u32(smem + s * kStage);
+        const uint32_t ah = st, al = st + A_TILE, bh = st + 2 * A_TILE, bl = bh + kBTile;
 #pragma unroll
         for (int kk = 0; kk < TK / 16; ++kk) {
           const uint32_t off = kk * 32;  // 16 BF16 along K
           // each chunk restarts its accumulator
           const uint32_t acc0 = (kb > c * CHUNK_KB || kk > 0) ? 1u : 0u;
-          umma_bf16(acc_tm, sdesc_sw64(ah + off), sdesc_sw64(bh + off), acc0);
-          umma_bf16(acc_tm, sdesc_sw64(ah + off), sdesc_sw64(bl + off), 1u);
-          umma_bf16(acc_tm, sdesc_sw64(al + off), sdesc_sw64(bh + off), 1u);
+          umma_bf16(acc_tm, sdesc_sw64(ah + off), sdesc_sw64(bh + off), idesc(2 * W), acc0);
+          umma_bf16(acc_tm, sdesc_sw64(ah + off), sdesc_sw64(bl + off), idesc(2 * W), 1u);
+          umma_bf16(acc_tm, sdesc_sw64(al + off), sdesc_sw64(bh + off), idesc(2 * W), 1u);
         }
         umma_commit(smem_u32(&bars[STAGES + s]));  // stage free once these MMAs finish
       }
@@ -392,12 +403,12 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
   } else if (warp >= 2) {
     // ------------------------------------------------------- epilogue
     const int q = warp & 3;                  // TMEM lane quarter this warp may access
-    const int h = (warp - 2) >> 2;           // complex columns [h*64, h*64 + 64) of the tile
+    const int h = (warp - 2) >> 2;           // complex columns [h*HALF, h*HALF + HALF) of the tile
     const int64_t row = m0 + q * 32 + lane;
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-    float sre[64], sim[64];                  // chunk sums, round-to-nearest FP32 adds
+    float sre[HALF], sim[HALF];                  // chunk sums, round-to-nearest FP32 adds
 #pragma unroll
-    for (int j = 0; j < 64; ++j) {
+    for (int j = 0; j < HALF; ++j) {
       sre[j] = 0.f;
       sim[j] = 0.f;
     }
@@ -409,16 +420,18 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
       go = __all_sync(0xffffffffu, ok && !*(volatile int*)&s_abort);
       if (!go) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t ta = tl + (uint32_t)(b * TN + h * 64);
+      const uint32_t ta = tl + (uint32_t)(b * TN + h * HALF);
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        float v[32];
-        tmem_ld32(ta + half * 32, v);
+      for (int g = 0; g < HALF / 16; ++g) {
+        float v[16], u[16];
+        tmem_ld16(ta + g * 16, v);
+        tmem_ld16(ta + W + g * 16, u);
+        tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) sre[half * 32 + j] += v[j];
-        tmem_ld32(ta + 128 + half * 32, v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) sim[half * 32 + j] += v[j];
+        for (int j = 0; j < 16; ++j) {
+          sre[g * 16 + j] += v[j];
+          sim[g * 16 + j] += u[j];
+        }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -426,8 +439,8 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
     }
     if (go && row < P.N) {
 #pragma unroll
-      for (int jj = 0; jj < 64; ++jj) {  // fully unrolled: the sums stay in registers
-        const int64_t col = tile * 128 + h * 64 + jj;
+      for (int jj = 0; jj < HALF; ++jj) {  // fully unrolled: the sums stay in registers
+        const int64_t col = tile * W + h * HALF + jj;
         if (col < P.j0 || col >= P.ncols) continue;
         const float2 yc = P.Ycur[row + col * P.N];
         float2* yp = P.Yprev + row + col * P.N;
@@ -444,7 +457,7 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
           split2f(vr, rh, rl);
           split2f(vi, ih, il);
           split2f(-vi, nh, nl);
-          const int64_t br = brow_re(col), bi = br + 128, ld = 2 * P.Np;
+          const int64_t br = tile * 2 * W + h * HALF + jj, bi = br + W, ld = 2 * P.Np;
           P.Bn_hi[br * ld + row] = rh;
           P.Bn_lo[br * ld + row] = rl;
           P.Bn_hi[br * ld + P.Np + row] = nh;
@@ -468,6 +481,18 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
   }
 }
 
+// The tile in the step's width.
+__device__ __forceinline__ void mixed_tile_of(const CUtensorMap* ah, const CUtensorMap* al,
+                                              const CUtensorMap* bh, const CUtensorMap* bl,
+                                              const Params& P, unsigned rp, unsigned ct,
+                                              bool maps_in_global) {
+  switch (P.width) {
+    case 32: mixed_tile<32>(ah, al, bh, bl, P, rp, ct, maps_in_global); break;
+    case 64: mixed_tile<64>(ah, al, bh, bl, P, rp, ct, maps_in_global); break;
+    default: mixed_tile<128>(ah, al, bh, bl, P, rp, ct, maps_in_global); break;
+  }
+}
+
 __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
     mixed_filter_kernel(const __grid_constant__ CUtensorMap tmAh,
                         const __grid_constant__ CUtensorMap tmAl,
@@ -475,7 +500,7 @@ __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
                         const __grid_constant__ CUtensorMap tmBl, Params P) {
   unsigned rp, ct;  // pair row and column tile of this pair (grouped raster order)
   grouped_tile(blockIdx.x / PAIR, (unsigned)P.nrow, (unsigned)P.ncol, P.group, rp, ct);
-  mixed_tile(&tmAh, &tmAl, &tmBh, &tmBl, P, rp, ct, false);
+  mixed_tile_of(&tmAh, &tmAl, &tmBh, &tmBl, P, rp, ct, false);
 }
 
 // Many problems' filter steps in one launch: entry p of the table holds problem
@@ -503,7 +528,7 @@ __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
   unsigned rp, ct;
   grouped_tile((unsigned)(id - e->first) / PAIR, (unsigned)P.nrow, (unsigned)P.ncol, P.group, rp,
                ct);
-  mixed_tile(&e->ah, &e->al, &e->bh, &e->bl, P, rp, ct, true);
+  mixed_tile_of(&e->ah, &e->al, &e->bh, &e->bl, P, rp, ct, true);
 }
 
 // ----------------------------------------------------------- conversions
@@ -554,7 +579,8 @@ __global__ void __launch_bounds__(256)
 
 // Columns j0..ncols of Y (column-major complex) -> B^T planes (K-major rows)
 // and the FP32 recurrence state S (ld N).
-__global__ void split_y_kernel(int64_t N, int64_t Np, int64_t j0, const double2* __restrict__ Y,
+__global__ void split_y_kernel(int64_t N, int64_t Np, int64_t j0, int width,
+                               const double2* __restrict__ Y,
                                int64_t ldy, __nv_bfloat16* __restrict__ hi,
                                __nv_bfloat16* __restrict__ lo, float2* __restrict__ S) {
   const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
@@ -570,7 +596,7 @@ __global__ void split_y_kernel(int64_t N, int64_t Np, int64_t j0, const double2*
   split3(b.y, fb.y, bih, bil);
   S[k + j * N] = fa;
   if (two) S[k + 1 + j * N] = fb;
-  const int64_t ld = 2 * Np, re = brow_re(j) * ld + k, im = re + 128 * ld;
+  const int64_t ld = 2 * Np, re = brow_re(j, width) * ld + k, im = re + width * ld;
   auto put = [](__nv_bfloat16* p, unsigned v) { *reinterpret_cast<unsigned*>(p) = v; };
   const unsigned rh = bf_pair(arh, brh), rl = bf_pair(arl, brl);
   const unsigned ih = bf_pair(aih, bih), il = bf_pair(ail, bil);
@@ -624,18 +650,42 @@ bool make_map(CUtensorMap* m, void* base, int64_t rows, int64_t Np, int box_rows
 }
 
 struct Maps {
-  CUtensorMap ah, al, bh[2], bl[2];
+  CUtensorMap ah, al, bh[kNumWidths][2], bl[kNumWidths][2];  // operand boxes of every width
 };
+int width_index(int w) {
+  return (int)(std::find(kWidths, kWidths + kNumWidths, w) - kWidths);
+}
+// rows of an operand plane for ne columns in tiles of any width
+int64_t operand_rows(int64_t ne) { return 2 * (ne + kMaxWidth); }
+
+// Width of a filter's tiles: a wave of tiles takes as long as one, W plus the time to
+// fill and finish it (8 columns' worth), and narrow tiles are bound by their reads of
+// A (a width of 40 at least). A narrower tile has to promise a fifth: it is for
+// products of few tiles, 512 rows and 60 columns as 4 pairs of width 32 (20 us a step)
+// instead of 2 of width 128 with half of it padding (31 us). Where the chip is full
+// anyway, padding costs less than the extra tiles: 13379 rows and 1072 columns took
+// 59 to 61 ms in 6.3 waves of width 128 and 61.4 in 7.0 of width 112.
+int choose_width(int64_t N, int64_t ncols) {
+  const int64_t pairs = num_sms() / PAIR, rows = cdiv(N, PAIR * TM);
+  auto cost = [&](int64_t w) {
+    return cdiv(rows * cdiv(ncols, w), pairs) * (std::max<int64_t>(w, 40) + 8);
+  };
+  int best = kMaxWidth;
+  for (int i = 0; i < kNumWidths - 1; ++i)
+    if (10 * cost(kWidths[i]) <= 8 * cost(kMaxWidth) && cost(kWidths[i]) < cost(best))
+      best = kWidths[i];
+  return best;
+}
 
 }  // namespace
 
 // Layout of MixedWork: Ahi/Alo = N x 2Np planes; Yhi/Ylo = two B^T plane pairs
-// (ping-pong), each brows x 2Np with brows = 256 * ceil(ne / 128); maps after.
+// (ping-pong), each operand_rows(ne) x 2Np; maps after.
 cudaError_t mixed_alloc(MixedWork& w, int64_t N, int64_t ne) {
   w.N = N;
   w.ne = ne;
   const int64_t Np = cdiv(N, KPAD) * KPAD;
-  const int64_t brows = cdiv(ne, 128) * 256;
+  const int64_t brows = operand_rows(ne);
   const size_t a_bytes = (size_t)N * 2 * Np * sizeof(__nv_bfloat16);
   const size_t b_bytes = (size_t)brows * 2 * Np * sizeof(__nv_bfloat16);
   if (!get_encoder()) return cudaErrorNotSupported;
@@ -656,8 +706,9 @@ cudaError_t mixed_alloc(MixedWork& w, int64_t N, int64_t ne) {
   for (int b = 0; b < 2; ++b) {
     char* yh = static_cast<char*>(w.Yhi) + b * b_bytes;
     char* yl = static_cast<char*>(w.Ylo) + b * b_bytes;
-    ok = ok && make_map(&maps->bh[b], yh, brows, Np, B_HALF) &&
-         make_map(&maps->bl[b], yl, brows, Np, B_HALF);
+    for (int i = 0; i < kNumWidths; ++i)
+      ok = ok && make_map(&maps->bh[i][b], yh, brows, Np, kWidths[i]) &&
+           make_map(&maps->bl[i][b], yl, brows, Np, kWidths[i]);
   }
   if (!ok) return cudaErrorInvalidValue;
   if ((e = cudaMalloc(&w.S32, (size_t)2 * N * ne * sizeof(float2))) != cudaSuccess) return e;
@@ -681,22 +732,22 @@ void mixed_free(MixedWork& w) {
 namespace {
 // Operand planes of A and of Y_0 = V (into operand buffer 0 and FP32 state 0).
 void mixed_prologue(cudaStream_t s, int64_t N, const double2* A, int64_t lda, const double2* V,
-                    int64_t ldv, int64_t ncols, MixedWork& w) {
+                    int64_t ldv, int64_t ncols, int width, MixedWork& w) {
   const int64_t Np = cdiv(N, KPAD) * KPAD;
   split_a_kernel<<<dim3((unsigned)cdiv(N, SA_K), (unsigned)cdiv(N, 32), 1), dim3(32, 8, 1), 0, s>>>(
       N, Np, A, lda, static_cast<__nv_bfloat16*>(w.Ahi), static_cast<__nv_bfloat16*>(w.Alo));
   count_launch();
   split_y_kernel<<<dim3((unsigned)cdiv(N, 512), (unsigned)ncols, 1), 256, 0, s>>>(
-      N, Np, 0, V, ldv, static_cast<__nv_bfloat16*>(w.Yhi), static_cast<__nv_bfloat16*>(w.Ylo),
+      N, Np, 0, width, V, ldv, static_cast<__nv_bfloat16*>(w.Yhi), static_cast<__nv_bfloat16*>(w.Ylo),
       static_cast<float2*>(w.S32));
   count_launch();
 }
 
 // Parameters of filter step i (1-based) and the operand-plane buffer it reads.
 Params step_params(int64_t N, int64_t ncols, const int32_t* degs, double c, const double* al,
-                   const double* be, int i, int group, MixedWork& w, int* bin_out) {
+                   const double* be, int i, int width, int group, MixedWork& w, int* bin_out) {
   const int64_t Np = cdiv(N, KPAD) * KPAD;
-  const int64_t brows = cdiv(w.ne, 128) * 256;
+  const int64_t brows = operand_rows(w.ne);
   const size_t b_elems = (size_t)brows * 2 * Np;
   float2* st[2] = {static_cast<float2*>(w.S32), static_cast<float2*>(w.S32) + (size_t)N * w.ne};
   const int dmax = degs[ncols - 1];
@@ -716,7 +767,8 @@ Params step_params(int64_t N, int64_t ncols, const int32_t* degs, double c, cons
   P.Bn_lo = static_cast<__nv_bfloat16*>(w.Ylo) + bout * b_elems;
   P.write_next = i < dmax;
   P.nrow = (int)cdiv(N, PAIR * TM);
-  P.ncol = (int)((ncols - 1) / 128 - P.j0 / 128 + 1);
+  P.width = width;
+  P.ncol = (int)((ncols - 1) / width - P.j0 / width + 1);
   P.group = group;
   P.err = w.err;
   *bin_out = (i - 1) & 1;
@@ -760,7 +812,10 @@ int tuned_group(int64_t N, unsigned coltiles) {
 unsigned step_ctas(const Params& P) { return (unsigned)P.nrow * (unsigned)P.ncol * PAIR; }
 
 int tune_group(cudaStream_t s, const Maps* maps, Params P) {
+  // the order matters once several waves share the planes
+  if ((int64_t)P.nrow * P.ncol <= num_sms()) return kDefaultGroup;
   const int cached = tuned_group(P.N, (unsigned)P.ncol);
+  const int wi = width_index(P.width);
   if (cached) return cached;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
@@ -773,7 +828,8 @@ int tune_group(cudaStream_t s, const Maps* maps, Params P) {
       P.group = kGroupCandidates[i];
       cudaEventRecord(e0, s);
       mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al,
-                                                                     maps->bh[0], maps->bl[0], P);
+                                                                     maps->bh[wi][0],
+                                                                     maps->bl[wi][0], P);
       count_launch();
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) break;
@@ -819,16 +875,17 @@ int mixed_filter(cudaStream_t s, int64_t N, const double2* A, int64_t lda, doubl
   (void)W;
   (void)ldw;
   const Maps* maps = static_cast<const Maps*>(w.maps);
-  mixed_prologue(s, N, A, lda, V, ldv, ncols, w);
+  const int width = choose_width(N, ncols), wi = width_index(width);
+  mixed_prologue(s, N, A, lda, V, ldv, ncols, width, w);
   if (cudaMemsetAsync(w.err, 0, sizeof(int), s) != cudaSuccess) return CHASE_CUDA_FAIL();
   const int dmax = degs[ncols - 1];
   int group = kDefaultGroup;
   for (int i = 1; i <= dmax; ++i) {
     int bin = 0;
-    Params P = step_params(N, ncols, degs, c, al, be, i, group, w, &bin);
+    Params P = step_params(N, ncols, degs, c, al, be, i, width, group, w, &bin);
     if (i == 1 && autotune) P.group = group = tune_group(s, maps, P);
-    mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[bin],
-                                                                   maps->bl[bin], P);
+    mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[wi][bin],
+                                                                   maps->bl[wi][bin], P);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return CHASE_CUDA_FAIL();
   }
@@ -884,7 +941,8 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
   for (int k = 0; k < count; ++k) {
     const MixedGroupItem& it = items[k];
     if (it.ncols == 0) continue;
-    mixed_prologue(s, it.N, it.A, it.lda, it.V, it.ldv, it.ncols, *it.w);
+    mixed_prologue(s, it.N, it.A, it.lda, it.V, it.ldv, it.ncols, choose_width(it.N, it.ncols),
+                   *it.w);
     if (cudaMemsetAsync(it.w->err, 0, sizeof(int), s) != cudaSuccess) return CHASE_CUDA_FAIL();
   }
   GroupEntry* host = static_cast<GroupEntry*>(t.host);
@@ -898,15 +956,16 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
       const MixedGroupItem& it = items[k];
       if (it.ncols == 0 || it.degs[it.ncols - 1] < i) continue;
       const Maps* maps = static_cast<const Maps*>(it.w->maps);
-      const int g = tuned_group(it.N, (unsigned)((it.ncols - 1) / 128 + 1));
+      const int width = choose_width(it.N, it.ncols), wi = width_index(width);
+      const int g = tuned_group(it.N, (unsigned)((it.ncols - 1) / width + 1));
       int bin = 0;
       GroupEntry& e = host[n++];
-      e.P = step_params(it.N, it.ncols, it.degs, it.c, it.al, it.be, i,
+      e.P = step_params(it.N, it.ncols, it.degs, it.c, it.al, it.be, i, width,
                         g ? g : kDefaultGroup, *it.w, &bin);
       e.ah = maps->ah;
       e.al = maps->al;
-      e.bh = maps->bh[bin];
-      e.bl = maps->bl[bin];
+      e.bh = maps->bh[wi][bin];
+      e.bl = maps->bl[wi][bin];
       e.first = first;
       e.pad = 0;
       first += (int)step_ctas(e.P);
