@@ -1080,7 +1080,9 @@ struct Maps {
 // slowest. Tiles that fill the chip several times over stay whole; a product of
 // few tiles (the 8 of a 512 x 60 block, the 30 of a 316 x 316 Gram over 9273
 // rows) is cut so that its parts fill one wave. A cut has to gain a tenth: parts
-// read the right operand no less often and meet at two cluster barriers. It
+// read the right operand no less often and meet at two cluster barriers. Past five
+// waves there is nothing to even out (a 1072 x 1072 Gram over 13379 rows, 306 tiles: 8
+// parts a tile took 0.4 ms more than 2). It
 // depends on the product alone, so a problem's result is the same in a group.
 constexpr int kMaxSplit = 8;
 int choose_split(int64_t tiles, int64_t Np) {
@@ -1088,6 +1090,7 @@ int choose_split(int64_t tiles, int64_t Np) {
   int best = 1;
   double best_cost = 1e300;
   for (int s = 1; s <= kMaxSplit && 4 * s <= nkb; s *= 2) {  // at least half a chunk each
+    if (s > 1 && tiles * s > 5 * sms) break;
     const double cost = (double)cdiv(tiles * s, sms) *
                         ((double)cdiv(nkb, s) / CHUNK_KB + 1.0 + 1.5 / s);
     if (cost < 0.9 * best_cost) {
