@@ -197,7 +197,23 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
       "h"((uint16_t)3)
       : "memory");
 }
-// 16 consecutive TMEM columns of this warp's 32 lanes (no wait).
+// 32 (with the wait) or 16 consecutive TMEM columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+      "%28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -421,16 +437,26 @@ __device__ __forceinline__ void mixed_tile(const CUtensorMap* tmAh, const CUtens
       if (!go) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ta = tl + (uint32_t)(b * TN + h * HALF);
+      if constexpr (HALF >= 32) {
 #pragma unroll
-      for (int g = 0; g < HALF / 16; ++g) {
+        for (int half = 0; half < HALF / 32; ++half) {
+          float v[32];
+          tmem_ld32(ta + half * 32, v);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) sre[half * 32 + j] += v[j];
+          tmem_ld32(ta + W + half * 32, v);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) sim[half * 32 + j] += v[j];
+        }
+      } else {
         float v[16], u[16];
-        tmem_ld16(ta + g * 16, v);
-        tmem_ld16(ta + W + g * 16, u);
+        tmem_ld16(ta, v);
+        tmem_ld16(ta + W, u);
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          sre[g * 16 + j] += v[j];
-          sim[g * 16 + j] += u[j];
+          sre[j] += v[j];
+          sim[j] += u[j];
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -493,6 +519,7 @@ __device__ __forceinline__ void mixed_tile_of(const CUtensorMap* ah, const CUten
   }
 }
 
+template <int W>
 __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
     mixed_filter_kernel(const __grid_constant__ CUtensorMap tmAh,
                         const __grid_constant__ CUtensorMap tmAl,
@@ -500,7 +527,7 @@ __global__ void __cluster_dims__(PAIR, 1, 1) __launch_bounds__(NTHREADS, 1)
                         const __grid_constant__ CUtensorMap tmBl, Params P) {
   unsigned rp, ct;  // pair row and column tile of this pair (grouped raster order)
   grouped_tile(blockIdx.x / PAIR, (unsigned)P.nrow, (unsigned)P.ncol, P.group, rp, ct);
-  mixed_tile_of(&tmAh, &tmAl, &tmBh, &tmBl, P, rp, ct, false);
+  mixed_tile<W>(&tmAh, &tmAl, &tmBh, &tmBl, P, rp, ct, false);
 }
 
 // Many problems' filter steps in one launch: entry p of the table holds problem
@@ -658,23 +685,17 @@ int width_index(int w) {
 // rows of an operand plane for ne columns in tiles of any width
 int64_t operand_rows(int64_t ne) { return 2 * (ne + kMaxWidth); }
 
-// Width of a filter's tiles: a wave of tiles takes as long as one, W plus the time to
-// fill and finish it (8 columns' worth), and narrow tiles are bound by their reads of
-// A (a width of 40 at least). A narrower tile has to promise a fifth: it is for
-// products of few tiles, 512 rows and 60 columns as 4 pairs of width 32 (20 us a step)
-// instead of 2 of width 128 with half of it padding (31 us). Where the chip is full
-// anyway, padding costs less than the extra tiles: 13379 rows and 1072 columns took
-// 59 to 61 ms in 6.3 waves of width 128 and 61.4 in 7.0 of width 112.
+// Width of a filter's tiles: the narrowest at which all of them run in one wave. 512
+// rows and 60 columns are 4 pairs of width 32 (20 us a step) instead of 2 of width 128
+// with half of it padding (31 us), a filter with 3000 rows and 140 columns takes 1.02
+// instead of 1.34 ms. Where narrow tiles take more waves their extra reads of A cost
+// more than the padding: 6500 rows and 500 columns, 208 tiles of width 64 6.9 ms, 104
+// of width 128 5.6.
 int choose_width(int64_t N, int64_t ncols) {
   const int64_t pairs = num_sms() / PAIR, rows = cdiv(N, PAIR * TM);
-  auto cost = [&](int64_t w) {
-    return cdiv(rows * cdiv(ncols, w), pairs) * (std::max<int64_t>(w, 40) + 8);
-  };
-  int best = kMaxWidth;
-  for (int i = 0; i < kNumWidths - 1; ++i)
-    if (10 * cost(kWidths[i]) <= 8 * cost(kMaxWidth) && cost(kWidths[i]) < cost(best))
-      best = kWidths[i];
-  return best;
+  for (int w : kWidths)
+    if (rows * cdiv(ncols, w) <= pairs) return w;
+  return kMaxWidth;
 }
 
 }  // namespace
@@ -714,8 +735,11 @@ cudaError_t mixed_alloc(MixedWork& w, int64_t N, int64_t ne) {
   if ((e = cudaMalloc(&w.S32, (size_t)2 * N * ne * sizeof(float2))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.err, sizeof(int))) != cudaSuccess) return e;
   if ((e = cudaMemset(w.err, 0, sizeof(int))) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(mixed_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              SMEM_BYTES);
+  for (auto k : {mixed_filter_kernel<32>, mixed_filter_kernel<64>, mixed_filter_kernel<128>})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) !=
+        cudaSuccess)
+      return e;
+  return cudaSuccess;
 }
 
 void mixed_free(MixedWork& w) {
@@ -810,12 +834,20 @@ int tuned_group(int64_t N, unsigned coltiles) {
 }
 
 unsigned step_ctas(const Params& P) { return (unsigned)P.nrow * (unsigned)P.ncol * PAIR; }
+void launch_step(cudaStream_t s, const Maps* maps, int bin, const Params& P) {
+  const int wi = width_index(P.width);
+  auto* k = P.width == 32   ? mixed_filter_kernel<32>
+            : P.width == 64 ? mixed_filter_kernel<64>
+                            : mixed_filter_kernel<128>;
+  k<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[wi][bin],
+                                               maps->bl[wi][bin], P);
+  count_launch();
+}
 
 int tune_group(cudaStream_t s, const Maps* maps, Params P) {
   // the order matters once several waves share the planes
   if ((int64_t)P.nrow * P.ncol <= num_sms()) return kDefaultGroup;
   const int cached = tuned_group(P.N, (unsigned)P.ncol);
-  const int wi = width_index(P.width);
   if (cached) return cached;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
@@ -827,10 +859,7 @@ int tune_group(cudaStream_t s, const Maps* maps, Params P) {
     for (int i = 0; i < nc; ++i) {
       P.group = kGroupCandidates[i];
       cudaEventRecord(e0, s);
-      mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al,
-                                                                     maps->bh[wi][0],
-                                                                     maps->bl[wi][0], P);
-      count_launch();
+      launch_step(s, maps, 0, P);
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) break;
       float ms = 0.f;
@@ -875,7 +904,7 @@ int mixed_filter(cudaStream_t s, int64_t N, const double2* A, int64_t lda, doubl
   (void)W;
   (void)ldw;
   const Maps* maps = static_cast<const Maps*>(w.maps);
-  const int width = choose_width(N, ncols), wi = width_index(width);
+  const int width = choose_width(N, ncols);
   mixed_prologue(s, N, A, lda, V, ldv, ncols, width, w);
   if (cudaMemsetAsync(w.err, 0, sizeof(int), s) != cudaSuccess) return CHASE_CUDA_FAIL();
   const int dmax = degs[ncols - 1];
@@ -884,9 +913,7 @@ int mixed_filter(cudaStream_t s, int64_t N, const double2* A, int64_t lda, doubl
     int bin = 0;
     Params P = step_params(N, ncols, degs, c, al, be, i, width, group, w, &bin);
     if (i == 1 && autotune) P.group = group = tune_group(s, maps, P);
-    mixed_filter_kernel<<<step_ctas(P), NTHREADS, SMEM_BYTES, s>>>(maps->ah, maps->al, maps->bh[wi][bin],
-                                                                   maps->bl[wi][bin], P);
-    count_launch();
+    launch_step(s, maps, bin, P);
     if (cudaGetLastError() != cudaSuccess) return CHASE_CUDA_FAIL();
   }
   // even degrees: every column's final value is in state buffer 0
