@@ -7,7 +7,8 @@
 // fall on the 152 SMs. The tiles are therefore small, 16 x 16 with two warps of
 // 2 x 2 accumulators, up to a dozen CTAs on an SM: a 2600 x 195 x 2600 product
 // is 2119 tiles, 13.9 per SM, where 64 x 64 tiles were 164 CTAs, two on some SMs
-// and one on the others, with a quarter of the columns padding.
+// and one on the others, with a quarter of the columns padding (a filter of degree
+// up to 10 on it: 147.5 -> 67.6 ms).
 // Double-buffered shared memory; the epilogues fuse the Chebyshev three-term
 // update (Eq. 1), plain stores, and the per-column residual sums of squares
 // (Alg. 2 residual lines).
