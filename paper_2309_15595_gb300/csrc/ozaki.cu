@@ -1241,7 +1241,7 @@ namespace {
 // Launch that may begin while its predecessor in the stream still runs; the kernel
 // waits for it (wait_for_predecessor).
 template <typename... KArgs, typename... Args>
-void launch_early(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args... args) {
+cudaError_t launch_early(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
@@ -1252,22 +1252,23 @@ void launch_early(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   count_launch();
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);  // the caller checks
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
-// Digits of columns j0 .. j0 + n of B (K rows) into w.Bd (`brows` rows a plane).
+// Digits of columns j0 .. j0 + n of B (K rows) into w.Bd (`brows` rows a plane). A
+// product must not follow a refused launch: it would take the digits of another block.
 template <int NS>
-void slice_right(cudaStream_t s, int64_t K, int64_t j0, int64_t n, const double2* B, int64_t ldb,
+cudaError_t slice_right(cudaStream_t s, int64_t K, int64_t j0, int64_t n, const double2* B, int64_t ldb,
                  int64_t brows, OzakiWork& w) {
   __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w.Bd);
   const int64_t Kp = ozaki_np(K);
-  if (K <= kOnePass) {
-    launch_early(slice_b_column_kernel<NS>, dim3((unsigned)n, 1, 1), 256, s, K, Kp, brows, j0, B,
-                 ldb, w.eb, out);
-    return;
-  }
-  launch_early(colexp_kernel, dim3((unsigned)n, 1, 1), 256, s, K, j0, B, ldb, w.eb);
-  launch_early(slice_b_kernel<NS>, dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, s, K, Kp,
-               brows, j0, B, ldb, (const int*)w.eb, out);
+  if (K <= kOnePass)
+    return launch_early(slice_b_column_kernel<NS>, dim3((unsigned)n, 1, 1), 256, s, K, Kp, brows,
+                        j0, B, ldb, w.eb, out);
+  const cudaError_t e =
+      launch_early(colexp_kernel, dim3((unsigned)n, 1, 1), 256, s, K, j0, B, ldb, w.eb);
+  if (e != cudaSuccess) return e;
+  return launch_early(slice_b_kernel<NS>, dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, s, K,
+                      Kp, brows, j0, B, ldb, (const int*)w.eb, out);
 }
 
 }  // namespace
@@ -1277,7 +1278,8 @@ cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const doub
   const int64_t N = w.N;
   const int64_t n = ncols_end - j0;
   if (n <= 0) return cudaSuccess;
-  slice_right<OS>(s, N, j0, n, B, ldb, w.brows, w);
+  const cudaError_t e = slice_right<OS>(s, N, j0, n, B, ldb, w.brows, w);
+  if (e != cudaSuccess) return e;
   const Maps* maps = static_cast<const Maps*>(w.maps);
   const Params P = product_params(w, ncols_end, j0, B, ldb, ep);
   return launch_product(s, maps->a, maps->b, P, PAIRS_21);
@@ -1360,10 +1362,11 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
                                                                                    w.el, L);
       count_launch();
     }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else if ((e = slice_left<OS>(s, M, K, X, ldx, w)) != cudaSuccess) {  // left = X, M x K
     return e;
   }
-  slice_right<OS>(s, K, 0, ncols, B, ldb, w.brows, w);
+  if ((e = slice_right<OS>(s, K, 0, ncols, B, ldb, w.brows, w)) != cudaSuccess) return e;
   CUtensorMap ma, mb;
   if (!make_map(&ma, w.Ld, (int64_t)OS * M, Kp, TM) ||
       !make_map(&mb, w.Bd, (int64_t)OS * w.brows, Kp, TN))
@@ -1387,9 +1390,10 @@ cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2*
   if (M > w.N || Kp > ozaki_fine_inner(w, M)) return cudaErrorInvalidValue;
   cudaError_t e = clear_left(s, M, K, OS7, w);
   if (e != cudaSuccess || (e = slice_left<OS7>(s, M, K, X, ldx, w)) != cudaSuccess) return e;
-  // as many columns at a time as the right operand's planes hold, in whole tiles
+  // as many columns at a time as the right operand's planes hold, in whole tiles, and
+  // as a grid has rows
   const int64_t fit = OS * w.brows * w.Np / (OS7 * Kp) / TN * CT;
-  const int64_t block = std::min({ncols, fit, std::max(w.N, w.ne)});
+  const int64_t block = std::min({ncols, fit, std::max(w.N, w.ne), (int64_t)65535 / CT * CT});
   const int64_t brows = cdiv(block, CT) * TN;
   CUtensorMap ma, mb;
   if (!make_map(&ma, w.Ld, (int64_t)OS7 * M, Kp, TM) ||
@@ -1397,7 +1401,7 @@ cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2*
     return cudaErrorInvalidValue;
   for (int64_t c0 = 0; c0 < ncols; c0 += block) {
     const int64_t nc = std::min(block, ncols - c0);
-    slice_right<OS7>(s, K, 0, nc, B + c0 * ldb, ldb, brows, w);
+    if ((e = slice_right<OS7>(s, K, 0, nc, B + c0 * ldb, ldb, brows, w)) != cudaSuccess) return e;
     Epilogue ec = ep;
     if (ec.X) ec.X += c0 * ec.ldx;
     if (ec.Y) ec.Y += c0 * ec.ldy;
@@ -1563,15 +1567,20 @@ int ozaki_filter_grouped(cudaStream_t s, int count, const OzakiGroupItem* items,
     return CHASE_CUDA_FAIL();
   const OzGroupEntry* dev = static_cast<const OzGroupEntry*>(t.dev);
   const OzSliceEntry* sdev = static_cast<const OzSliceEntry*>(t.sdev);
-  for (int i = 1; i <= dmax_all; ++i) {
+  cudaError_t first = cudaSuccess;  // a graph without one of its steps is not launched
+  for (int i = 1; i <= dmax_all && first == cudaSuccess; ++i) {
     const int cnt = (int)(off[i + 1] - off[i]);
     slice_b_grouped_kernel<<<(unsigned)cols[i], 256, 0, s>>>(sdev + off[i], cnt);
     count_launch();
-    launch_clusters(ozaki_filter_grouped_kernel, (unsigned)ctas[i], cluster[i], false, s, dev + off[i], cnt,
-                    cluster[i] > 1);
+    if ((first = cudaGetLastError()) == cudaSuccess)
+      first = launch_clusters(ozaki_filter_grouped_kernel, (unsigned)ctas[i], cluster[i], false, s,
+                              dev + off[i], cnt, cluster[i] > 1);
   }
   const cudaError_t ce = cudaStreamEndCapture(s, &graph);
-  if (ce != cudaSuccess || !graph) return CHASE_CUDA_FAIL();
+  if (first != cudaSuccess || ce != cudaSuccess || !graph) {
+    if (ce == cudaSuccess && graph) cudaGraphDestroy(graph);
+    return CHASE_CUDA_FAIL();
+  }
   const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (ie != cudaSuccess) return CHASE_CUDA_FAIL();
