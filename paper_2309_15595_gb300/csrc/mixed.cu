@@ -920,6 +920,7 @@ int mixed_filter(cudaStream_t s, int64_t N, const double2* A, int64_t lda, doubl
   state_to_f64_kernel<<<dim3((unsigned)cdiv(N, 256), (unsigned)ncols, 1), 256, 0, s>>>(
       N, static_cast<const float2*>(w.S32), V, ldv);
   count_launch();
+  if (cudaGetLastError() != cudaSuccess) return CHASE_CUDA_FAIL();
   return check_err(s, w.err);
 }
 
@@ -970,7 +971,9 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
     if (it.ncols == 0) continue;
     mixed_prologue(s, it.N, it.A, it.lda, it.V, it.ldv, it.ncols, choose_width(it.N, it.ncols),
                    *it.w);
-    if (cudaMemsetAsync(it.w->err, 0, sizeof(int), s) != cudaSuccess) return CHASE_CUDA_FAIL();
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemsetAsync(it.w->err, 0, sizeof(int), s) != cudaSuccess)
+      return CHASE_CUDA_FAIL();
   }
   GroupEntry* host = static_cast<GroupEntry*>(t.host);
   std::vector<size_t> off(dmax_all + 2, 0);
@@ -1009,13 +1012,18 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
   if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
     return CHASE_CUDA_FAIL();
   const GroupEntry* dev = static_cast<const GroupEntry*>(t.dev);
-  for (int i = 1; i <= dmax_all; ++i) {
+  cudaError_t first = cudaSuccess;  // a graph without one of its steps is not launched
+  for (int i = 1; i <= dmax_all && first == cudaSuccess; ++i) {
     mixed_filter_grouped_kernel<<<(unsigned)ctas[i], NTHREADS, SMEM_BYTES, s>>>(
         dev + off[i], (int)(off[i + 1] - off[i]));
     count_launch();
+    first = cudaGetLastError();
   }
   const cudaError_t ce = cudaStreamEndCapture(s, &graph);
-  if (ce != cudaSuccess || !graph) return CHASE_CUDA_FAIL();
+  if (first != cudaSuccess || ce != cudaSuccess || !graph) {
+    if (ce == cudaSuccess && graph) cudaGraphDestroy(graph);
+    return CHASE_CUDA_FAIL();
+  }
   const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (ie != cudaSuccess) return CHASE_CUDA_FAIL();
@@ -1032,9 +1040,10 @@ int mixed_filter_grouped(cudaStream_t s, int count, const MixedGroupItem* items,
         it.N, static_cast<const float2*>(it.w->S32), it.V, it.ldv);
     count_launch();
   }
+  const cudaError_t ve = cudaGetLastError();
   const cudaError_t se = cudaStreamSynchronize(s);
   cudaGraphExecDestroy(exec);
-  if (se != cudaSuccess) return CHASE_CUDA_FAIL();
+  if (ve != cudaSuccess || se != cudaSuccess) return CHASE_CUDA_FAIL();
   for (int k = 0; k < count; ++k)
     if (items[k].ncols > 0) RC_M(check_err(s, items[k].w->err));
   return CHASE_OK;

@@ -70,13 +70,15 @@ class Problem:
 # 60 columns of 700 (digits of a column by one CTA) and of 1100 rows (two passes); in
 # both, the adjoints' N x N product runs on the tensor cores
 @pytest.mark.parametrize("N,ne", [(700, 60), (1100, 60)])
-@pytest.mark.parametrize("op", ["filter", "residuals", "rr", "qr1", "qr2", "filter_vjp", "eig_vjp"])
+@pytest.mark.parametrize("op", ["filter", "mixed", "residuals", "rr", "qr1", "qr2", "filter_vjp",
+                                "eig_vjp"])
 def test_refused_launch(fake, op, N, ne):
-    p = Problem(fake, N, ne, 1)
+    p = Problem(fake, N, ne, 1, int(op == "mixed"))
     L, c, A, V, B, d = p.lib, p.ctx, p.A, p.V, p.B, p.d
     degs = (ctypes.c_int32 * ne)(*([2] * (ne // 2) + [4] * (ne - ne // 2)))
     call = {
         "filter": lambda: L.chase_filter(c, A, N, V, N, ne, degs, 0.5, 1.0, -1.0, 0),
+        "mixed": lambda: L.chase_filter(c, A, N, V, N, ne, degs, 0.5, 1.0, -1.0, 1),
         "residuals": lambda: L.chase_residuals(c, A, N, V, N, d, ne, d),
         "rr": lambda: L.chase_rayleigh_ritz(c, A, N, V, N, ne, d),
         "qr1": lambda: L.chase_qr(c, V, N, ne, 10.0, None),
@@ -90,7 +92,7 @@ def test_refused_launch(fake, op, N, ne):
     p.close()
 
 
-@pytest.mark.parametrize("mixed", [0])
+@pytest.mark.parametrize("mixed", [0, 1])
 def test_refused_launch_in_a_batch(fake, mixed):
     # two worker threads: an error left behind by the grouped filter's thread is not theirs
     probs = [Problem(fake, N, ne, 1, mixed) for N, ne in ((300, 20), (200, 12))]
