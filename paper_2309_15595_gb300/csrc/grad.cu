@@ -242,7 +242,8 @@ int filter_step(chase_ctx* c, const double2* A, int64_t lda, const double2* X, i
 // cores, whose FP64 rate bounds it, 0.8 ms from seven digits; N = 2048, K = 64: 1.7
 // ms there. Seven digits keep the product's error at FP64's: with six, 2^-49 of the
 // row and column maxima, the filter adjoint's error against 64 bits grew by up to 1 %
-// and the eigenpair adjoint's by 7 %.
+// and the eigenpair adjoint's by 7 %. Operands with an infinity or NaN, which have no
+// digits, take the CUDA cores, where they reach Y.
 int outer_product(chase_ctx* c, int64_t K, const double2* Z, const double2* W, int64_t ldw,
                   double beta, double2* Y, int64_t ldy) {
   const int64_t N = c->N;
@@ -260,14 +261,17 @@ int outer_product(chase_ctx* c, int64_t K, const double2* Z, const double2* W, i
     CK(zgemm_nn(c->stream, N, N, K, Z, N, W, ldw, ep));
     return CHASE_OK;
   }
+  CK(ozaki_fine_begin(c->stream, N, K, Z, N, N, W, ldw, c->ow));
+  Epilogue part = ep;
   for (int64_t k0 = 0; k0 < K; k0 += most) {
-    if (k0 > 0) {  // later parts add to the first
-      ep.mode = EPI_FILTER;
-      ep.beta = 1.0;
-    }
-    CK(ozaki_gemm_fine(c->stream, N, std::min(most, K - k0), Z + k0 * N, N, N, W + k0, ldw, ep,
+    CK(ozaki_gemm_fine(c->stream, N, std::min(most, K - k0), Z + k0 * N, N, N, W + k0, ldw, part,
                        c->ow));
+    part.mode = EPI_FILTER;  // later parts add to the first
+    part.beta = 1.0;
   }
+  bool formed = false;
+  CK(ozaki_fine_end(c->stream, c->ow, &formed));
+  if (!formed) CK(zgemm_nn(c->stream, N, N, K, Z, N, W, ldw, ep));
   return CHASE_OK;
 }
 

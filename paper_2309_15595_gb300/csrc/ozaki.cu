@@ -260,6 +260,7 @@ struct Params {
   const double* theta;        // resid
   double* partial;            // resid: [32-row tile + col * ceil(N / 32)]
   int* err;
+  const int* skip;            // seven digits: the product is not formed where this is set
   int nrow, ncol;             // tiles
   int split;                  // CTAs that share a tile's K range
 };
@@ -694,6 +695,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       Params P) {
   let_successor_start();
+  if constexpr (NS == OS7) {
+    wait_for_predecessor();
+    if (*P.skip) return;  // the same in every CTA
+  }
   ozaki_tile<LMAX, NS>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
 }
 
@@ -864,6 +869,23 @@ __global__ void __launch_bounds__(256)
       *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
     }
   }
+}
+
+// *bad = 1 where an operand of the seven-digit product X B (X: M x K, B: K x n) holds an
+// infinity or NaN, which digits cannot carry: one CTA per k, column k of X and row k of
+// B. X and B are read once more for it: 20 us for M = n = 1500, K = 480.
+__global__ void __launch_bounds__(256)
+    finite_kernel(int64_t M, int64_t n, const double2* __restrict__ X, int64_t ldx,
+                  const double2* __restrict__ B, int64_t ldb, int* __restrict__ bad) {
+  const int64_t k = blockIdx.x;
+  bool ok = true;
+  auto look = [&](double2 v) {
+    ok = ok && (__double2hiint(v.x) & 0x7ff00000) != 0x7ff00000 &&
+         (__double2hiint(v.y) & 0x7ff00000) != 0x7ff00000;
+  };
+  for (int64_t i = threadIdx.x; i < M; i += 256) look(X[i + k * ldx]);
+  for (int64_t j = threadIdx.x; j < n; j += 256) look(B[k + j * ldb]);
+  if (!ok) *bad = 1;
 }
 
 // X (M x K, column-major) <- the value its six digits represent when X is the
@@ -1166,6 +1188,7 @@ Params product_params(const OzakiWork& w, int64_t ncols_end, int64_t j0, const d
   P.theta = ep.theta;
   P.partial = ep.partial;
   P.err = w.err;
+  P.skip = w.bad;
   set_tiles(P);
   return P;
 }
@@ -1191,8 +1214,9 @@ cudaError_t ozaki_alloc(OzakiWork& w, int64_t N, int64_t ne) {
   if ((e = cudaMalloc(&w.eb, std::max(N, ne) * sizeof(int))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.amax, N * sizeof(unsigned long long))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.diag, N * sizeof(double2))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&w.err, sizeof(int))) != cudaSuccess) return e;
-  if ((e = cudaMemset(w.err, 0, sizeof(int))) != cudaSuccess) return e;
+  if ((e = cudaMalloc(&w.err, 2 * sizeof(int))) != cudaSuccess) return e;
+  if ((e = cudaMemset(w.err, 0, 2 * sizeof(int))) != cudaSuccess) return e;
+  w.bad = w.err + 1;
   // general left operands of the N x n^2 products: X^H (ne x N) or Q (N x ne)
   const int64_t npe = ozaki_np(ne);
   w.l_elems = (size_t)OS7 * std::max((size_t)ne * 2 * w.Np, (size_t)N * 2 * npe);
@@ -1337,6 +1361,7 @@ Params general_params(int64_t M, int64_t K, int64_t ncols, const double2* B, int
   P.theta = ep.theta;
   P.partial = ep.partial;
   P.err = w.err;
+  P.skip = w.bad;
   set_tiles(P);
   return P;
 }
@@ -1380,6 +1405,25 @@ int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M) {
   // one column tile of the right operand has to fit too
   const int64_t right = OS * w.brows * w.Np / (OS7 * TN) / KPAD * KPAD;
   return std::min(left, right);
+}
+
+cudaError_t ozaki_fine_begin(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
+                             int64_t ncols, const double2* B, int64_t ldb, OzakiWork& w) {
+  const cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int), s);
+  if (e != cudaSuccess || M <= 0 || ncols <= 0 || K <= 0) return e;
+  finite_kernel<<<(unsigned)K, 256, 0, s>>>(M, ncols, X, ldx, B, ldb, w.bad);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t ozaki_fine_end(cudaStream_t s, const OzakiWork& w, bool* formed) {
+  int bad = 0;
+  const cudaError_t e = cudaMemcpyAsync(&bad, w.bad, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e != cudaSuccess) return e;
+  *formed = false;
+  const cudaError_t se = cudaStreamSynchronize(s);
+  if (se == cudaSuccess) *formed = bad == 0;
+  return se;
 }
 
 cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,

@@ -21,6 +21,7 @@ struct OzakiWork {
   int* el = nullptr;            // row exponents of the general left operand
   int64_t l_M = 0, l_K = 0;     // layout of the planes in Ld (0: not yet written)
   int l_ns = 0;
+  int* bad = nullptr;           // device: an operand of the seven-digit product is not finite
   int64_t N = 0, ne = 0, Np = 0, brows = 0;
 };
 
@@ -46,11 +47,17 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
                                bool extended = false);
 // P = X * B (M x K times K x ncols, any ncols) from seven digits of each operand, 28
 // digit pairs: an error of about sqrt(2K) 2^-57 of the row and column maxima, which
-// is FP64's. ep: EPI_STORE or EPI_FILTER. K at most ozaki_fine_inner, which is at
-// least ne for M = N.
+// is FP64's. ep: EPI_STORE or EPI_FILTER. K at most ozaki_fine_inner. Several parts of K
+// may follow an ozaki_fine_begin over all of X and B, which looks for infinities and
+// NaN: where there are any, the parts leave Y as it is, ozaki_fine_end (which
+// synchronises s) says so, and the caller forms the product in FP64.
+cudaError_t ozaki_fine_begin(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
+                             int64_t ncols, const double2* B, int64_t ldb, OzakiWork& w);
+cudaError_t ozaki_fine_end(cudaStream_t s, const OzakiWork& w, bool* formed);
 cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
                             int64_t ncols, const double2* B, int64_t ldb, const Epilogue& ep,
                             OzakiWork& w);
+// Largest K that the planes of w have room for (0: none).
 int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M);
 // X (M x K, column-major, M <= N) <- the digits it has as the left
 // operand of ozaki_gemm_general (rows scaled by powers of two, six digits), so
