@@ -24,7 +24,7 @@ constexpr int MT = 2;        // accumulators per thread and direction
 constexpr int BM = 16;       // rows of a tile
 constexpr int RESID_BM = 64;  // rows of a tile of the residual epilogue: one partial each
 constexpr int threads_of(int bm) { return bm / MT * (BN / MT); }
-constexpr int kMaxSplits = 8;
+constexpr int kMinSplits = 8;
 constexpr size_t kMinGramWs = (size_t)1 << 19;  // room for many splits of a small product
 
 // A operand: normal (M x K column-major) or conjugate-transpose of a K x M
@@ -339,7 +339,7 @@ cudaError_t resid_reduce(cudaStream_t s, const double* partial, int64_t ntiles, 
 }
 
 size_t gram_workspace_elems(int64_t m, int64_t n) {
-  return std::max((size_t)kMaxSplits * m * n, kMinGramWs);
+  return std::max((size_t)kMinSplits * m * n, kMinGramWs);
 }
 
 cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2* X, int64_t ldx,
@@ -349,20 +349,24 @@ cudaError_t zgram(cudaStream_t s, int64_t K, int64_t m, int64_t n, const double2
   if (ws_elems < (size_t)m * n) return cudaErrorInvalidValue;  // no room for one partial
   const int64_t tm = cdiv(m, BM), tn = cdiv(n, BN);
   const int64_t tiles = hermitian ? tm * (tm + 1) / 2 : tm * tn;
-  // split-K factor: the one (up to the workspace and K / 64) for which the most
-  // loaded SM has the fewest k steps, a tile counting 16 more for its start and
+  // split-K factor: the one (from kMinSplits or parts of 512 up to the workspace and
+  // K / 64) for which the most loaded SM has the fewest k steps, a tile counting 16 more for its start and
   // its partial. A tile has two warps, so one CTA on an SM drives half of its FP64
   // pipe and shows all its latencies: fewer than three CTAs an SM count more (a
-  // 64 x 64 Gram over 2048 rows, 16 tiles: split 9 ways 142 us); ties to fewer splits
+  // 64 x 64 Gram over 2048 rows, 16 tiles: split 9 ways 142 us); ties to fewer splits.
+  // The lower end is for the rounding, which grows with the length of a part: against
+  // 100 bits, Rayleigh-Ritz with 2600 rows and 400 columns was 18 % further off with
+  // the two parts that spread best than with five. A part more costs a partial.
   const int64_t sms = num_sms();
   const int64_t smax = std::max<int64_t>(
       1, std::min<int64_t>(K / 64, (int64_t)(ws_elems / ((size_t)m * n))));
-  int64_t splits = 1;
+  const int64_t smin = std::min<int64_t>({(int64_t)kMinSplits, std::max<int64_t>(1, K / 512), smax});
+  int64_t splits = smin;
   double best = 0.0;
-  for (int64_t sp = 1; sp <= smax && tiles * (sp - 1) < 8 * sms; ++sp) {
+  for (int64_t sp = smin; sp <= smax && (sp == smin || tiles * (sp - 1) < 8 * sms); ++sp) {
     const int64_t r = cdiv(tiles * sp, sms);
     const double load = (double)(r * (cdiv(K, sp) + 16)) * (r >= 3 ? 1.0 : r == 2 ? 1.2 : 2.2);
-    if (sp == 1 || load < best) {
+    if (sp == smin || load < best) {
       best = load;
       splits = sp;
     }
