@@ -240,12 +240,14 @@ int filter_step(chase_ctx* c, const double2* A, int64_t lda, const double2* X, i
 // Y = beta Y + Z W (beta 0 or 1) for Z (N x K, ld N) and W (K x N, ld ldw), on the
 // tensor cores from 0.2 ms of CUDA-core work on. N = 1500, K = 480: 7.2 ms on the CUDA
 // cores, whose FP64 rate bounds it, 0.8 ms from seven digits; N = 2048, K = 64: 1.7
-// ms there. Seven digits keep the product's error at FP64's: with six, 2^-49 of the
-// row and column maxima, the filter adjoint's error against 64 bits grew by up to 1 %
-// and the eigenpair adjoint's by 7 %. Operands with an infinity or NaN, which have no
-// digits, take the CUDA cores, where they reach Y.
+// ms there. Seven digits, cut after z_k and w_k have been brought to one size, keep the
+// product's error below FP64's: with six, 2^-49 of the row and column maxima, the filter
+// adjoint's error against 64 bits grew by up to 1 % and the eigenpair adjoint's by 7 %,
+// and without the balance it grew with the spread of the columns (see ozaki.cu).
+// Operands with an infinity or NaN, which have no digits, take the CUDA cores, where
+// they reach Y. kexp: K ints of device scratch.
 int outer_product(chase_ctx* c, int64_t K, const double2* Z, const double2* W, int64_t ldw,
-                  double beta, double2* Y, int64_t ldy) {
+                  double beta, double2* Y, int64_t ldy, int* kexp) {
   const int64_t N = c->N;
   Epilogue ep{};
   ep.mode = beta != 0.0 ? EPI_FILTER : EPI_STORE;
@@ -261,11 +263,11 @@ int outer_product(chase_ctx* c, int64_t K, const double2* Z, const double2* W, i
     CK(zgemm_nn(c->stream, N, N, K, Z, N, W, ldw, ep));
     return CHASE_OK;
   }
-  CK(ozaki_fine_begin(c->stream, N, K, Z, N, N, W, ldw, c->ow));
+  CK(ozaki_fine_begin(c->stream, N, K, Z, N, N, W, ldw, kexp, c->ow));
   Epilogue part = ep;
   for (int64_t k0 = 0; k0 < K; k0 += most) {
-    CK(ozaki_gemm_fine(c->stream, N, std::min(most, K - k0), Z + k0 * N, N, N, W + k0, ldw, part,
-                       c->ow));
+    CK(ozaki_gemm_fine(c->stream, N, std::min(most, K - k0), Z + k0 * N, N, N, W + k0, ldw,
+                       kexp + k0, part, c->ow));
     part.mode = EPI_FILTER;  // later parts add to the first
     part.beta = 1.0;
   }
@@ -315,13 +317,14 @@ extern "C" int chase_filter_vjp(chase_ctx* c, const chase_c128* Ac, int64_t lda,
   // Z_{ks..ks+seg+1}, and the scaled conjugate transpose of the segment states
   const size_t blk = (size_t)N * n;
   const size_t nblk = 2 * (size_t)nseg + seg + (seg + 2) + seg;
-  RC(ensure_workspace(c, nblk * blk, (size_t)seg + 8));
+  RC(ensure_workspace(c, nblk * blk, (size_t)seg + 8 + cdiv(seg * n, 2)));
   double2* ck_cur = c->gw;
   double2* ck_prev = ck_cur + nseg * blk;
   double2* yseg = ck_prev + nseg * blk;
   double2* zseg = yseg + seg * blk;
   double2* wt = zseg + (seg + 2) * blk;  // (seg n) x N, ld seg n
   double* dscale = c->gd;
+  int* kexp = reinterpret_cast<int*>(c->gd + seg + 8);  // seg n powers of two
   RC(ctx_prepare_a(c, A, lda));
 
   // forward sweep, keeping only the checkpoints: ping-pong in yseg[0], yseg[1]
@@ -381,7 +384,7 @@ extern "C" int chase_filter_vjp(chase_ctx* c, const chase_c128* Ac, int64_t lda,
                             0, s>>>(N, K, yseg, N, dscale, n, wt, K);
     count_launch();
     CK(cudaGetLastError());
-    RC(outer_product(c, K, zseg + blk, wt, K, 1.0, Ab, ldab));
+    RC(outer_product(c, K, zseg + blk, wt, K, 1.0, Ab, ldab, kexp));
     // the host copy of the scales must outlive the enqueued copy
     CK(cudaStreamSynchronize(s));
     // carry Z_{i0}, Z_{i0+1} to the next (earlier) segment's top slots
@@ -413,7 +416,7 @@ extern "C" int chase_eig_vjp(chase_ctx* c, const chase_c128* Ac, int64_t lda,
   cudaStream_t s = c->stream;
   const int64_t nx = ne - nev;  // extra Ritz vectors: initial guess of the complement solves
   const size_t blk = (size_t)N * nev;
-  RC(ensure_workspace(c, 5 * blk, 7 * (size_t)nev + 8));
+  RC(ensure_workspace(c, 5 * blk, 8 * (size_t)nev + 8));
   double2* Z = c->gw;
   double2* R = Z + blk;
   double2* P = R + blk;
@@ -550,7 +553,8 @@ extern "C" int chase_eig_vjp(chase_ctx* c, const chase_c128* Ac, int64_t lda,
   conj_transpose_kernel<<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(nev, 32), 1), dim3(32, 8, 1),
                           0, s>>>(N, nev, X, ldx, nullptr, 1, XwH, nev);
   count_launch();
-  RC(outer_product(c, nev, M, XwH, nev, 0.0, Ab, ldab));
+  RC(outer_product(c, nev, M, XwH, nev, 0.0, Ab, ldab,
+                   reinterpret_cast<int*>(d + 7 * nev)));
   CK(hermitian_part(s, N, Ab, ldab));
   RC(finish(c));
   if (cg_iters) *cg_iters = iters;

@@ -391,8 +391,6 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   const int64_t tile = P.j0 / CT + ct;            // absolute CT-column tile
   const int nkb_all = (int)((2 * P.Np) / TK);
   const int kb0 = (int)part * nkb_all / P.split;  // this CTA's K blocks, its chunks from there
-  const int nkb = ((int)part + 1) * nkb_all / P.split - kb0;
-  const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -417,7 +415,10 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   const uint32_t tmem = *tmem_slot;
   wait_for_predecessor();
 
-  bool go = true;
+  // a product that is not to be formed (the same in every CTA) has no K blocks
+  bool go = NS != OS7 || *P.skip == 0;
+  const int nkb = go ? ((int)part + 1) * nkb_all / P.split - kb0 : 0;
+  const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
   if (warp == 0) {
     if (lane == 0) {  // ------------------------------------ TMA producer
       if (maps_in_global) {  // tensor maps read from global memory by the TMA unit
@@ -695,10 +696,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       Params P) {
   let_successor_start();
-  if constexpr (NS == OS7) {
-    wait_for_predecessor();
-    if (*P.skip) return;  // the same in every CTA
-  }
   ozaki_tile<LMAX, NS>(&tmA, &tmB, P, blockIdx.x, false, P.split > 1);
 }
 
@@ -747,7 +744,8 @@ __device__ __forceinline__ long long fixed(double x, int e) {  // rint(x 2^(BITS
   const int E = (int)(b >> 52) & 0x7ff;
   const long long m = (b & 0xfffffffffffffll) | (E ? 1ll << 52 : 0);
   const int sh = 1075 - BITS - (E ? E : 1) + e;
-  if (E == 0x7ff || sh < 48 - BITS - 2) return __double2ll_rn(ldexp(x * ldexp(1.0, -e), BITS));
+  if (E == 0x7ff || sh < 48 - BITS - 2)  // a zero whose row or column has a tiny scale, or no number
+    return m == 0 ? 0 : __double2ll_rn(ldexp(x * ldexp(1.0, -e), BITS));
   if (sh > 53) return 0;
   if (sh < 1) return b < 0 ? -(m << -sh) : m << -sh;  // more bits than x has
   const long long X = (m + (1ll << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh;
@@ -802,6 +800,75 @@ __device__ __forceinline__ int exp_of_bits(unsigned long long b) {
   return f - 1021;
 }
 
+// The seven-digit product X B moves a power of two 2^t_k from column k of X to row k of
+// B before the digits are cut, so that their largest entries are of one size: the
+// digits' error follows max_k |x_ik| max_k |b_kj|, and FP64's, which it must not exceed,
+// sum_k |x_ik| |b_kj|. (Columns graded over 2, 8 and 16 decades on one side and their
+// inverse on the other cost 6e-16, 3e-10 and 3e-2 of Abar.) No entry is touched: t_k
+// only enters the exponents. A k whose column or row is zero is dropped, lest the other
+// side set the scales.
+constexpr int kDrop = 1 << 20;    // t_k of a dropped k: the exponents put its digits at zero
+constexpr int kNoExp = -100000;   // exponent of zero
+// E with 2^(E - 1) <= x < 2^E for x > 0 given by its bit pattern
+__device__ __forceinline__ int bin_exp(unsigned long long b) {
+  const int f = (int)(b >> 52);
+  return f != 0 ? f - 1022 : b != 0 ? 64 - 1074 - __clzll((long long)b) : kNoExp;
+}
+__device__ __forceinline__ int bin_exp(double2 a) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a.x) & ~(1ull << 63);
+  const unsigned long long y = (unsigned long long)__double_as_longlong(a.y) & ~(1ull << 63);
+  return bin_exp(x > y ? x : y);  // 1025 for an infinity or NaN
+}
+// exponent to cut an entry of X (SIGN 1) or B (-1) with, in a row or column of scale e
+template <int SIGN>
+__device__ __forceinline__ int cut_exp(int e, int t) {
+  return e + (t == kDrop ? kDrop : SIGN * t);
+}
+__device__ __forceinline__ int block_max(int m, int* red) {  // 256 threads
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = max(m, red[w]);
+  return m;
+}
+
+// t_k (kexp), one CTA per k, and *bad = 1 where an entry is an infinity or NaN, which
+// digits cannot carry. X (M x K) and B (K x n) are read once more for it: 7 us for M = n =
+// 1500, K = 480.
+__global__ void __launch_bounds__(256)
+    balance_kernel(int64_t M, int64_t n, const double2* __restrict__ X, int64_t ldx,
+                   const double2* __restrict__ B, int64_t ldb, int* __restrict__ kexp,
+                   int* __restrict__ bad) {
+  __shared__ int red[2][8];
+  const int64_t k = blockIdx.x;
+  int x = kNoExp, b = kNoExp;
+  for (int64_t i = threadIdx.x; i < M; i += 256) x = max(x, bin_exp(X[i + k * ldx]));
+  for (int64_t j = threadIdx.x; j < n; j += 256) b = max(b, bin_exp(B[k + j * ldb]));
+  x = block_max(x, red[0]);
+  b = block_max(b, red[1]);
+  if (threadIdx.x != 0) return;
+  kexp[k] = x == kNoExp || b == kNoExp ? kDrop : (x - b) >> 1;
+  if (max(x, b) > 1024) *bad = 1;
+}
+// Scales of the rows of X (M x K): ea[i] = the largest exponent of X_ik 2^-t_k, plus one.
+// ea starts far below every exponent. kRowK columns a CTA: K is a few hundred here, and
+// a chain of 128 columns in 6 CTAs took 40 us for 1500 rows.
+constexpr int kRowK = 16;
+__global__ void row_scale_kernel(int64_t M, int64_t K, const double2* __restrict__ X, int64_t ldx,
+                                 const int* __restrict__ kexp, int* __restrict__ ea) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= M) return;
+  const int64_t k0 = (int64_t)blockIdx.y * kRowK, k1 = min(K, k0 + kRowK);
+  int m = kNoExp;
+#pragma unroll 8
+  for (int64_t k = k0; k < k1; ++k) {
+    const int t = kexp[k];
+    if (t != kDrop) m = max(m, bin_exp(X[i + k * ldx]) - t);
+  }
+  atomicMax(&ea[i], max(m + 1, kNoExp));
+}
+
 // Row maxima of A (column-major): amax[i] = max_k max(|Re A_ik|, |Im A_ik|),
 // as the bit pattern of a non-negative double (monotone in unsigned order).
 __global__ void rowmax_kernel(int64_t M, int64_t K, bool skip_diag, const double2* __restrict__ A,
@@ -830,16 +897,16 @@ __global__ void exps_kernel(int64_t n, const unsigned long long* __restrict__ mx
 }
 
 // A (M x K, column-major) -> OS digit planes, each M rows x 2 Np (row-major
-// [Ar | Ai]), stacked, and the rows' exponents from their maxima; skip_diag leaves the
-// diagonal out (square A). A warp
+// [Ar | Ai]), stacked, and the rows' exponents from their maxima (of seven digits: ea
+// holds them, kexp the columns' own); skip_diag leaves the diagonal out (square A). A warp
 // writes a row of 64 entries, two per lane: 128 bytes of each of its 12 rows.
 constexpr int SA_K = 64;
 template <int NS>
 __global__ void __launch_bounds__(256)
     slice_a_kernel(int64_t M, int64_t K, int64_t Np, bool skip_diag,
                    const double2* __restrict__ A, int64_t lda,
-                   const unsigned long long* __restrict__ amax, int* __restrict__ ea,
-                   __nv_bfloat16* __restrict__ out) {
+                   const unsigned long long* __restrict__ amax, const int* __restrict__ kexp,
+                   int* __restrict__ ea, __nv_bfloat16* __restrict__ out) {
   __shared__ double2 tile[SA_K][33];
   const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * SA_K;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -854,14 +921,25 @@ __global__ void __launch_bounds__(256)
   const size_t plane = (size_t)M * ld;
   const int64_t k = k0 + 2 * tx;  // k + 1 may be K: the padding's digits are zero
   if (k >= K) return;
+  int t0 = 0, t1 = 0;
+  if constexpr (NS == OS7) {
+    t0 = kexp[k];
+    t1 = k + 1 < K ? kexp[k + 1] : 0;
+  }
   for (int r = ty; r < 32; r += 8) {
     const int64_t i = i0 + r;
     if (i >= M) continue;
     const double2 a0 = tile[2 * tx][r], a1 = tile[2 * tx + 1][r];
-    const int e = exp_of_bits(amax[i]);
-    if (k0 == 0 && tx == 0) ea[i] = e;
-    const Digits<NS> r0 = digits_of<NS>(a0.x, e), r1 = digits_of<NS>(a1.x, e);
-    const Digits<NS> c0 = digits_of<NS>(a0.y, e), c1 = digits_of<NS>(a1.y, e);
+    int e0, e1;
+    if constexpr (NS == OS7) {
+      e0 = cut_exp<1>(ea[i], t0);
+      e1 = cut_exp<1>(ea[i], t1);
+    } else {
+      e0 = e1 = exp_of_bits(amax[i]);
+      if (k0 == 0 && tx == 0) ea[i] = e0;
+    }
+    const Digits<NS> r0 = digits_of<NS>(a0.x, e0), r1 = digits_of<NS>(a1.x, e1);
+    const Digits<NS> c0 = digits_of<NS>(a0.y, e0), c1 = digits_of<NS>(a1.y, e1);
     __nv_bfloat16* o = out + i * ld + k;
 #pragma unroll
     for (int d = 0; d < NS; ++d) {
@@ -869,23 +947,6 @@ __global__ void __launch_bounds__(256)
       *reinterpret_cast<unsigned*>(o + d * plane + Np) = pack_digits(c0.d[d], c1.d[d]);
     }
   }
-}
-
-// *bad = 1 where an operand of the seven-digit product X B (X: M x K, B: K x n) holds an
-// infinity or NaN, which digits cannot carry: one CTA per k, column k of X and row k of
-// B. X and B are read once more for it: 20 us for M = n = 1500, K = 480.
-__global__ void __launch_bounds__(256)
-    finite_kernel(int64_t M, int64_t n, const double2* __restrict__ X, int64_t ldx,
-                  const double2* __restrict__ B, int64_t ldb, int* __restrict__ bad) {
-  const int64_t k = blockIdx.x;
-  bool ok = true;
-  auto look = [&](double2 v) {
-    ok = ok && (__double2hiint(v.x) & 0x7ff00000) != 0x7ff00000 &&
-         (__double2hiint(v.y) & 0x7ff00000) != 0x7ff00000;
-  };
-  for (int64_t i = threadIdx.x; i < M; i += 256) look(X[i + k * ldx]);
-  for (int64_t j = threadIdx.x; j < n; j += 256) look(B[k + j * ldb]);
-  if (!ok) *bad = 1;
 }
 
 // X (M x K, column-major) <- the value its six digits represent when X is the
@@ -948,15 +1009,34 @@ __device__ __forceinline__ unsigned long long column_max(int64_t N, const double
   for (int64_t k = threadIdx.x; k < N; k += 256) m = max_bits(m, Y[k]);
   return block_max_bits(m, red);
 }
+// Scale of a column of the right operand: the exponent of its maximum, plus one; with
+// seven digits of its entries times 2^t_k.
+template <int NS>
+__device__ __forceinline__ int column_scale(int64_t N, const double2* __restrict__ Y,
+                                            const int* __restrict__ kexp,
+                                            unsigned long long* red) {
+  if constexpr (NS == OS) {
+    return scale_exp(__longlong_as_double((long long)column_max(N, Y, red)));
+  } else {
+    int m = kNoExp;
+#pragma unroll 4
+    for (int64_t k = threadIdx.x; k < N; k += 256) {
+      const int t = kexp[k];
+      if (t != kDrop) m = max(m, bin_exp(Y[k]) + t);
+    }
+    return max(block_max(m, reinterpret_cast<int*>(red)) + 1, kNoExp);
+  }
+}
+template <int NS>
 __global__ void __launch_bounds__(256)
     colexp_kernel(int64_t N, int64_t j0, const double2* __restrict__ Y, int64_t ldy,
-                  int* __restrict__ eb) {
+                  const int* __restrict__ kexp, int* __restrict__ eb) {
   __shared__ unsigned long long red[8];
   const int64_t j = j0 + blockIdx.x;
   let_successor_start();
   wait_for_predecessor();
-  const unsigned long long m = column_max(N, Y + j * ldy, red);
-  if (threadIdx.x == 0) eb[j] = scale_exp(__longlong_as_double((long long)m));
+  const int e = column_scale<NS>(N, Y + j * ldy, kexp, red);
+  if (threadIdx.x == 0) eb[j] = e;
 }
 
 // Digits of entries k, k + 1 (zero past N) of one column of the right operand
@@ -964,12 +1044,18 @@ __global__ void __launch_bounds__(256)
 template <int NS>
 __device__ __forceinline__ void slice_b_pair(int64_t N, int64_t Np, size_t plane, int64_t k,
                                              const double2* __restrict__ Y, int e,
+                                             const int* __restrict__ kexp,
                                              __nv_bfloat16* __restrict__ re,
                                              __nv_bfloat16* __restrict__ im) {
   const double2 y0 = Y[k];
   const double2 y1 = k + 1 < N ? Y[k + 1] : make_double2(0.0, 0.0);
-  const Digits<NS> r0 = digits_of<NS>(y0.x, e), r1 = digits_of<NS>(y1.x, e);
-  const Digits<NS> c0 = digits_of<NS>(y0.y, e), c1 = digits_of<NS>(y1.y, e);
+  int e0 = e, e1 = e;
+  if constexpr (NS == OS7) {
+    e0 = cut_exp<-1>(e, kexp[k]);
+    if (k + 1 < N) e1 = cut_exp<-1>(e, kexp[k + 1]);
+  }
+  const Digits<NS> r0 = digits_of<NS>(y0.x, e0), r1 = digits_of<NS>(y1.x, e1);
+  const Digits<NS> c0 = digits_of<NS>(y0.y, e0), c1 = digits_of<NS>(y1.y, e1);
 #pragma unroll
   for (int d = 0; d < NS; ++d) {
     const unsigned r = pack_digits(r0.d[d], r1.d[d]), c = pack_digits(c0.d[d], c1.d[d]);
@@ -985,15 +1071,15 @@ __device__ __forceinline__ void slice_b_pair(int64_t N, int64_t Np, size_t plane
 template <int NS>
 __global__ void slice_b_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
                                const double2* __restrict__ Y, int64_t ldy, const int* __restrict__ eb,
-                               __nv_bfloat16* __restrict__ out) {
+                               const int* __restrict__ kexp, __nv_bfloat16* __restrict__ out) {
   const int64_t k = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   const int64_t j = j0 + blockIdx.y;
   let_successor_start();
   wait_for_predecessor();
   if (k >= N) return;
   const int64_t ld = 2 * Np, br = brow_re(j);
-  slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], out + br * ld,
-               out + (br + CT) * ld);
+  slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y + j * ldy, eb[j], kexp, out + br * ld,
+                   out + (br + CT) * ld);
 }
 
 // Maximum, exponent and digits of one column of the right operand by one CTA of 256
@@ -1005,24 +1091,26 @@ constexpr int64_t kOnePass = 1024;
 template <int NS>
 __device__ __forceinline__ void slice_b_column(int64_t N, int64_t Np, int64_t brows, int64_t j,
                                                const double2* __restrict__ Y,
+                                               const int* __restrict__ kexp,
                                                int* __restrict__ eb, __nv_bfloat16* __restrict__ out,
                                                unsigned long long* red) {
-  const int ex = scale_exp(__longlong_as_double((long long)column_max(N, Y, red)));
+  const int ex = column_scale<NS>(N, Y, kexp, red);
   if (threadIdx.x == 0) eb[j] = ex;
   const int64_t ld = 2 * Np, br = brow_re(j);
   for (int64_t k = 2 * threadIdx.x; k < N; k += 512)
-    slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y, ex, out + br * ld, out + (br + CT) * ld);
+    slice_b_pair<NS>(N, Np, (size_t)brows * ld, k, Y, ex, kexp, out + br * ld,
+                     out + (br + CT) * ld);
 }
 template <int NS>
 __global__ void __launch_bounds__(256)
     slice_b_column_kernel(int64_t N, int64_t Np, int64_t brows, int64_t j0,
-                          const double2* __restrict__ Y, int64_t ldy, int* __restrict__ eb,
-                          __nv_bfloat16* __restrict__ out) {
+                          const double2* __restrict__ Y, int64_t ldy, const int* __restrict__ kexp,
+                          int* __restrict__ eb, __nv_bfloat16* __restrict__ out) {
   __shared__ unsigned long long red[8];
   const int64_t j = j0 + blockIdx.x;
   let_successor_start();
   wait_for_predecessor();
-  slice_b_column<NS>(N, Np, brows, j, Y + j * ldy, eb, out, red);
+  slice_b_column<NS>(N, Np, brows, j, Y + j * ldy, kexp, eb, out, red);
 }
 // The same for the left operand X^H: row i is the conjugate of X's column i.
 __global__ void __launch_bounds__(256)
@@ -1063,7 +1151,7 @@ __global__ void __launch_bounds__(256)
   const OzSliceEntry& e = tab[lo];
   const int64_t N = e.N, j = e.j0 + (id - e.first);
   const double2* __restrict__ Y = e.B + j * e.ldb;
-  slice_b_column<OS>(N, e.Np, e.brows, j, Y, e.eb, e.out, red);
+  slice_b_column<OS>(N, e.Np, e.brows, j, Y, nullptr, e.eb, e.out, red);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 lookup_encoder() {
@@ -1255,7 +1343,7 @@ cudaError_t ozaki_prepare_a(cudaStream_t s, const double2* A, int64_t lda, Ozaki
   diag_kernel<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(N, A, lda, w.diag);
   count_launch();
   slice_a_kernel<OS><<<dim3((unsigned)cdiv(N, 32), (unsigned)cdiv(N, SA_K), 1), dim3(32, 8, 1), 0, s>>>(
-      N, N, w.Np, true, A, lda, w.amax, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
+      N, N, w.Np, true, A, lda, w.amax, nullptr, w.ea, static_cast<__nv_bfloat16*>(w.Ad));
   count_launch();
   w.A_ready = A;
   return cudaGetLastError();
@@ -1282,17 +1370,17 @@ cudaError_t launch_early(void (*kernel)(KArgs...), dim3 grid, int threads, cudaS
 // product must not follow a refused launch: it would take the digits of another block.
 template <int NS>
 cudaError_t slice_right(cudaStream_t s, int64_t K, int64_t j0, int64_t n, const double2* B, int64_t ldb,
-                 int64_t brows, OzakiWork& w) {
+                        int64_t brows, const int* kexp, OzakiWork& w) {
   __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w.Bd);
   const int64_t Kp = ozaki_np(K);
   if (K <= kOnePass)
     return launch_early(slice_b_column_kernel<NS>, dim3((unsigned)n, 1, 1), 256, s, K, Kp, brows,
-                        j0, B, ldb, w.eb, out);
+                        j0, B, ldb, kexp, w.eb, out);
   const cudaError_t e =
-      launch_early(colexp_kernel, dim3((unsigned)n, 1, 1), 256, s, K, j0, B, ldb, w.eb);
+      launch_early(colexp_kernel<NS>, dim3((unsigned)n, 1, 1), 256, s, K, j0, B, ldb, kexp, w.eb);
   if (e != cudaSuccess) return e;
   return launch_early(slice_b_kernel<NS>, dim3((unsigned)cdiv(K, 512), (unsigned)n, 1), 256, s, K,
-                      Kp, brows, j0, B, ldb, (const int*)w.eb, out);
+                      Kp, brows, j0, B, ldb, (const int*)w.eb, kexp, out);
 }
 
 }  // namespace
@@ -1302,7 +1390,7 @@ cudaError_t ozaki_gemm(cudaStream_t s, int64_t ncols_end, int64_t j0, const doub
   const int64_t N = w.N;
   const int64_t n = ncols_end - j0;
   if (n <= 0) return cudaSuccess;
-  const cudaError_t e = slice_right<OS>(s, N, j0, n, B, ldb, w.brows, w);
+  const cudaError_t e = slice_right<OS>(s, N, j0, n, B, ldb, w.brows, nullptr, w);
   if (e != cudaSuccess) return e;
   const Maps* maps = static_cast<const Maps*>(w.maps);
   const Params P = product_params(w, ncols_end, j0, B, ldb, ep);
@@ -1313,14 +1401,20 @@ namespace {
 // Digits of the left operand X (M x K) into w.Ld, row exponents into w.el.
 template <int NS>
 cudaError_t slice_left(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
-                       OzakiWork& w) {
-  const cudaError_t e = cudaMemsetAsync(w.amax, 0, M * sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
-  rowmax_kernel<<<dim3((unsigned)cdiv(M, 256), (unsigned)cdiv(K, 256), 1), 256, 0, s>>>(
-      M, K, false, X, ldx, w.amax);
+                       const int* kexp, OzakiWork& w) {
+  const unsigned rows = (unsigned)cdiv(M, 256);
+  cudaError_t e;
+  if constexpr (NS == OS7) {
+    if ((e = cudaMemsetAsync(w.el, 0x80, M * sizeof(int), s)) != cudaSuccess) return e;
+    row_scale_kernel<<<dim3(rows, (unsigned)cdiv(K, kRowK), 1), 256, 0, s>>>(M, K, X, ldx, kexp, w.el);
+  } else {
+    if ((e = cudaMemsetAsync(w.amax, 0, M * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+    rowmax_kernel<<<dim3(rows, (unsigned)cdiv(K, 256), 1), 256, 0, s>>>(M, K, false, X, ldx,
+                                                                        w.amax);
+  }
   count_launch();
   slice_a_kernel<NS><<<dim3((unsigned)cdiv(M, 32), (unsigned)cdiv(K, SA_K), 1), dim3(32, 8, 1), 0,
-                       s>>>(M, K, ozaki_np(K), false, X, ldx, w.amax, w.el,
+                       s>>>(M, K, ozaki_np(K), false, X, ldx, w.amax, kexp, w.el,
                             static_cast<__nv_bfloat16*>(w.Ld));
   count_launch();
   return cudaGetLastError();
@@ -1382,16 +1476,16 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
     if (K <= kOnePass) {
       slice_ct_column_kernel<<<(unsigned)M, 256, 0, s>>>(M, K, Kp, X, ldx, w.el, L);
     } else {
-      colexp_kernel<<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, w.el);
+      colexp_kernel<OS><<<(unsigned)M, 256, 0, s>>>(K, 0, X, ldx, nullptr, w.el);
       slice_ct_kernel<<<dim3((unsigned)cdiv(K, 512), (unsigned)M, 1), 256, 0, s>>>(M, K, Kp, X, ldx,
                                                                                    w.el, L);
       count_launch();
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  } else if ((e = slice_left<OS>(s, M, K, X, ldx, w)) != cudaSuccess) {  // left = X, M x K
+  } else if ((e = slice_left<OS>(s, M, K, X, ldx, nullptr, w)) != cudaSuccess) {  // left = X, M x K
     return e;
   }
-  if ((e = slice_right<OS>(s, K, 0, ncols, B, ldb, w.brows, w)) != cudaSuccess) return e;
+  if ((e = slice_right<OS>(s, K, 0, ncols, B, ldb, w.brows, nullptr, w)) != cudaSuccess) return e;
   CUtensorMap ma, mb;
   if (!make_map(&ma, w.Ld, (int64_t)OS * M, Kp, TM) ||
       !make_map(&mb, w.Bd, (int64_t)OS * w.brows, Kp, TN))
@@ -1408,10 +1502,11 @@ int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M) {
 }
 
 cudaError_t ozaki_fine_begin(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
-                             int64_t ncols, const double2* B, int64_t ldb, OzakiWork& w) {
+                             int64_t ncols, const double2* B, int64_t ldb, int* kexp,
+                             OzakiWork& w) {
   const cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int), s);
   if (e != cudaSuccess || M <= 0 || ncols <= 0 || K <= 0) return e;
-  finite_kernel<<<(unsigned)K, 256, 0, s>>>(M, ncols, X, ldx, B, ldb, w.bad);
+  balance_kernel<<<(unsigned)K, 256, 0, s>>>(M, ncols, X, ldx, B, ldb, kexp, w.bad);
   count_launch();
   return cudaGetLastError();
 }
@@ -1427,13 +1522,14 @@ cudaError_t ozaki_fine_end(cudaStream_t s, const OzakiWork& w, bool* formed) {
 }
 
 cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
-                            int64_t ncols, const double2* B, int64_t ldb, const Epilogue& ep,
-                            OzakiWork& w) {
+                            int64_t ncols, const double2* B, int64_t ldb, const int* kexp,
+                            const Epilogue& ep, OzakiWork& w) {
   if (M <= 0 || ncols <= 0 || K <= 0) return cudaSuccess;
   const int64_t Kp = ozaki_np(K);
   if (M > w.N || Kp > ozaki_fine_inner(w, M)) return cudaErrorInvalidValue;
   cudaError_t e = clear_left(s, M, K, OS7, w);
-  if (e != cudaSuccess || (e = slice_left<OS7>(s, M, K, X, ldx, w)) != cudaSuccess) return e;
+  if (e != cudaSuccess || (e = slice_left<OS7>(s, M, K, X, ldx, kexp, w)) != cudaSuccess)
+    return e;
   // as many columns at a time as the right operand's planes hold, in whole tiles, and
   // as a grid has rows
   const int64_t fit = OS * w.brows * w.Np / (OS7 * Kp) / TN * CT;
@@ -1445,7 +1541,8 @@ cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2*
     return cudaErrorInvalidValue;
   for (int64_t c0 = 0; c0 < ncols; c0 += block) {
     const int64_t nc = std::min(block, ncols - c0);
-    if ((e = slice_right<OS7>(s, K, 0, nc, B + c0 * ldb, ldb, brows, w)) != cudaSuccess) return e;
+    if ((e = slice_right<OS7>(s, K, 0, nc, B + c0 * ldb, ldb, brows, kexp, w)) != cudaSuccess)
+      return e;
     Epilogue ec = ep;
     if (ec.X) ec.X += c0 * ec.ldx;
     if (ec.Y) ec.Y += c0 * ec.ldy;

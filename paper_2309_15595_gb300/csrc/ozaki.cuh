@@ -46,17 +46,21 @@ cudaError_t ozaki_gemm_general(cudaStream_t s, int64_t M, int64_t K, const doubl
                                int64_t ldb, const Epilogue& ep, OzakiWork& w,
                                bool extended = false);
 // P = X * B (M x K times K x ncols, any ncols) from seven digits of each operand, 28
-// digit pairs: an error of about sqrt(2K) 2^-57 of the row and column maxima, which
-// is FP64's. ep: EPI_STORE or EPI_FILTER. K at most ozaki_fine_inner. Several parts of K
-// may follow an ozaki_fine_begin over all of X and B, which looks for infinities and
-// NaN: where there are any, the parts leave Y as it is, ozaki_fine_end (which
-// synchronises s) says so, and the caller forms the product in FP64.
+// digit pairs, in three calls. ozaki_fine_begin looks over all of X and B: kexp (device,
+// K ints) receives the power of two that moves from column k of X to row k of B before
+// the digits are cut, and infinities and NaN, which have no digits, are noted.
+// ozaki_gemm_fine forms the product (ep: EPI_STORE or EPI_FILTER), also in parts of K,
+// each with its columns of X, rows of B and entries of kexp; K of a part at most
+// ozaki_fine_inner. Its error is about sqrt(2K) 2^-55 of the largest |x_ik| |b_kj| of any
+// k, rows and columns scaled on their own, which is below FP64's. ozaki_fine_end
+// synchronises s; *formed is false where an operand was not finite: the parts have left
+// Y as it was, and the caller forms the product in FP64.
 cudaError_t ozaki_fine_begin(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
-                             int64_t ncols, const double2* B, int64_t ldb, OzakiWork& w);
-cudaError_t ozaki_fine_end(cudaStream_t s, const OzakiWork& w, bool* formed);
+                             int64_t ncols, const double2* B, int64_t ldb, int* kexp, OzakiWork& w);
 cudaError_t ozaki_gemm_fine(cudaStream_t s, int64_t M, int64_t K, const double2* X, int64_t ldx,
-                            int64_t ncols, const double2* B, int64_t ldb, const Epilogue& ep,
-                            OzakiWork& w);
+                            int64_t ncols, const double2* B, int64_t ldb, const int* kexp,
+                            const Epilogue& ep, OzakiWork& w);
+cudaError_t ozaki_fine_end(cudaStream_t s, const OzakiWork& w, bool* formed);
 // Largest K that the planes of w have room for (0: none).
 int64_t ozaki_fine_inner(const OzakiWork& w, int64_t M);
 // X (M x K, column-major, M <= N) <- the digits it has as the left
