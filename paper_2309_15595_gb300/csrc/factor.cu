@@ -83,7 +83,8 @@ __global__ void __cluster_dims__(PF_C, 1, 1) __launch_bounds__(FT)
     }
     if (r > j) {
       const double2* w = row_s[j & 1];
-      const double2 f = cscale(-(rd * rd), conjz(w[r]));
+      // one factor at a time: 1 / p itself may not be a number where p is subnormal
+      const double2 f = cscale(-rd, cscale(rd, conjz(w[r])));
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         const int c = 16 * b + c0;
