@@ -879,12 +879,12 @@ __global__ void __launch_bounds__(BJ_IT)
 
 // The FP32 stage of a matrix of order n <= 64 in one CTA: sweeps with the
 // stopping rule of run_block_jacobi32, eigenvectors written in FP64 (ld n). The
-// matrix is scaled by a power of two into FP32's range; *bad = 1 when it holds an
-// infinity or NaN.
+// matrix is scaled by a power of two into FP32's range; info[0] = 1 when it holds an
+// infinity or NaN, info[1] = sweeps.
 __global__ void __launch_bounds__(BJ_IT)
     jacobi32_small_kernel(int n, const double2* __restrict__ G, int64_t ldg, int max_sweeps,
                           double tol_conv, double tol_stag, double2* __restrict__ X,
-                          double* __restrict__ bad) {
+                          double* __restrict__ info) {
   extern __shared__ float2 bj_smem[];
   float2* S = bj_smem;
   float2* R = bj_smem + BJ_M * BJ_LD;
@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(BJ_IT)
   atomicMax(&s_exp, ex);
   __syncthreads();
   const int sh = 1023 - s_exp;
-  if (t == 0) *bad = s_exp == 0x7ff ? 1.0 : 0.0;
+  if (t == 0) info[0] = s_exp == 0x7ff ? 1.0 : 0.0;
   for (int e = t; e < BJ_M * BJ_M; e += BJ_IT) {
     const int a = e % BJ_M, c = e / BJ_M;
     float2 g = make_float2(0.f, 0.f);
@@ -914,7 +914,8 @@ __global__ void __launch_bounds__(BJ_IT)
     R[a * BJ_LD + c] = make_float2(a == c ? 1.f : 0.f, 0.f);
   }
   double off_prev = 1e300;
-  for (int sw = 0; sw <= max_sweeps; ++sw) {
+  int sw = 0;
+  for (; sw <= max_sweeps; ++sw) {
     __syncthreads();
     float o = 0.f, d = 0.f;
     for (int e = t; e < BJ_M * BJ_M; e += BJ_IT) {
@@ -946,6 +947,7 @@ __global__ void __launch_bounds__(BJ_IT)
     off_prev = off;
     if (sw < max_sweeps) bj_sweep(S, R, rots);
   }
+  if (t == 0) info[1] = (double)min(sw, max_sweeps);
   for (int e = t; e < n * n; e += BJ_IT) {
     const float2 r = R[(e % n) * BJ_LD + e / n];
     X[e] = make_double2((double)r.x, (double)r.y);
@@ -1583,7 +1585,7 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
   // lowered to the caller's cap when one is set
   auto cap = [&](int def) { return wk.max_sweeps > 0 ? std::min(def, wk.max_sweeps) : def; };
   constexpr double kTol32 = 4e-6, kStag32 = 1e-4;
-  double* out2 = wk.red + 2 * kCoopMaxGrid + 12;  // two maxima; [2]: non-finite input
+  double* out2 = wk.red + 2 * kCoopMaxGrid + 12;  // two maxima; [2]: non-finite input, [3]: FP32 sweeps
   if (n <= BJ_M) {
     set_bj_attrs();
     jacobi32_small_kernel<<<1, BJ_IT, BJ_INNER_SMEM, s>>>((int)n, G, ldg, cap(30), kTol32, kStag32,
@@ -1607,11 +1609,14 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
   frob2_kernel<<<dim3(gb, (unsigned)n, 1), 256, 0, s>>>(n, G, ldg, reinterpret_cast<double*>(wk.T));
   count_launch();
   max2_kernel<<<1, 256, 0, s>>>(nb, reinterpret_cast<double*>(wk.T), out2); count_launch();
-  if (cudaMemcpyAsync(wk.host_red, out2, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) !=
+  if (cudaMemcpyAsync(wk.host_red, out2, 4 * sizeof(double), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return CHASE_CUDA_FAIL();
-  if (n <= BJ_M && wk.host_red[2] != 0.0) return CHASE_ERR_HEEV_NOCONV;
+  if (n <= BJ_M) {
+    if (wk.host_red[2] != 0.0) return CHASE_ERR_HEEV_NOCONV;
+    sw32 = (int)wk.host_red[3];
+  }
   // sqrt(n) times the largest norm of a 256-row column segment: within a factor
   // sqrt(n) of ||G||_2 either way, enough for the 1e-14 cluster test below
   const double gscale = wk.host_red[0] * std::sqrt((double)n);
@@ -1721,7 +1726,11 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
     }
   }
   if (!conv || (cmax > cfinish && !clustered)) {
-    if (n <= SJ_MAX) return small_fp64();
+    if (n <= SJ_MAX) {
+      const int rc = small_fp64();
+      if (sweeps_out) *sweeps_out = sw32 + refine;
+      return rc;
+    }
     // pairs the refinement could not separate (or no convergence): FP64 Jacobi
     // sweeps on G' = X^H G X finish them; eigenvectors X Z'
     Epilogue ep{};
