@@ -130,7 +130,8 @@ __global__ void __launch_bounds__(SJ_T)
   int ex = 0;
   for (int e = t; e < n * n; e += SJ_T) {
     const double2 v = Gb[e];
-    ex = max(ex, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+    ex = max(ex, (__double2hiint(v.x) >> 20) & 0x7ff);
+    if constexpr (!REAL) ex = max(ex, (__double2hiint(v.y) >> 20) & 0x7ff);
   }
   atomicMax(&s_exp, ex);
   __syncthreads();
