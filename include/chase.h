@@ -264,7 +264,8 @@ CHASE_API int chase_solve_batch(int64_t count, struct chase_ctx* const* ctxs,
  * torch uses). A is Hermitian, so the adjoint written for A is the Hermitian
  * part of the unconstrained one. Both calls use the context's product path
  * (FP64 CUDA-core or, with fp64_tensor, tensor-core FP64 for the products with
- * A), allocate their workspace on first use (kept until chase_destroy), and
+ * A and, from 2e8 operations on, for the N x N product that forms Abar, whose
+ * non-finite operands take the CUDA cores), allocate their workspace on first use (kept until chase_destroy), and
  * synchronise the context's stream before returning. */
 
 /* Adjoint of Y = p(A) V, the Eq. 1 recurrence with the same degree `deg` for

@@ -47,13 +47,17 @@ __device__ bool converged_rule(double off, double fro, double off_prev) {
 // ------------------------------------------------- single-CTA batched version
 constexpr int SJ_MAX = 64, SJ_T = 256;
 // Eigenproblems of order up to kSmallFp64 run in FP64 in one CTA; its time grows
-// like n^3 (one SM has two DFMA a clock: 5 ms at n = 60, about 0.4 ms at 24), so
-// larger ones start in FP32 (0.3 ms in one CTA) and refine in FP64 on many SMs
-// (0.1 ms a step).
+// like n^3 (one SM has two DFMA a clock), so larger ones start in FP32 in one CTA and
+// refine in FP64 on many SMs. A Rayleigh-Ritz call with N = 300, FP64 against FP32 and
+// refinement, in us: n = 16 773 / 784, 20 914 / 894, 24 1184 / 913, 32 1600 / 1043, 64
+// 8270 / 1430. They cross at 16 to 20; 24 is where the line was drawn for a slower
+// FP64 kernel.
 constexpr int64_t kSmallFp64 = 24;
 // Largest order whose FP64 refinement multiplies on the CUDA cores: a product of
 // order 64 takes 20 us there and, with the digits of both operands, 60 us on the
-// tensor cores.
+// tensor cores. A Rayleigh-Ritz call with N = 1000, CUDA cores against tensor cores, in
+// ms: n = 65 2.21 / 2.28, 96 3.14 / 2.84, 128 2.92 / 2.90, 129 4.46 / 4.08, 256 7.63 /
+// 6.26 (the orders differ in their sweeps).
 constexpr int64_t kCoreRefine = 128;
 
 // A whole FP64 Jacobi in one CTA, n <= 64 (one SM: two DFMA a clock, so FP64

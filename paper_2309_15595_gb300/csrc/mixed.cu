@@ -35,8 +35,9 @@
 // and the TMA writes 24 KB of shared memory, 480 cycles of its 128 bytes a cycle
 // for 384 cycles of products. A pair shares the operand rows: 24 and 16 KB, 320
 // cycles, so the products bound it. N = 13379, 1072 columns, degree 20: 63.3 ->
-// 60.9 ms of kernel time, 1.65 PFLOP/s with the padding of the last tiles, which is
-// 0.97 of the power-capped bf16 rate.
+// 60.6 ms of kernel time, 1.52 PFLOP/s (1.66 with the padding of the last tiles, 0.97 of
+// the power-capped bf16 rate); the whole call 61.9 to 65.8 ms as the cap has it, 68.1
+// before. N = 40000, 3000 columns inside a seconds-long step: 1.45 to 1.52 PFLOP/s.
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the kernel
 // records an error code and winds down instead of spinning.
 #include <cuda.h>

@@ -494,7 +494,7 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   } else {
     // ------------------------------------------------------- epilogue warps
     const int q = warp & 3;                   // TMEM lane quarter
-    const int h = (warp - 2) >> 2;            // complex column half: [h*24, h*24+24)
+    const int h = (warp - 2) >> 2;            // complex column half: [h HC, h HC + HC)
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
     long long acc[2 * HC];                    // re[0..16), im[16..32): levels 2-5, weight 2^-40
     // levels 6-LMAX. In FP32 at weight 2^-48; in the extended variant in int64 at
