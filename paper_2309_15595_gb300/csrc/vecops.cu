@@ -151,9 +151,14 @@ __global__ void lz_bounds_kernel(int nvec, int k, int kmax, const double* ab, co
     wt[e] = cabs2(z) / nvec;
   }
   __syncthreads();
+  // ranks: ties by index, NaN last. Every slot of ord has to be written: with NaN that
+  // compare as equal to nothing, several values shared a rank and the slots left over
+  // were read as indexes.
+  auto below = [](double a, double b) { return a < b || (b != b && a == a); };
   for (int e = t; e < tot; e += blockDim.x) {
     int rk = 0;
-    for (int j = 0; j < tot; ++j) rk += (th[j] < th[e]) || (th[j] == th[e] && j < e);
+    for (int j = 0; j < tot; ++j)
+      rk += below(th[j], th[e]) || (!below(th[e], th[j]) && j < e);
     ord[rk] = e;
   }
   __syncthreads();
