@@ -357,12 +357,29 @@ __device__ __forceinline__ RotT<T> load_rot_t(const T* __restrict__ params, int 
   return r;
 }
 
-__global__ void init32_kernel(int64_t n, const double2* G, int64_t ldg, float2* G32, float2* Z32) {
+// *out = the largest exponent field of G's entries (0 before)
+__global__ void max_exp_kernel(int64_t n, const double2* __restrict__ G, int64_t ldg,
+                               int* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t j = blockIdx.y;
+  int e = 0;
+  if (i < n) {
+    const double2 g = G[i + j * ldg];
+    e = max((__double2hiint(g.x) >> 20) & 0x7ff, (__double2hiint(g.y) >> 20) & 0x7ff);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0 && e > *(volatile int*)out) atomicMax(out, e);
+}
+// G32 = G times a power of two that brings its entries below 2 (the rotations square
+// them, and 1.8e19 is where FP32 ends); not where *max_exp says that G is not finite.
+__global__ void init32_kernel(int64_t n, const double2* G, int64_t ldg, const int* max_exp,
+                              float2* G32, float2* Z32) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j = blockIdx.y;
   if (i >= n) return;
   const double2 g = G[i + j * ldg];
-  G32[i + j * n] = make_float2((float)g.x, (float)g.y);
+  const int sh = *max_exp == 0x7ff ? 0 : 1023 - *max_exp;
+  G32[i + j * n] = make_float2((float)ldexp(g.x, sh), (float)ldexp(g.y, sh));
   Z32[i + j * n] = make_float2(i == j ? 1.f : 0.f, 0.f);
 }
 __global__ void promote_kernel(int64_t n, const float2* Z32, double2* Z) {
@@ -1597,7 +1614,10 @@ int jacobi_heev(cudaStream_t s, int64_t n, const double2* G, int64_t ldg, double
                                                           wk.Zw, out2 + 2);
     count_launch();
   } else {
-    init32_kernel<<<g2, 128, 0, s>>>(n, G, ldg, wk.G32a, wk.Z32); count_launch();
+    int* max_exp = reinterpret_cast<int*>(out2 + 2);
+    if (cudaMemsetAsync(max_exp, 0, sizeof(int), s) != cudaSuccess) return CHASE_CUDA_FAIL();
+    max_exp_kernel<<<g2, 128, 0, s>>>(n, G, ldg, max_exp); count_launch();
+    init32_kernel<<<g2, 128, 0, s>>>(n, G, ldg, max_exp, wk.G32a, wk.Z32); count_launch();
     // blocked FP32 Jacobi: G32a is G (in place), Rb the block rotations
     if (jacobi_rot_elems(n) > wk.rb_elems) return CHASE_ERR_INVALID_ARG;
     RC_(run_block_jacobi32(s, n, wk.G32a, wk.Z32, wk.Rb, wk.red, wk.host_part, cap(30), kTol32,
