@@ -391,6 +391,8 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   const int64_t tile = P.j0 / CT + ct;            // absolute CT-column tile
   const int nkb_all = (int)((2 * P.Np) / TK);
   const int kb0 = (int)part * nkb_all / P.split;  // this CTA's K blocks, its chunks from there
+  int nkb = ((int)part + 1) * nkb_all / P.split - kb0;
+  int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -416,9 +418,11 @@ __device__ __forceinline__ void ozaki_tile(const CUtensorMap* tmA, const CUtenso
   wait_for_predecessor();
 
   // a product that is not to be formed (the same in every CTA) has no K blocks
-  bool go = NS != OS7 || *P.skip == 0;
-  const int nkb = go ? ((int)part + 1) * nkb_all / P.split - kb0 : 0;
-  const int nchunks = (nkb + CHUNK_KB - 1) / CHUNK_KB;
+  bool go = true;
+  if constexpr (NS == OS7) {
+    go = *P.skip == 0;
+    if (!go) nkb = nchunks = 0;
+  }
   if (warp == 0) {
     if (lane == 0) {  // ------------------------------------ TMA producer
       if (maps_in_global) {  // tensor maps read from global memory by the TMA unit
